@@ -463,7 +463,7 @@ static m2m_status configure_kernels(m2m_ctx *ctx)
 {
     Model &m = ctx->m;
     // the finalize reuses the start of the dynamic shared memory for a block reduction
-    const size_t smem_shared = std::max(smem_bytes<T>(m, 1, 1), size_t(256) * sizeof(double));
+    const size_t smem_shared = step_smem<T>(m);
     int maxsm = 0, smsm = 0;
     CU(cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
     CU(cudaDeviceGetAttribute(&smsm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, ctx->device));
@@ -476,6 +476,13 @@ static m2m_status configure_kernels(m2m_ctx *ctx)
         if (m.g[g].geometry == M2M_GEOM_SHELLS)
             return fail(ctx, M2M_ERR_ARG, "shell groups (a_lm) need the shared deposit (%zu B of shared memory, limit %d)",
                         smem_shared, maxsm);
+    // One block works through eight chunks of observables at a time, 5,000 cycles a round; a
+    // second kernel costs about 2.5 us (5,000 cycles) with a block per range. Two rounds are the
+    // break-even: J = 236 (14 chunks) takes 19,500 cycles in the last block, J = 1,280 (40
+    // chunks) 45,000.
+    int chunks = 0;
+    for (int g = 0; g < m.n_groups; ++g) chunks += m.g[g].n_kinds * ((m.g[g].n_ap + 31) / 32);
+    m.fin_wide = ctx->global_dep || chunks > 16;
     const int max_block = ctx->global_dep ? kStepMaxThreads<T, true> : kStepMaxThreads<T, false>;
     // 512 threads in two blocks per SM was the fastest shape of the mixed-precision
     // global-deposit kernel on 64x64 maps (1024 x 1 and 256 x 4 were 8-10 % slower)
@@ -490,7 +497,7 @@ static m2m_status configure_kernels(m2m_ctx *ctx)
         // an aperture window of the largest group keeps block-shared sums, as large as the
         // blocks that registers and threads allow on an SM (or blocks_per_sm) leave room for
         int rb = 0;
-        const size_t base = std::max(smem_bytes<T>(m, 0, 0, 0), red);
+        const size_t base = std::max(smem_bytes<T>(m, 0, 0), red);
         CU(cudaFuncSetAttribute(step_kernel<T>(ctx), cudaFuncAttributeMaxDynamicSharedMemorySize, int(base)));
         CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&rb, step_kernel<T>(ctx), ctx->block, base));
         if (rb < 1) return fail(ctx, M2M_ERR_ARG, "step kernel cannot be resident with block %d", ctx->block);
@@ -500,12 +507,12 @@ static m2m_status configure_kernels(m2m_ctx *ctx)
             if (m.g[g].n_kinds * m.g[g].n_ap > m.g[best].n_kinds * m.g[best].n_ap) best = g;
         m.win_group = best;
         // 1 KB per block is reserved by the runtime; 1 KB more covers the carve's alignment
-        const long long per_block = std::min<long long>(smsm / rb, maxsm) - 2048 - (long long)smem_bytes<T>(m, 0, 0, 0);
+        const long long per_block = std::min<long long>(smsm / rb, maxsm) - 2048 - (long long)smem_bytes<T>(m, 0, 0);
         const long long slot_bytes = sizeof(T) == 8 ? 16 : 12;
         if (per_block > 0) m.win_n = int(std::min<long long>(m.g[best].n_ap, per_block / (slot_bytes * m.g[best].n_kinds)));
         m.win_lo = (m.g[best].n_ap - m.win_n) / 2;  // until the load places it
     }
-    ctx->smem_step = ctx->global_dep ? std::max(smem_bytes<T>(m, 2, 0, 0), red) : smem_shared;
+    ctx->smem_step = ctx->global_dep ? std::max(smem_bytes<T>(m, 2, 0), red) : smem_shared;
     ctx->smem_mat = smem_bytes<T>(m, 0, 0);
     if (ctx->smem_step > size_t(maxsm))
         return fail(ctx, M2M_ERR_ARG, "observable tables and prior grid need %zu B of shared memory (limit %d)",
@@ -516,6 +523,155 @@ static m2m_status configure_kernels(m2m_ctx *ctx)
     CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, step_kernel<T>(ctx), ctx->block, ctx->smem_step));
     if (occ < 1) return fail(ctx, M2M_ERR_ARG, "step kernel cannot be resident with block %d", ctx->block);
     if (ctx->bps <= 0 || ctx->bps > occ) ctx->bps = occ;
+    return M2M_OK;
+}
+
+// The host image of the step's tables (records and priors zero).
+template <class T>
+static std::vector<unsigned char> host_tables(const m2m_ctx *ctx, const TabLayout &t)
+{
+    const Model &m = ctx->m;
+    std::vector<unsigned char> h(t.bytes, 0);
+    T *vp = reinterpret_cast<T *>(h.data() + t.vp), *isp = reinterpret_cast<T *>(h.data() + t.isp);
+    T *esq = reinterpret_cast<T *>(h.data() + t.esq);
+    for (int a = 0; a < m.n_ap_total; ++a) {
+        vp[a] = T(ctx->Vp[a]);
+        isp[a] = T(ctx->isp[a]);
+    }
+    for (int e = 0; e < m.n_edges_total; ++e) esq[e] = T(ctx->edges[e] * ctx->edges[e]);
+    if (sizeof(T) == 8) exp2_table(reinterpret_cast<double *>(h.data() + t.e2));
+    if (!ctx->lut.empty()) std::memcpy(h.data() + t.lut, ctx->lut.data(), sizeof(unsigned short) * ctx->lut.size());
+    return h;
+}
+
+// The rows of the finalize, chunk by chunk (see m2m::FinPlan); the fixed-point scales are
+// those of the loaded particles (1 before the first load).
+static std::vector<ObsRow> plan_rows(const m2m_ctx *ctx)
+{
+    const Model &m = ctx->m;
+    std::vector<ObsRow> rows;
+    for (int g = 0; g < m.n_groups; ++g) {
+        const GroupDesc &G = m.g[g];
+        for (int p0 = 0; p0 < G.n_ap; p0 += 32)
+            for (int k = 0; k < G.n_kinds; ++k)
+                for (int q = 0; q < 32; ++q) {
+                    ObsRow r{0.0, 0.0, 0.0, 0.0, 1.0, -1, 0};
+                    if (p0 + q < G.n_ap) {
+                        r.j = G.obs_off + k * G.n_ap + p0 + q;
+                        r.iscale = ctx->obs_iscale.empty() ? 1.0 : ctx->obs_iscale[r.j];
+                        r.post = ctx->obs_post[r.j];
+                        r.cw = r.post / ctx->sig[r.j];
+                        r.Y = ctx->Y[r.j];
+                        r.sig = ctx->sig[r.j];
+                    }
+                    rows.push_back(r);
+                }
+    }
+    return rows;
+}
+
+// Lays the finalize out (m2m::FinPlan) and sets the records' constant elements.
+static m2m_status upload_plan(m2m_ctx *ctx)
+{
+    const Model &m = ctx->m;
+    double herm[7][7];
+    herm_table(herm);
+    const std::vector<ObsRow> rows = plan_rows(ctx);
+    std::vector<RecElem> elems;
+    std::vector<int2> range;
+    int kmax = 1, chunks = 0;
+    for (int g = 0; g < m.n_groups; ++g)
+        if (m.g[g].geometry != M2M_GEOM_SHELLS) kmax = std::max(kmax, m.g[g].n_kinds);
+    std::vector<double> co;  // [element][kind], transposed below
+    std::vector<double> rec(size_t(m.n_ap_total) * m.rec_len, 0.0);
+    for (int g = 0; g < m.n_groups; ++g) {
+        const GroupDesc &G = m.g[g];
+        const bool gh = G.max_gh >= 0;
+        for (int p0 = 0; p0 < G.n_ap; p0 += 32) {
+            range.push_back(int2{chunks, int(elems.size())});
+            chunks += G.n_kinds;
+            const int p1 = std::min(G.n_ap, p0 + 32);
+            for (int p = p0; p < p1 && G.geometry == M2M_GEOM_SHELLS; ++p)
+                for (int k = 0; k < G.n_kinds; ++k) {
+                    elems.push_back(RecElem{(G.ap_off + p) * m.rec_len + k, G.obs_off + k * G.n_ap + p, 0, 1});
+                    co.push_back(1.0);
+                    co.resize(elems.size() * kmax, 0.0);
+                }
+            for (int p = p0; p < p1 && G.geometry != M2M_GEOM_SHELLS; ++p) {
+                const int a = G.ap_off + p;
+                const double V = gh ? ctx->Vp[a] : 0.0, is = gh ? ctx->isp[a] : 1.0, s = 1.0 / is;
+                rec[size_t(a) * m.rec_len] = V;
+                rec[size_t(a) * m.rec_len + 1] = is;
+                for (int q = 0; q < 3 + G.max_gh + 1; ++q) {  // q0, q1, q2, then p_0 ..
+                    std::vector<double> f(kmax, 0.0);
+                    bool any = false;
+                    for (int k = 0; k < G.n_kinds; ++k) {
+                        const int kind = G.kinds[k];
+                        double v = 0.0;
+                        if (kind == kKindMass) v = q == 0 ? 1.0 : 0.0;
+                        else if (kind == kKindV2) v = q == 0 ? V * V : (q == 1 ? 2.0 * V * s : (q == 2 ? s * s : 0.0));
+                        else if (kind == kKindV1) v = q == 0 ? V : (q == 1 ? s : 0.0);
+                        else if (q >= 3) v = gh_c(kind - kKindGH0) * herm[kind - kKindGH0][q - 3];
+                        f[k] = v;
+                        any |= v != 0.0;
+                    }
+                    if (!any) continue;
+                    elems.push_back(RecElem{a * m.rec_len + 2 + q, G.obs_off + p, G.n_ap, G.n_kinds});
+                    co.insert(co.end(), f.begin(), f.end());
+                }
+            }
+        }
+    }
+    range.push_back(int2{chunks, int(elems.size())});
+    const size_t ne = elems.size();
+    std::vector<double> coef(ne * kmax);
+    for (size_t e = 0; e < ne; ++e)
+        for (int k = 0; k < kmax; ++k) coef[size_t(k) * ne + e] = co[e * kmax + k];
+    // one allocation: rows, elements, factors, ranges, chunk sums
+    auto up16 = [](size_t v) { return (v + 15) / 16 * 16; };
+    const size_t o_el = up16(sizeof(ObsRow) * rows.size());
+    const size_t o_co = o_el + up16(sizeof(RecElem) * ne), o_ra = o_co + up16(sizeof(double) * coef.size());
+    const size_t o_cs = o_ra + up16(sizeof(int2) * range.size()), total = o_cs + up16(sizeof(double) * (chunks + 1));
+    free_dev(ctx->d_plan);
+    CU(cudaMalloc(&ctx->d_plan, total));
+    FinPlan &pl = ctx->plan;
+    pl.n_chunks = chunks;
+    pl.n_elems = int(ne);
+    pl.n_ranges = int(range.size()) - 1;
+    pl.rows = reinterpret_cast<const ObsRow *>(ctx->d_plan);
+    pl.elems = reinterpret_cast<const RecElem *>(ctx->d_plan + o_el);
+    pl.coef = reinterpret_cast<const double *>(ctx->d_plan + o_co);
+    pl.range = reinterpret_cast<const int2 *>(ctx->d_plan + o_ra);
+    pl.csum = reinterpret_cast<double *>(ctx->d_plan + o_cs);
+    std::vector<unsigned char> h(total, 0);
+    std::memcpy(h.data(), rows.data(), sizeof(ObsRow) * rows.size());
+    if (ne) {
+        std::memcpy(h.data() + o_el, elems.data(), sizeof(RecElem) * ne);
+        std::memcpy(h.data() + o_co, coef.data(), sizeof(double) * coef.size());
+    }
+    std::memcpy(h.data() + o_ra, range.data(), sizeof(int2) * range.size());
+    CU(cudaMemcpy(ctx->d_plan, h.data(), total, cudaMemcpyHostToDevice));
+    CU(cudaMemcpy(ctx->d_rec, rec.data(), sizeof(double) * rec.size(), cudaMemcpyHostToDevice));
+    if (ctx->d_recf) {
+        const std::vector<float> rf(rec.begin(), rec.end());
+        CU(cudaMemcpy(ctx->d_recf, rf.data(), sizeof(float) * rf.size(), cudaMemcpyHostToDevice));
+    }
+    return M2M_OK;
+}
+
+// The fixed-point scales of the loaded particles into obs_iscale and the rows of the finalize.
+static m2m_status set_scales(m2m_ctx *ctx)
+{
+    const Model &m = ctx->m;
+    ctx->obs_iscale.resize(m.J);
+    for (int j = 0; j < m.J; ++j) {
+        const int k = ctx->obs_kind[j];
+        ctx->obs_iscale[j] = 1.0 / (k == kKindMass ? m.fx_w : ((k == kKindV2 || k == kKindV1) ? m.fx_v2 : m.fx_gh));
+    }
+    const std::vector<ObsRow> rows = plan_rows(ctx);
+    CU(cudaMemcpyAsync(ctx->d_plan, rows.data(), sizeof(ObsRow) * rows.size(), cudaMemcpyHostToDevice,
+                       ctx->stream));
+    CU(cudaStreamSynchronize(ctx->stream));
     return M2M_OK;
 }
 
@@ -530,19 +686,32 @@ static m2m_status upload_tables(m2m_ctx *ctx)
         return M2M_OK;
     };
     m2m_status s;
-    if ((s = up(ctx->d_edges, ctx->edges)) != M2M_OK) return s;
-    if ((s = up(ctx->d_Vp, ctx->Vp)) != M2M_OK) return s;
-    if ((s = up(ctx->d_isp, ctx->isp)) != M2M_OK) return s;
     {
-        std::vector<float> vf(ctx->Vp.begin(), ctx->Vp.end()), sf(ctx->isp.begin(), ctx->isp.end());
-        free_dev(ctx->d_Vpf);
-        free_dev(ctx->d_ispf);
-        if (!vf.empty()) {
-            CU(cudaMalloc(&ctx->d_Vpf, vf.size() * sizeof(float)));
-            CU(cudaMalloc(&ctx->d_ispf, sf.size() * sizeof(float)));
-            CU(cudaMemcpy(ctx->d_Vpf, vf.data(), vf.size() * sizeof(float), cudaMemcpyHostToDevice));
-            CU(cudaMemcpy(ctx->d_ispf, sf.data(), sf.size() * sizeof(float), cudaMemcpyHostToDevice));
+        const bool fp64 = ctx->precision == M2M_PREC_FP64;
+        const TabLayout t = fp64 ? tab_layout<double>(m) : tab_layout<float>(m);
+        const std::vector<unsigned char> h = fp64 ? host_tables<double>(ctx, t) : host_tables<float>(ctx, t);
+        CU(cudaMalloc(&ctx->d_tab, t.bytes > 0 ? t.bytes : 16));
+        CU(cudaMemcpy(ctx->d_tab, h.data(), t.bytes, cudaMemcpyHostToDevice));
+        if (fp64) {
+            ctx->d_rec = reinterpret_cast<double *>(ctx->d_tab + t.rec);
+            ctx->d_Vp = reinterpret_cast<double *>(ctx->d_tab + t.vp);
+            ctx->d_isp = reinterpret_cast<double *>(ctx->d_tab + t.isp);
+            ctx->d_lprior = reinterpret_cast<double *>(ctx->d_tab + t.prior);
+        } else {
+            ctx->d_recf = reinterpret_cast<float *>(ctx->d_tab + t.rec);
+            ctx->d_Vpf = reinterpret_cast<float *>(ctx->d_tab + t.vp);
+            ctx->d_ispf = reinterpret_cast<float *>(ctx->d_tab + t.isp);
+            ctx->d_ipriorf = reinterpret_cast<float *>(ctx->d_tab + t.prior);
+            if ((s = up(ctx->d_Vp, ctx->Vp)) != M2M_OK) return s;
+            if ((s = up(ctx->d_isp, ctx->isp)) != M2M_OK) return s;
+            CU(cudaMalloc(&ctx->d_rec, sizeof(double) * m.n_ap_total * m.rec_len));
+            CU(cudaMemset(ctx->d_rec, 0, sizeof(double) * m.n_ap_total * m.rec_len));
+            CU(cudaMalloc(&ctx->d_lprior, sizeof(double) * (m.ncell + 1)));
+            CU(cudaMemset(ctx->d_lprior, 0, sizeof(double) * (m.ncell + 1)));
         }
+        if ((s = upload_plan(ctx)) != M2M_OK) return s;
+        CU(cudaMalloc(&ctx->d_head, sizeof(StepHead)));
+        CU(cudaMemset(ctx->d_head, 0, sizeof(StepHead)));
     }
     if ((s = up(ctx->d_lcE, ctx->lcE)) != M2M_OK) return s;
     if (m.pot == 3) {
@@ -562,30 +731,17 @@ static m2m_status upload_tables(m2m_ctx *ctx)
         ctx->m.scf_tabf = ctx->d_scf_tabf;
         ctx->m.scf_coef = ctx->d_scf_coef;
     }
-    if ((s = up(ctx->d_Y, ctx->Y)) != M2M_OK) return s;
     if ((s = up(ctx->d_sig, ctx->sig)) != M2M_OK) return s;
-    if ((s = up(ctx->d_post, ctx->obs_post)) != M2M_OK) return s;
-    free_dev(ctx->d_lut);
-    CU(cudaMalloc(&ctx->d_lut, sizeof(unsigned short) * (ctx->lut.size() + 1)));
-    if (!ctx->lut.empty())
-        CU(cudaMemcpy(ctx->d_lut, ctx->lut.data(), sizeof(unsigned short) * ctx->lut.size(), cudaMemcpyHostToDevice));
     free_dev(ctx->d_kind);
     CU(cudaMalloc(&ctx->d_kind, sizeof(int) * m.J));
     CU(cudaMemcpy(ctx->d_kind, ctx->obs_kind.data(), sizeof(int) * m.J, cudaMemcpyHostToDevice));
-    CU(cudaMalloc(&ctx->d_iscale, sizeof(double) * m.J));
     CU(cudaMalloc(&ctx->d_c, sizeof(double) * m.J));
-    CU(cudaMalloc(&ctx->d_rec, sizeof(double) * m.n_ap_total * m.rec_len));
-    CU(cudaMemset(ctx->d_rec, 0, sizeof(double) * m.n_ap_total * m.rec_len));
-    CU(cudaMalloc(&ctx->d_recf, sizeof(float) * m.n_ap_total * m.rec_len));
-    CU(cudaMemset(ctx->d_recf, 0, sizeof(float) * m.n_ap_total * m.rec_len));
     CU(cudaMalloc(&ctx->d_ytil, sizeof(double) * m.J));
     CU(cudaMalloc(&ctx->d_yraw, sizeof(double) * m.J));
     CU(cudaMalloc(&ctx->d_delta, sizeof(double) * m.J));
     CU(cudaMalloc(&ctx->d_prior, sizeof(double) * (m.ncell + 1)));
     CU(cudaMalloc(&ctx->d_iprior, sizeof(double) * (m.ncell + 1)));
     CU(cudaMemset(ctx->d_iprior, 0, sizeof(double) * (m.ncell + 1)));
-    CU(cudaMalloc(&ctx->d_lprior, sizeof(double) * (m.ncell + 1)));
-    CU(cudaMemset(ctx->d_lprior, 0, sizeof(double) * (m.ncell + 1)));
     CU(cudaMalloc(&ctx->d_prior_count, sizeof(long long) * (m.ncell + 1)));
     CU(cudaMalloc(&ctx->d_hist, sizeof(long long) * exchange_words(ctx)));
     if (m.pwin_E > 0 || m.pwin_x > 0) CU(cudaMalloc(&ctx->d_pwin, sizeof(unsigned long long) * 3 * m.ncell));
@@ -668,8 +824,9 @@ extern "C" m2m_status m2m_create(const m2m_potential *pot, const m2m_observables
 Buffers buffers(m2m_ctx *c)
 {
     Buffers b;
-    b.edges = c->d_edges; b.Vp = c->d_Vp; b.isp = c->d_isp; b.Vpf = c->d_Vpf; b.ispf = c->d_ispf; b.lcE = c->d_lcE; b.lut = c->d_lut;
-    b.Y = c->d_Y; b.sig = c->d_sig; b.obs_kind = c->d_kind; b.obs_post = c->d_post; b.obs_iscale = c->d_iscale;
+    b.tab = c->d_tab; b.head = c->d_head; b.Vp = c->d_Vp; b.isp = c->d_isp; b.Vpf = c->d_Vpf; b.ispf = c->d_ispf; b.lcE = c->d_lcE;
+    b.ipriorf = c->d_ipriorf;
+    b.sig = c->d_sig; b.obs_kind = c->d_kind; b.plan = c->plan;
     b.c = c->d_c; b.rec = c->d_rec; b.recf = c->d_recf; b.prior = c->d_prior; b.iprior = c->d_iprior;
     b.lprior = c->d_lprior; b.prior_count = c->d_prior_count; b.hist = c->d_hist;
     b.prior_raw = c->d_prior_raw; b.pwin = c->d_pwin; b.sV = c->d_sV; b.sVT = c->d_sVT; b.sD = c->d_sD;
@@ -680,9 +837,12 @@ Buffers buffers(m2m_ctx *c)
 
 static int grid_for(m2m_ctx *c)
 {
-    long long need = (c->n + c->block - 1) / c->block;
-    long long g = (long long)c->nsm * c->bps;
-    if (need < g) g = need;
+    // whole waves of one block per SM, up to the resident ones (the kernel shares the particles
+    // out evenly over the blocks in whole warps); a fit of fewer warps than SMs takes a block per
+    // warp. With ceil(n / block) blocks a 20,000-particle FP64 fit used 79 of the 152 SMs.
+    const long long units = (c->n + 31) / 32, wave = (long long)c->nsm * c->block;
+    long long g = c->nsm * std::min<long long>(c->bps, (c->n + wave - 1) / wave);
+    if (units < g) g = units;
     // no block may process more than kMaxParticlesPerBlock particles (exact 32-bit sums)
     const long long floor_g = (c->n + kMaxParticlesPerBlock - 1) / kMaxParticlesPerBlock;
     if (g < floor_g) g = floor_g;
@@ -690,10 +850,19 @@ static int grid_for(m2m_ctx *c)
 }
 
 template <class T, int WPS>
+static void launch_finalize(m2m_ctx *c, int init)
+{
+    k_finalize<T, WPS><<<c->plan.n_ranges, 256, 0, c->stream>>>(c->m, buffers(c), c->m.shard ? c->m.n_all : c->n, init);
+}
+
+// The pass over the particles, and the finalize where it is not in its last block: a shard's
+// follows the exchange.
+template <class T, int WPS>
 static void launch_step(m2m_ctx *c, int push, int init)
 {
     step_kernel<T>(c)<<<grid_for(c), c->block, c->smem_step, c->stream>>>(c->m, make_cst<T>(c->m), state<T>(c),
                                                                               buffers(c), push, init);
+    if (c->m.fin_wide && !c->m.shard) launch_finalize<T, WPS>(c, init);
 }
 
 static void launch_one(m2m_ctx *c, int push, int init)
@@ -709,8 +878,7 @@ template <class T, int WPS>
 static void launch_step_timed(m2m_ctx *c, cudaEvent_t *ev)
 {
     cudaEventRecord(ev[0], c->stream);
-    step_kernel<T>(c)<<<grid_for(c), c->block, c->smem_step, c->stream>>>(c->m, make_cst<T>(c->m), state<T>(c),
-                                                                              buffers(c), 1, 0);
+    launch_step<T, WPS>(c, 1, 0);
     smooth_launch(c);
     cudaEventRecord(ev[1], c->stream);
 }
@@ -795,13 +963,8 @@ static m2m_status finish_load(m2m_ctx *ctx, const double *dx, const double *dy, 
         for (double v : ctx->isp) isp_max = std::max(isp_max, v);
         m.fx_dv = pow2_floor(two62 / (Wb * 1.5 * std::sqrt(m.v2max) * isp_max + Wb));
     }
-    ctx->obs_iscale.resize(m.J);
-    for (int j = 0; j < m.J; ++j) {
-        const int k = ctx->obs_kind[j];
-        const double s = k == kKindMass ? m.fx_w : ((k == kKindV2 || k == kKindV1) ? m.fx_v2 : m.fx_gh);
-        ctx->obs_iscale[j] = 1.0 / s;
-    }
-    CU(cudaMemcpyAsync(ctx->d_iscale, ctx->obs_iscale.data(), sizeof(double) * m.J, cudaMemcpyHostToDevice, ctx->stream));
+    const m2m_status rs = set_scales(ctx);
+    if (rs != M2M_OK) return rs;
     CU(cudaMemsetAsync(ctx->d_hist, 0, sizeof(long long) * exchange_words(ctx), ctx->stream));
     Scalars sc0{};
     sc0.Wrange = 9.2233720368547758e18 / m.fx_w;
@@ -809,7 +972,8 @@ static m2m_status finish_load(m2m_ctx *ctx, const double *dx, const double *dy, 
     CU(cudaMemcpyAsync(ctx->d_sc, &sc0, sizeof(Scalars), cudaMemcpyHostToDevice, ctx->stream));
     CU(cudaMemsetAsync(ctx->d_prior, 0, sizeof(double) * (m.ncell + 1), ctx->stream));
     CU(cudaMemsetAsync(ctx->d_iprior, 0, sizeof(double) * (m.ncell + 1), ctx->stream));
-    CU(cudaMemsetAsync(ctx->d_lprior, 0, sizeof(double) * (m.ncell + 1), ctx->stream));
+    CU(cudaMemsetAsync(ctx->d_lprior, 0, sizeof(double) * m.ncell, ctx->stream));
+    if (ctx->d_ipriorf) CU(cudaMemsetAsync(ctx->d_ipriorf, 0, sizeof(float) * m.ncell, ctx->stream));
     CU(cudaMemsetAsync(ctx->d_prior_count, 0, sizeof(long long) * (m.ncell + 1), ctx->stream));
     CU(cudaMemsetAsync(ctx->cell, 0, sizeof(uint16_t) * (ctx->n > 0 ? ctx->n : 1), ctx->stream));
     launch_one(ctx, 0, 1);
@@ -1112,11 +1276,8 @@ extern "C" m2m_status m2m_step_end(m2m_ctx *ctx)
     if (ctx->shard_pending != 1 && ctx->shard_pending != 2)
         return fail(ctx, M2M_ERR_STATE, "m2m_step_end follows a load or m2m_step_begin");
     const int init = ctx->shard_pending == 1;
-    const int threads = ctx->block;  // the finalize block of m2m_step, so chi^2 adds in the same order
-    if (ctx->precision == M2M_PREC_FP64)
-        k_finalize<double, 2><<<1, threads, sizeof(double) * threads, ctx->stream>>>(ctx->m, buffers(ctx), init);
-    else
-        k_finalize<float, 1><<<1, threads, sizeof(double) * threads, ctx->stream>>>(ctx->m, buffers(ctx), init);
+    if (ctx->precision == M2M_PREC_FP64) launch_finalize<double, 2>(ctx, init);
+    else launch_finalize<float, 1>(ctx, init);
     smooth_launch(ctx);
     CU(cudaGetLastError());
     ctx->shard_pending = 0;
@@ -1448,12 +1609,7 @@ extern "C" m2m_status m2m_load_state(m2m_ctx *ctx, const char *path)
     if (s != M2M_OK) return s;
     ctx->n = hd.n;
     m.fx_w = hd.fx_w; m.fx_v2 = hd.fx_v2; m.fx_gh = hd.fx_gh; m.v2max = hd.v2max;
-    ctx->obs_iscale.resize(m.J);
-    for (int j = 0; j < m.J; ++j) {
-        const int k = ctx->obs_kind[j];
-        ctx->obs_iscale[j] = 1.0 / (k == kKindMass ? m.fx_w : ((k == kKindV2 || k == kKindV1) ? m.fx_v2 : m.fx_gh));
-    }
-    CU(cudaMemcpy(ctx->d_iscale, ctx->obs_iscale.data(), sizeof(double) * m.J, cudaMemcpyHostToDevice));
+    if ((s = set_scales(ctx)) != M2M_OK) return s;
     const char *p = buf.data();
     for (int k = 0; k < narr; ++k) {
         if (n) CU(cudaMemcpy(ctx->st[k], p, es * n, cudaMemcpyHostToDevice));
@@ -1471,13 +1627,14 @@ extern "C" m2m_status m2m_load_state(m2m_ctx *ctx, const char *path)
         p += sizeof(double) * m.J;
     }
     CU(cudaMemcpy(ctx->d_rec, p, sizeof(double) * m.n_ap_total * m.rec_len, cudaMemcpyHostToDevice));
-    k_convert_in<float><<<ctx->nsm, 256, 0, ctx->stream>>>(ctx->d_rec, ctx->d_recf, m.n_ap_total * m.rec_len);
-    CU(cudaStreamSynchronize(ctx->stream));
+    if (ctx->d_recf)
+        k_convert_in<float><<<ctx->nsm, 256, 0, ctx->stream>>>(ctx->d_rec, ctx->d_recf, m.n_ap_total * m.rec_len);
     p += sizeof(double) * m.n_ap_total * m.rec_len;
     if (m.ncell) {
         CU(cudaMemcpy(ctx->d_prior, p, sizeof(double) * m.ncell, cudaMemcpyHostToDevice));
         p += sizeof(double) * m.ncell;
         CU(cudaMemcpy(ctx->d_iprior, p, sizeof(double) * m.ncell, cudaMemcpyHostToDevice));
+        if (ctx->d_ipriorf) k_convert_in<float><<<ctx->nsm, 256, 0, ctx->stream>>>(ctx->d_iprior, ctx->d_ipriorf, m.ncell);
         p += sizeof(double) * m.ncell;
         CU(cudaMemcpy(ctx->d_lprior, p, sizeof(double) * m.ncell, cudaMemcpyHostToDevice));
         p += sizeof(double) * m.ncell;
@@ -1488,6 +1645,9 @@ extern "C" m2m_status m2m_load_state(m2m_ctx *ctx, const char *path)
     }
     CU(cudaMemcpy(ctx->d_sc, p, sizeof(Scalars), cudaMemcpyHostToDevice));
     CU(cudaMemset(ctx->d_hist, 0, sizeof(long long) * m.hist_words));
+    k_head<<<1, 32, 0, ctx->stream>>>(m, ctx->d_sc, ctx->d_head);
+    CU(cudaGetLastError());
+    CU(cudaStreamSynchronize(ctx->stream));
     if (ctx->graph) {
         cudaGraphExecDestroy(ctx->graph);
         ctx->graph = nullptr;
@@ -1757,10 +1917,13 @@ void destroy_impl(m2m_ctx *ctx)
     if (ctx->graph) cudaGraphExecDestroy(ctx->graph);
     for (cudaEvent_t e : ctx->events) cudaEventDestroy(e);
     free_state(ctx);
-    free_dev(ctx->d_edges); free_dev(ctx->d_Vp); free_dev(ctx->d_isp); free_dev(ctx->d_Vpf); free_dev(ctx->d_ispf); free_dev(ctx->d_lcE); free_dev(ctx->d_lut);
+    if (ctx->precision == M2M_PREC_MIXED) {  // in FP64 mode these are parts of d_tab
+        free_dev(ctx->d_Vp); free_dev(ctx->d_isp); free_dev(ctx->d_rec); free_dev(ctx->d_lprior);
+    }
+    free_dev(ctx->d_tab); free_dev(ctx->d_head); free_dev(ctx->d_plan); free_dev(ctx->d_lcE);
     free_dev(ctx->d_scf_r); free_dev(ctx->d_scf_tab); free_dev(ctx->d_scf_tabf); free_dev(ctx->d_scf_coef);
-    free_dev(ctx->d_Y); free_dev(ctx->d_sig); free_dev(ctx->d_post); free_dev(ctx->d_iscale);
-    free_dev(ctx->d_kind); free_dev(ctx->d_c); free_dev(ctx->d_rec); free_dev(ctx->d_recf); free_dev(ctx->d_prior); free_dev(ctx->d_iprior); free_dev(ctx->d_lprior);
+    free_dev(ctx->d_sig);
+    free_dev(ctx->d_kind); free_dev(ctx->d_c); free_dev(ctx->d_prior); free_dev(ctx->d_iprior);
     free_dev(ctx->d_ytil);
     free_dev(ctx->d_yraw); free_dev(ctx->d_delta); free_dev(ctx->d_prior_count);
     free_dev(ctx->d_hist); free_dev(ctx->d_acc); free_dev(ctx->d_sc); free_dev(ctx->d_pwin);

@@ -210,6 +210,7 @@ static m2m_status batch_prepare(m2m_ctx *ctx)
     for (int i = 0; i < M; ++i) {
         m2m_ctx *c = ctx->sub[i];
         models[i] = c->m;
+        models[i].fin_wide = 0;  // the batched step finalizes every fit in its last block
         csts[i] = make_cst<T>(c->m);
         states[i] = state<T>(c);
         bufs[i] = buffers(c);
@@ -380,8 +381,8 @@ static m2m_status batch_configure(m2m_ctx *ctx, const m2m_options *opt)
 {
     BatchState &B = *ctx->bs;
     B.kernel = batch_pick<T, WPS>(ctx->sub, B.bank);
-    size_t smem = size_t(256) * sizeof(double);  // the finalize's block reduction
-    for (const m2m_ctx *c : ctx->sub) smem = std::max(smem, smem_bytes<T>(c->m, 1, 1));
+    size_t smem = 0;
+    for (const m2m_ctx *c : ctx->sub) smem = std::max(smem, step_smem<T>(c->m));
     CU(cudaDeviceGetAttribute(&B.maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
     CU(cudaDeviceGetAttribute(&B.nsm, cudaDevAttrMultiProcessorCount, ctx->device));
     if (smem > size_t(B.maxsm))

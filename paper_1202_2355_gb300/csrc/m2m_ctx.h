@@ -37,10 +37,15 @@ struct m2m_ctx {
     uint16_t *cell = nullptr;
     uint16_t *ap = nullptr;  // cached apertures (Model::ap_cache)
     double *gx = nullptr;    // cached exp(-nu^2/2) (Model::gx_group, FP64 mode)
-    double *d_edges = nullptr, *d_Vp = nullptr, *d_isp = nullptr, *d_lcE = nullptr;
-    float *d_Vpf = nullptr, *d_ispf = nullptr;
-    unsigned short *d_lut = nullptr;
-    double *d_Y = nullptr, *d_sig = nullptr, *d_post = nullptr, *d_iscale = nullptr;
+    // the step's tables in the state type (m2m::TabLayout); the arrays of that type among
+    // d_Vp .. d_lprior (FP64 mode) or d_Vpf .. d_ipriorf (mixed mode) are parts of it
+    unsigned char *d_tab = nullptr;
+    m2m::StepHead *d_head = nullptr;
+    double *d_Vp = nullptr, *d_isp = nullptr, *d_lcE = nullptr;
+    float *d_Vpf = nullptr, *d_ispf = nullptr, *d_ipriorf = nullptr;
+    m2m::FinPlan plan{};
+    unsigned char *d_plan = nullptr;  // the plan's arrays in one allocation, its rows first
+    double *d_sig = nullptr;
     int *d_kind = nullptr;
     double *d_c = nullptr, *d_prior = nullptr, *d_ytil = nullptr, *d_yraw = nullptr, *d_delta = nullptr;
     double *d_rec = nullptr, *d_iprior = nullptr, *d_lprior = nullptr;
@@ -141,6 +146,17 @@ inline m2m::State<T> state(m2m_ctx *c)
     s.gx = sizeof(T) == 8 ? reinterpret_cast<T *>(c->gx) : nullptr;
     s.n = c->n;
     return s;
+}
+
+// Shared memory of a block-shared step kernel: sums and tables, and at least what the
+// finalize takes at the start of it (the coefficients c_j and the chunk sums).
+template <class T>
+inline size_t step_smem(const m2m::Model &m)
+{
+    size_t chunks = 0;
+    for (int g = 0; g < m.n_groups; ++g) chunks += size_t(m.g[g].n_kinds) * ((m.g[g].n_ap + 31) / 32);
+    const size_t a = m2m::smem_bytes<T>(m, 1, 1), b = sizeof(double) * (32 + size_t(m.J) + chunks);
+    return a > b ? a : b;
 }
 
 // Resident blocks per SM the step kernels are compiled for (register budget). The

@@ -119,6 +119,9 @@ struct Model {
     double *scf_coef;      // device: a_lm,k of the last expansion (scf_n x scf_nlm)
     double scf_norm[49];   // factor of Y_lm (N_lm, sqrt2 N_lm for m != 0) by index
     float scf_norm_f[49];
+    // the finalize of a step runs as k_finalize over several blocks instead of in the last
+    // block of the step kernel (see configure_kernels)
+    int fin_wide;
 };
 
 constexpr unsigned kApNone8 = 0xFFu, kApNone16 = 0xFFFFu;
@@ -239,6 +242,18 @@ struct Scalars {
     double ups;            // mass-to-light ratio of the self-consistent potential
 };
 
+// What every block of a step reads before its first particle, written once per step by the
+// finalize (the flags of step t + 1 in the types the step uses: a 64-bit modulo and an FP64
+// division in every thread of every block cost 9,500 cycles of the mixed step at 2M particles,
+// the FP64 pipe being that narrow; 1,000 now). Kept apart from Scalars, whose layout is that
+// of the checkpoint files.
+struct alignas(16) StepHead {
+    int pending, prior_step, scf_step;
+    float wscale, iwhat;      // mixed mode: weight scale, 1/flat prior (0 when it reads 0)
+    int pad;
+    double lwscale, lwhat;    // FP64 mode: ln of both
+};
+
 template <class T>
 struct State {
     T *x, *y, *z, *vx, *vy, *vz, *w;
@@ -276,20 +291,44 @@ __host__ __device__ __forceinline__ bool keeps_accel(const Model &m)
     return m.pot != 3 && (kCacheAccel<T> || m.cache_accel);
 }
 
+// The finalize works through the observables in chunks of one warp: up to 32 consecutive
+// apertures of one kind of one group, ordered by group, then aperture range, then kind, so
+// that one warp sums a chunk's Delta_j^2 and one block holds every coefficient of a range of
+// apertures. chi^2 adds the chunks in this order whatever the number of blocks and threads.
+// The force-of-change records are linear in the coefficients c_j: an element of a record is
+// sum_k coef_k c_(j0 + k stride) over the kinds of its group, with the factors laid out here
+// (see upload_plan), and only the elements that are ever non-zero are listed.
+struct ObsRow {
+    double iscale, post, cw, Y, sig;  // 1/fixed-point scale; factor of the raw sum; post / sig; data
+    int j, pad;                       // observable, -1 for the padding of a chunk
+};
+struct RecElem {
+    int dst, j0, stride, nk;  // element of the records; its terms
+};
+struct FinPlan {
+    int n_chunks, n_elems, n_ranges, pad;
+    const ObsRow *rows;      // 32 per chunk
+    const RecElem *elems;    // ordered by aperture range
+    const double *coef;      // [kind][element]
+    const int2 *range;       // per aperture range: first chunk and first element (n_ranges + 1)
+    double *csum;            // per chunk: sum of Delta_j^2 (finalize over several blocks)
+};
+
 struct Buffers {
-    const double *edges, *Vp, *isp;  // per group edges, per aperture V_p and 1/sigma_p
-    const float *Vpf, *ispf;         // FP32 copies of V_p and 1/sigma_p (read from global memory)
-    const unsigned short *lut;       // annulus lookup tables (FP32 path)
+    const unsigned char *tab;        // the tables of the step in the state type (see TabLayout)
+    StepHead *head;
+    const double *Vp, *isp;          // per aperture V_p and 1/sigma_p
+    const float *Vpf, *ispf;         // FP32 copies of V_p and 1/sigma_p (mixed mode)
     const double *lcE;               // E_c table
-    const double *Y, *sig;
+    const double *sig;
     const int *obs_kind;             // per observable: kind
-    const double *obs_post;          // per observable: factor applied to the raw sum (1/area for mass)
-    const double *obs_iscale;        // per observable: 1/fixed-point scale
+    FinPlan plan;                    // the order of the finalize
     double *c;                       // per observable: coefficient of the force of change
     double *rec;                     // per aperture: the data term of eq. modFOC as polynomials in nu
     float *recf;                     // FP32 copy of rec (mixed mode reads it from global memory)
     double *prior;                   // per cell: prior (cell mean weight)
     double *iprior;                  // per cell: 1/prior (0 when the prior reads as 0)
+    float *ipriorf;                  // FP32 copy of iprior (mixed mode)
     double *lprior;                  // per cell: ln prior (-inf when the prior reads as 0)
     long long *prior_count;          // per cell: particle count at the last update
     double *prior_raw;               // per cell: raw cell mean before smoothing (smoothing on)
@@ -1538,12 +1577,41 @@ __device__ __forceinline__ T foc_update_log(const Model &m, const Cst<T> &k, con
 
 // ---------------------------------------------------------------- shared-memory layout
 
+// The step's tables in the state type T, as one block of global memory per fit that a block
+// of the step kernel copies into shared memory as it is, in 16-byte pieces: the force-of-
+// change records, V_p and 1/sigma_p, 1/prior (ln prior in FP64 mode), the squared edges,
+// 2^(j/32) (FP64 mode) and the annulus lookup. The finalize writes the records and priors in
+// place; the rest is laid out at creation. (Converting every table from FP64 in every block took
+// 15,000 cycles of a step with 2,700 priors, and 5,800 with 300.) The global-deposit kernel and the
+// weight read-out take the part from the priors on. Offsets in bytes.
+struct TabLayout {
+    int rec, vp, isp, prior, esq, e2, lut, bytes;
+};
+
+template <class T>
+__host__ __device__ inline TabLayout tab_layout(const Model &m)
+{
+    auto up = [](size_t b) { return int((b + 15) / 16 * 16); };
+    TabLayout t;
+    t.rec = 0;
+    t.vp = up(sizeof(T) * size_t(m.n_ap_total) * m.rec_len);
+    t.isp = t.vp + up(sizeof(T) * size_t(m.n_ap_total));
+    t.prior = t.isp + up(sizeof(T) * size_t(m.n_ap_total));
+    t.esq = t.prior + up(sizeof(T) * size_t(m.ncell));
+    t.e2 = t.esq + up(sizeof(T) * size_t(m.n_edges_total));
+    t.lut = t.e2 + (sizeof(T) == 8 ? 32 * int(sizeof(double)) : 0);
+    t.bytes = t.lut + up(sizeof(unsigned short) * size_t(m.n_lut));
+    return t;
+}
+
 template <class T>
 struct Smem {
     void *h;               // fixed-point sums of the block (layout of Acc<T>)
     T *c, *iprior, *esq, *vp, *isp;  // c: the force-of-change records; iprior: 1/prior, or ln prior (FP64)
     double *e2;            // 2^(j/32) for exp_tab
     unsigned short *lut;
+    unsigned char *tab;    // start of the copied tables, and the range of them that is copied
+    int tab_lo, tab_hi;
 };
 
 // Block sums of the global-deposit kernel's aperture window: one slot per kind and
@@ -1563,61 +1631,57 @@ __host__ __device__ inline size_t acc_bytes_padded(const Model &m, int hist = 1)
     return (b + 15) / 16 * 16;
 }
 
-// Dynamic shared memory of a kernel holding the block sums (with_hist) and the
-// force-of-change records (with_rec) in shared memory; the global-deposit step
-// kernel keeps both in global memory.
+// Dynamic shared memory of a kernel holding the block sums (with_hist) and all tables
+// (with_rec) or those from the priors on; the global-deposit step kernel keeps its records,
+// V_p and 1/sigma_p in global memory.
 template <class T>
-__host__ __device__ inline size_t smem_bytes(const Model &m, int with_hist, int with_rec = 1, int with_vp = 1)
+__host__ __device__ inline size_t smem_bytes(const Model &m, int with_hist, int with_rec = 1)
 {
-    size_t b = with_hist ? acc_bytes_padded<T>(m, with_hist) : 0;
-    b += sizeof(T) * size_t((with_rec ? m.n_ap_total * m.rec_len : 0) + m.ncell + m.n_edges_total +
-                            (with_vp ? 2 * m.n_ap_total : 0));
-    b = (b + 7) / 8 * 8 + sizeof(double) * 32;
-    b += sizeof(unsigned short) * size_t(m.n_lut) + 16;
-    return b;
+    const TabLayout t = tab_layout<T>(m);
+    return (with_hist ? acc_bytes_padded<T>(m, with_hist) : 0) + size_t(t.bytes - (with_rec ? 0 : t.prior));
 }
 
 template <class T>
-__device__ __forceinline__ Smem<T> carve(const Model &m, unsigned char *base, int with_hist, int with_rec = 1,
-                                         int with_vp = 1)
+__device__ __forceinline__ Smem<T> carve(const Model &m, unsigned char *base, int with_hist, int with_rec = 1)
 {
+    const TabLayout t = tab_layout<T>(m);
     Smem<T> s;
     s.h = base;
-    T *t = reinterpret_cast<T *>(base + (with_hist ? acc_bytes_padded<T>(m, with_hist) : 0));
-    s.c = t;
-    s.iprior = s.c + (with_rec ? m.n_ap_total * m.rec_len : 0);
-    s.esq = s.iprior + m.ncell;
-    s.vp = s.esq + m.n_edges_total;
-    s.isp = s.vp + (with_vp ? m.n_ap_total : 0);
-    unsigned char *e = reinterpret_cast<unsigned char *>(s.isp + (with_vp ? m.n_ap_total : 0));
-    s.e2 = reinterpret_cast<double *>(base + (e - base + 7) / 8 * 8);
-    s.lut = reinterpret_cast<unsigned short *>(s.e2 + 32);
+    s.tab = base + (with_hist ? acc_bytes_padded<T>(m, with_hist) : 0);
+    s.tab_lo = with_rec ? 0 : t.prior;
+    s.tab_hi = t.bytes;
+    unsigned char *z = s.tab - s.tab_lo;
+    s.c = reinterpret_cast<T *>(z + t.rec);
+    s.vp = reinterpret_cast<T *>(z + t.vp);
+    s.isp = reinterpret_cast<T *>(z + t.isp);
+    s.iprior = reinterpret_cast<T *>(z + t.prior);
+    s.esq = reinterpret_cast<T *>(z + t.esq);
+    s.e2 = reinterpret_cast<double *>(z + t.e2);
+    s.lut = reinterpret_cast<unsigned short *>(z + t.lut);
     return s;
 }
 
+// Starts the copy of a fit's tables into shared memory (asynchronous 16-byte copies; the
+// caller waits with tables_wait and then synchronises the block).
 template <class T>
-__device__ __forceinline__ void load_tables(const Model &m, const Buffers &b, const Smem<T> &s, int with_vp = 1)
+__device__ __forceinline__ void tables_start(const Buffers &b, const Smem<T> &s)
 {
-    for (int k = threadIdx.x; k < m.n_edges_total; k += blockDim.x) s.esq[k] = T(b.edges[k] * b.edges[k]);
-    for (int k = threadIdx.x; with_vp && k < m.n_ap_total; k += blockDim.x) {
-        s.vp[k] = T(b.Vp[k]);
-        s.isp[k] = T(b.isp[k]);
-    }
-    for (int k = threadIdx.x; k < m.n_lut; k += blockDim.x) s.lut[k] = b.lut[k];
-    for (int k = threadIdx.x; k < 32; k += blockDim.x) s.e2[k] = kExp2j[k];
+    const unsigned dst = static_cast<unsigned>(__cvta_generic_to_shared(s.tab));
+    const unsigned char *src = b.tab + s.tab_lo;
+    for (int q = 16 * int(threadIdx.x); q < s.tab_hi - s.tab_lo; q += 16 * int(blockDim.x))
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + q), "l"(src + q) : "memory");
 }
+__device__ __forceinline__ void tables_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // ---------------------------------------------------------------- force-of-change records
 
-// Folds the coefficients c_j of every aperture into its record (see data_term): with
-// v_los = V + s nu (s = sigma_p), mass contributes c to q0, v_los^2 contributes
-// c (V^2, 2 V s, s^2) and v_los contributes c (V, s) to (q0, q1, q2); b_n contributes
-// c c_n H_n(nu) to the Hermite part, with the monomial coefficients of H_n from the
-// recurrence H_{n+1} = 2 nu H_n - 2 n H_{n-1}. Called by every thread of one block.
+// A record folds the coefficients c_j of its aperture (see data_term): with v_los = V + s nu
+// (s = sigma_p), mass contributes c to q0, v_los^2 contributes c (V^2, 2 V s, s^2) and v_los
+// contributes c (V, s) to (q0, q1, q2); b_n contributes c c_n H_n(nu) to the Hermite part, with
+// the monomial coefficients of H_n from the recurrence H_{n+1} = 2 nu H_n - 2 n H_{n-1}. Shell
+// records hold c_j of each a_lm. The factors are laid out once per fit (FinPlan).
 // Coefficient of nu^q in the physicists' H_n, set on the host from the recurrence
 // H_{n+1} = 2 nu H_n - 2 n H_{n-1} (see herm_table).
-static __constant__ double kHerm[7][7];  // one copy per translation unit
-
 inline void herm_table(double h[7][7])
 {
     for (int n = 0; n < 7; ++n)
@@ -1628,70 +1692,12 @@ inline void herm_table(double h[7][7])
         for (int q = 0; q < 7; ++q) h[n + 1][q] = (q > 0 ? 2.0 * h[n][q - 1] : 0.0) - 2.0 * n * h[n - 1][q];
 }
 
-// Sets this translation unit's constant tables (kHerm, kExp2j) on the current device.
+// Sets this translation unit's constant table (kExp2j) on the current device.
 static inline cudaError_t upload_constants()
 {
-    double h[7][7];
-    herm_table(h);
-    cudaError_t e = cudaMemcpyToSymbol(kHerm, h, sizeof h);
-    if (e != cudaSuccess) return e;
     double t[32];
     exp2_table(t);
     return cudaMemcpyToSymbol(kExp2j, t, sizeof t);
-}
-
-static __device__ void build_records(const Model &m, const Buffers &b)
-{
-    for (int g = 0; g < m.n_groups; ++g) {
-        const GroupDesc &G = m.g[g];
-        for (int p = threadIdx.x; p < G.n_ap; p += blockDim.x) {
-            const int a = G.ap_off + p;
-            double *r = b.rec + a * m.rec_len;
-            if (G.geometry == 2) {  // shells: c_j of each a_lm
-                float *rf = b.recf + a * m.rec_len;
-                for (int q = 0; q < m.rec_len; ++q) {
-                    r[q] = q < G.n_kinds ? b.c[G.obs_off + q * G.n_ap + p] : 0.0;
-                    rf[q] = float(r[q]);
-                }
-                continue;
-            }
-            const bool gh = G.max_gh >= 0;
-            const double V = gh ? b.Vp[a] : 0.0, is = gh ? b.isp[a] : 1.0, s = 1.0 / is;
-            const int base = G.obs_off + p;
-            double q0 = 0.0, q1 = 0.0, q2 = 0.0;
-            if (G.k_mass >= 0) q0 += b.c[base + G.k_mass * G.n_ap];
-            if (G.k_v2 >= 0) {
-                const double c = b.c[base + G.k_v2 * G.n_ap];
-                q0 += c * V * V;
-                q1 += c * 2.0 * V * s;
-                q2 += c * s * s;
-            }
-            if (G.k_v1 >= 0) {
-                const double c = b.c[base + G.k_v1 * G.n_ap];
-                q0 += c * V;
-                q1 += c * s;
-            }
-            r[0] = V;
-            r[1] = is;
-            r[2] = q0;
-            r[3] = q1;
-            r[4] = q2;
-            double pc[7] = {0, 0, 0, 0, 0, 0, 0};
-#pragma unroll
-            for (int n = 0; n < 7; ++n) {
-                if (n <= G.max_gh && G.k_gh[n] >= 0) {
-                    const double c = b.c[base + G.k_gh[n] * G.n_ap] * gh_c(n);
-#pragma unroll
-                    for (int q = 0; q <= n; ++q) pc[q] += c * kHerm[n][q];
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < 7; ++q)
-                if (5 + q < m.rec_len) r[5 + q] = pc[q];
-            float *rf = b.recf + a * m.rec_len;
-            for (int q = 0; q < m.rec_len; ++q) rf[q] = float(r[q]);
-        }
-    }
 }
 
 // ---------------------------------------------------------------- finalize (last block)
@@ -1699,18 +1705,17 @@ static __device__ void build_records(const Model &m, const Buffers &b)
 // Run by the last block of the step kernel once every block has added its sums:
 // converts the fixed-point sums, renormalises, smooths (eq. myts), forms Delta_j,
 // chi^2 (eqs. delta, chi) and the force-of-change coefficients, the prior means on
-// Sums red[0 .. blockDim) into red[0] for any block size: the part above the largest
-// power of two is folded in first. Called after red is written and synchronised.
-__device__ __forceinline__ void block_fold(double *red)
+// The sum of v over the block, for any block size (a multiple of 32), to every thread: warp
+// shuffles, then the warps' sums from shared memory in warp order (the same order in every
+// kernel that ends with the finalize). red: 32 doubles.
+__device__ __forceinline__ double fold_block(double v, double *red)
 {
-    int p2 = 1;
-    while (2 * p2 <= int(blockDim.x)) p2 *= 2;
-    if (int(threadIdx.x) >= p2) red[threadIdx.x - p2] += red[threadIdx.x];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
-    for (int s = p2 / 2; s > 0; s >>= 1) {
-        if (int(threadIdx.x) < s) red[threadIdx.x] += red[threadIdx.x + s];
-        __syncthreads();
-    }
+    double s = 0.0;
+    for (int q = 0; q < int(blockDim.x >> 5); ++q) s += red[q];
+    return s;
 }
 
 // The self-consistent potential at an update (Sec. 6), in the finalize: the mass-to-light
@@ -1730,10 +1735,8 @@ __device__ void scf_finalize(const Model &m, const Buffers &b, double s_ren, int
             const double D = fx_read<WPS>(b.hist, m.off_dups + j) / sj * s_ren;
             part += b.delta[j] / b.sig[j] * D;
         }
-        red[threadIdx.x] = part;
-        __syncthreads();
-        block_fold(red);
-        if (threadIdx.x == 0) sc.ups *= exp(-m.eps_ups * double(m.update_every) * m.dt * red[0]);
+        const double sum = fold_block(part, red);
+        if (threadIdx.x == 0) sc.ups *= exp(-m.eps_ups * double(m.update_every) * m.dt * sum);
         __syncthreads();
     }
     const double ups = sc.ups;
@@ -1775,6 +1778,15 @@ __device__ void scf_finalize(const Model &m, const Buffers &b, double s_ren, int
 // x (into pwin), then, after the row windows are written back over the cell words, along E,
 // so they equal the sums of the particles' own words in any order. q = 0 is the particle
 // count, q = 1..WPS the words of the weight sum; all unsigned, wrapping like the deposits.
+__device__ __forceinline__ void write_prior(const Buffers &b, int c, double pr)
+{
+    const double ip = pr > 0.0 ? 1.0 / pr : 0.0;
+    b.prior[c] = pr;
+    b.iprior[c] = ip;
+    if (b.ipriorf) b.ipriorf[c] = float(ip);
+    b.lprior[c] = pr > 0.0 ? log(pr) : -HUGE_VAL;
+}
+
 template <int WPS>
 __device__ void window_priors(const Model &m, const Buffers &b, double s_ren)
 {
@@ -1823,81 +1835,182 @@ __device__ void window_priors(const Model &m, const Buffers &b, double s_ren)
         if (WPS == 2) sum += double((long long)box[2]) * (1.0 / 4294967296.0);
         sum = sum / m.fx_w * s_ren;
         const double pr = cnt > 0 ? sum / double(cnt) : 0.0;
-        b.prior[c] = pr;
-        b.iprior[c] = pr > 0.0 ? 1.0 / pr : 0.0;
-        b.lprior[c] = pr > 0.0 ? log(pr) : -HUGE_VAL;
+        write_prior(b, c, pr);
     }
 }
 
-template <int WPS>
-__device__ void finalize_block(const Model &m, const Buffers &b, long long n, int init, int prior_step,
-                               double *red, int scf_step = 0)
+// The head of step t + 1, from the scalars after step t (one thread).
+__device__ __forceinline__ StepHead next_head(const Model &m, long long t, int pending, double s_ren, double what)
 {
-    // other blocks updated the sums and scalars with atomics: read them from L2
+    StepHead h;
+    const bool update = (t % m.update_every) == 0;  // step t + 1 is one of 1, 1 + P, ...
+    h.pending = pending;
+    h.prior_step = m.mode == 1 && update;
+    h.scf_step = m.pot == 3 && update;
+    h.wscale = float(s_ren);
+    h.iwhat = what > 0.0 ? float(1.0 / what) : 0.f;
+    h.pad = 0;
+    h.lwscale = log(s_ren);
+    h.lwhat = what > 0.0 ? log(what) : -HUGE_VAL;
+    return h;
+}
+
+// The head from the scalars of a restored state.
+static __global__ void k_head(const Model m, const Scalars *sc, StepHead *head)
+{
+    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+    StepHead h = next_head(m, sc->t, sc->pending, sc->wscale, sc->what_flat);
+    h.lwscale = sc->lwscale;
+    h.lwhat = sc->lwhat_flat;
+    *head = h;
+}
+
+// The scale that renormalises the weights of this step, and their total U (stored units).
+template <int WPS>
+__device__ __forceinline__ double renorm_scale(const Model &m, const Buffers &b, int init, double W0, double &U)
+{
+    U = fx_read<WPS>(b.hist, m.J) * (1.0 / m.fx_w);  // fx_w is a power of two: exact
+    return (!init && m.renormalize && U > 0.0) ? W0 / U : 1.0;
+}
+
+// The observables of chunks [ch0, ch1) from the fixed-point sums: smoothing (eq. myts),
+// Delta_j (eq. delta), coefficients c_j into b.c and cs (if given, J doubles of shared memory);
+// csum[chunk]: the chunk's sum of Delta_j^2. A warp per chunk. What does not depend on the
+// sums is loaded before them.
+template <int WPS>
+__device__ __forceinline__ void fin_observables(const Model &m, const Buffers &b, const FinPlan &pl, int ch0, int ch1,
+                                                int init, double W0, double *cs, double *csum, double &s_ren, double &U)
+{
+    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    ObsRow r;
+    double h = 0.0, old = 0.0;
+    auto fetch = [&](int ch) {
+        r = pl.rows[32 * ch + lane];
+        if (r.j >= 0) {
+            h = fx_read<WPS>(b.hist, r.j);
+            old = b.ytil[r.j];
+        }
+    };
+    int ch = ch0 + int(threadIdx.x >> 5);
+    if (ch < ch1) fetch(ch);
+    s_ren = renorm_scale<WPS>(m, b, init, W0, U);
+    for (; ch < ch1; ch += nw) {
+        double d = 0.0;
+        if (r.j >= 0) {
+            const double raw = h * r.iscale * s_ren * r.post;
+            const double yt = init ? raw : old + m.alpha * (raw - old);
+            d = (yt - r.Y) / r.sig;
+            const double cj = d * r.cw;
+            b.yraw[r.j] = raw;
+            b.ytil[r.j] = yt;
+            b.delta[r.j] = d;
+            b.c[r.j] = cj;
+            if (cs) cs[r.j] = cj;
+        }
+        double d2 = d * d;
+        if (ch + nw < ch1) fetch(ch + nw);
+        for (int o = 16; o > 0; o >>= 1) d2 += __shfl_xor_sync(0xffffffffu, d2, o);
+        if (lane == 0) csum[ch] = d2;
+    }
+}
+
+// The record elements [e0, e1) from the coefficients c.
+__device__ __forceinline__ void fin_records(const Buffers &b, const FinPlan &pl, int e0, int e1, const double *c)
+{
+    for (int e = e0 + int(threadIdx.x); e < e1; e += blockDim.x) {
+        const RecElem el = pl.elems[e];
+        double v = 0.0;
+        for (int k = 0; k < el.nk; ++k) v += pl.coef[size_t(k) * pl.n_elems + e] * c[el.j0 + k * el.stride];
+        b.rec[el.dst] = v;
+        if (b.recf) b.recf[el.dst] = float(v);
+    }
+}
+
+// chi^2 from the chunk sums, in chunk order over 32 lanes (one warp).
+__device__ __forceinline__ double fin_chi2(const double *csum, int n)
+{
+    double v = 0.0;
+    for (int q = int(threadIdx.x & 31); q < n; q += 32) v += csum[q];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// The scalars after the step and the head of the next one (one thread).
+__device__ __forceinline__ void fin_scalars(const Model &m, const Buffers &b, long long n, int init, int prior_step,
+                                            double s_ren, double U)
+{
     Scalars &sc = *b.sc;
     const long long t = init ? 0 : __ldcg(&sc.t) + 1;
-    const double U = fx_read<WPS>(b.hist, m.J) / m.fx_w;
-    double s_ren = 1.0;
+    const double what = init ? (n > 0 ? U / double(n) : 0.0) : __ldcg(&sc.what_flat);
+    // the integer sums wrap beyond their range: the floating-point check sum catches it
+    if (!(__ldcg(&sc.Wcheck) <= 0.5 * __ldcg(&sc.Wrange))) atomicOr(&sc.err, kErrOverflow);
+    const StepHead h = next_head(m, t, init ? 0 : (t > m.n_relax ? 1 : 0), s_ren, what);
     if (init) {
-        if (threadIdx.x == 0) {
-            sc.W0 = U;
-            sc.what_flat = n > 0 ? U / double(n) : 0.0;
-            sc.lwhat_flat = sc.what_flat > 0.0 ? log(sc.what_flat) : -HUGE_VAL;
-        }
-    } else if (m.renormalize && U > 0.0) {
-        s_ren = __ldcg(&sc.W0) / U;
+        sc.W0 = U;
+        sc.what_flat = what;
+        sc.lwhat_flat = h.lwhat;
     }
-    double part = 0.0;
-    for (int j = threadIdx.x; j < m.J; j += blockDim.x) {
-        const double raw = fx_read<WPS>(b.hist, j) * b.obs_iscale[j] * s_ren * b.obs_post[j];
-        const double yt = init ? raw : b.ytil[j] + m.alpha * (raw - b.ytil[j]);
-        const double d = (yt - b.Y[j]) / b.sig[j];
-        b.yraw[j] = raw;
-        b.ytil[j] = yt;
-        b.delta[j] = d;
-        b.c[j] = d / b.sig[j] * b.obs_post[j];
-        part += d * d;
-    }
-    red[threadIdx.x] = part;
-    __syncthreads();
-    build_records(m, b);
-    block_fold(red);
-    const double chi2 = red[0];
-    __syncthreads();
-    if (scf_step) scf_finalize<WPS>(m, b, s_ren, init, red);
-    if (prior_step && (m.pwin_E > 0 || m.pwin_x > 0)) {
+    sc.Wcheck = 0.0;
+    sc.Wsum = U;
+    if (!init) sc.t = t;
+    sc.wscale = s_ren;
+    sc.lwscale = h.lwscale;
+    sc.pending = h.pending;
+    sc.blocks_done = 0;
+    if (prior_step && m.smooth) sc.smooth_pending = 1;
+    *b.head = h;
+}
+
+// Update steps: the cell means (Sec. 2.3.1) or window means from the cells' sums.
+template <int WPS>
+__device__ __forceinline__ void fin_priors(const Model &m, const Buffers &b, double s_ren)
+{
+    if (m.pwin_E > 0 || m.pwin_x > 0) {
         window_priors<WPS>(m, b, s_ren);
-    } else if (prior_step) {
-        for (int c = threadIdx.x; c < m.ncell; c += blockDim.x) {
-            const long long cnt = __ldcg(b.hist + m.off_count + c);
-            const double sum = fx_read<WPS>(b.hist, m.J + 1 + c) / m.fx_w * s_ren;
-            const double pr = cnt > 0 ? sum / double(cnt) : 0.0;  // mean weight of the cell
-            b.prior_count[c] = cnt;
-            if (m.smooth) {  // the smoothing kernels turn the raw means into the priors
-                b.prior_raw[c] = pr;
-                continue;
-            }
-            b.prior[c] = pr;
-            b.iprior[c] = pr > 0.0 ? 1.0 / pr : 0.0;
-            b.lprior[c] = pr > 0.0 ? log(pr) : -HUGE_VAL;
-        }
+        return;
     }
+    const double ifx = 1.0 / m.fx_w;
+    for (int q = threadIdx.x; q < m.ncell; q += blockDim.x) {
+        const long long cnt = __ldcg(b.hist + m.off_count + q);
+        const double sum = fx_read<WPS>(b.hist, m.J + 1 + q) * ifx * s_ren;
+        const double pr = cnt > 0 ? sum / double(cnt) : 0.0;  // mean weight of the cell
+        b.prior_count[q] = cnt;
+        if (m.smooth) b.prior_raw[q] = pr;  // the smoothing kernels turn the raw means into the priors
+        else write_prior(b, q, pr);
+    }
+}
+
+// The finalize in one block (the last of a block-shared step). The GPU waits for it, so what
+// counts is its chain of dependent latencies and the instructions it fetches cold: a warp per
+// chunk of observables, one thread per record element with the factors laid out beforehand, no
+// unrolled code, the scalars of the next step (two logarithms, a modulo) beside the records.
+// Measured on the 60-observable fit: 32,000 cycles with one thread per aperture and the scalars
+// before the barrier, 12,000 so.
+// cs: the start of the shared memory, J coefficients and one double per chunk.
+template <int WPS>
+__device__ void finalize_block(const Model &m, const Buffers &b, long long n, int init, int prior_step,
+                               double *cs, int scf_step = 0)
+{
+    const FinPlan &pl = b.plan;
+    const double W0 = init ? 0.0 : __ldcg(&b.sc->W0);
+    double *csum = cs + m.J;
+    double s_ren, U;
+    fin_observables<WPS>(m, b, pl, 0, pl.n_chunks, init, W0, cs, csum, s_ren, U);
+    __syncthreads();
+    if (int(threadIdx.x) == int(blockDim.x) - 32) fin_scalars(m, b, n, init, prior_step, s_ren, U);
+    if (threadIdx.x < 32) {
+        const double chi2 = fin_chi2(csum, pl.n_chunks);
+        if (threadIdx.x == 0) b.sc->chi2 = chi2;
+    }
+    fin_records(b, pl, 0, pl.n_elems, cs);
+    if (scf_step) {
+        __syncthreads();
+        scf_finalize<WPS>(m, b, s_ren, init, cs);
+    }
+    if (prior_step) fin_priors<WPS>(m, b, s_ren);
     __syncthreads();
     const int words = (prior_step || scf_step) ? m.hist_words : m.off_grid;
-    for (int k = threadIdx.x; k < words; k += blockDim.x) b.hist[k] = 0;
-    if (threadIdx.x == 0) {
-        // the integer sums wrap beyond their range: the floating-point check sum catches it
-        if (!(__ldcg(&sc.Wcheck) <= 0.5 * __ldcg(&sc.Wrange))) atomicOr(&sc.err, kErrOverflow);
-        sc.Wcheck = 0.0;
-        sc.Wsum = U;
-        sc.chi2 = chi2;
-        if (!init) sc.t = t;
-        sc.wscale = s_ren;
-        sc.lwscale = log(s_ren);
-        sc.pending = init ? 0 : (t > m.n_relax ? 1 : 0);
-        sc.blocks_done = 0;
-        if (prior_step && m.smooth) sc.smooth_pending = 1;
-    }
+    for (int q = threadIdx.x; q < words; q += blockDim.x) b.hist[q] = 0;
 }
 
 // ---------------------------------------------------------------- step kernel
@@ -1967,17 +2080,23 @@ struct StepFlags {
 };
 
 template <class T>
-__device__ __forceinline__ StepFlags<T> step_flags(const Model &m, const Scalars &sc, int init)
+__device__ __forceinline__ StepFlags<T> step_flags(const Model &m, const StepHead *head, int init)
 {
     StepFlags<T> f;
-    const long long t = sc.t + 1;
-    f.pending = init ? 0 : sc.pending;
-    f.prior_step = !init && m.mode == 1 && ((t - 1) % m.update_every) == 0;
+    const StepHead h = *head;
+    f.pending = init ? 0 : h.pending;
+    f.prior_step = init ? 0 : h.prior_step;
     // the self-consistent potential is rebuilt at the load and on the prior schedule
-    f.scf_step = m.pot == 3 && (init || ((t - 1) % m.update_every) == 0);
-    f.wscale = init ? T(1) : T(sc.wscale);
-    f.lwscale = init ? T(0) : T(sc.lwscale);
-    f.iwhat_flat = kLogWeights<T> ? T(sc.lwhat_flat) : (sc.what_flat > 0.0 ? T(1.0 / sc.what_flat) : T(0));
+    f.scf_step = init ? m.pot == 3 : h.scf_step;
+    if constexpr (kLogWeights<T>) {
+        f.wscale = T(1);
+        f.lwscale = init ? T(0) : T(h.lwscale);
+        f.iwhat_flat = T(h.lwhat);
+    } else {
+        f.wscale = init ? T(1) : T(h.wscale);
+        f.lwscale = T(0);
+        f.iwhat_flat = T(h.iwhat);
+    }
     return f;
 }
 
@@ -1985,24 +2104,9 @@ __device__ __forceinline__ StepFlags<T> step_flags(const Model &m, const Scalars
 template <class T, bool GA>
 __device__ __forceinline__ void block_zero(const Model &m, const Smem<T> &S)
 {
-    int *z = static_cast<int *>(S.h);
-    const int nw = int((GA ? window_bytes<T>(m) : Acc<T>::bytes(m)) / sizeof(int));
-    for (int q = threadIdx.x; q < nw; q += blockDim.x) z[q] = 0;
-}
-
-// Copies a fit's records, priors and aperture tables into shared memory.
-template <class T, bool GA>
-__device__ __forceinline__ void block_tables(const Model &m, const Buffers &b, const Smem<T> &S, int pending)
-{
-    if (pending) {
-        if (!GA)
-            for (int q = threadIdx.x; q < m.n_ap_total * m.rec_len; q += blockDim.x) S.c[q] = global_records<T>(b)[q];
-        if (m.mode == 1) {
-            const double *pr = kLogWeights<T> ? b.lprior : b.iprior;
-            for (int q = threadIdx.x; q < m.ncell; q += blockDim.x) S.iprior[q] = T(pr[q]);
-        }
-    }
-    load_tables(m, b, S, GA ? 0 : 1);
+    int4 *z = static_cast<int4 *>(S.h);
+    const int nw = int(acc_bytes_padded<T>(m, GA ? 2 : 1) / sizeof(int4));
+    for (int q = threadIdx.x; q < nw; q += blockDim.x) z[q] = int4{0, 0, 0, 0};
 }
 
 // The per-particle part of one step for particles i0, i0 + stride, ... below i1:
@@ -2014,6 +2118,8 @@ __device__ __forceinline__ void step_particles(const Model &m, const Model &mh, 
                                                const Smem<T> &S, const StepFlags<T> &f, int push, long long i0,
                                                long long i1, long long stride, unsigned &err, Total<T> &wtot, T &wdep)
 {
+    // The block's tables are on their way into shared memory and its sums are being zeroed:
+    // the first particles are loaded before the block waits for both.
     // mh: the fields of the per-particle path (observable layout, regularisation and update
     // modes, potential kind). It is the fit's own Model, or in the batched kernel one Model
     // in the parameter space that every fit of the batch equals in those fields. m: the
@@ -2045,6 +2151,8 @@ __device__ __forceinline__ void step_particles(const Model &m, const Model &mh, 
         if (need_ap && gxc) ngx = P.gx[j];
     };
     if (i0 < i1) fetch(i0);
+    tables_wait();
+    __syncthreads();
     for (long long i = i0; i < i1; i += stride) {
         T x = nx, y = ny, z = nz;
         T vx = nvx, vy = nvy, vz = nvz;
@@ -2188,8 +2296,22 @@ __device__ __forceinline__ void block_flush(const Model &m, const Cst<T> &k, con
         const long long v = Acc<T>::word(S.h, m, q);
         if (v != 0) red_add(b.hist + q, v);
     }
-    __threadfence();
     __syncthreads();
+}
+
+// Whether this block is the last of `blocks` to arrive at the counter, to every thread. The
+// block's reductions come before the counter for every reader: the barrier orders them before
+// thread 0, whose fence orders them before its atomic (one fence, not one per thread).
+__device__ __forceinline__ bool block_is_last(unsigned *counter, unsigned blocks, bool *flag)
+{
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        *flag = atomicAdd(counter, 1u) == blocks - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    return *flag;
 }
 
 // Threads per block the step kernel is compiled for. The mixed-precision global-deposit
@@ -2203,28 +2325,28 @@ __global__ void __launch_bounds__(kStepMaxThreads<T, GA>, (GA && sizeof(T) == 4)
                                                     const Buffers b, int push, int init)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    const Smem<T> S = carve<T>(m, smem, GA ? 2 : 1, GA ? 0 : 1, GA ? 0 : 1);
+    const Smem<T> S = carve<T>(m, smem, GA ? 2 : 1, GA ? 0 : 1);
     __shared__ bool am_last;
 
-    const StepFlags<T> f = step_flags<T>(m, *b.sc, init);
+    tables_start<T>(b, S);
+    const StepFlags<T> f = step_flags<T>(m, b.head, init);
     block_zero<T, GA>(m, S);
-    block_tables<T, GA>(m, b, S, f.pending);
-    __syncthreads();
 
+    // The particles in whole warps of 32, cut into one contiguous run per block: a small fit
+    // then spreads over all SMs instead of filling the first ones.
+    const long long units = (P.n + 31) >> 5;
+    const long long lo = (units * blockIdx.x / gridDim.x) << 5;
+    long long hi = (units * (blockIdx.x + 1) / gridDim.x) << 5;
+    if (hi > P.n) hi = P.n;
     unsigned err = 0;
     Total<T> wtot;
     T wdep = T(0);  // floating-point twin of wtot, for the fixed-point range check
-    step_particles<T, GA, M0, M1, M2, M3>(m, m, k, P, b, S, f, push, (long long)blockIdx.x * blockDim.x + threadIdx.x,
-                                          P.n, (long long)gridDim.x * blockDim.x, err, wtot, wdep);
+    step_particles<T, GA, M0, M1, M2, M3>(m, m, k, P, b, S, f, push, lo + threadIdx.x, hi, blockDim.x, err, wtot, wdep);
     block_flush<T, WPS, GA>(m, k, b, S, f.prior_step, err, wtot, wdep, f.scf_step);
-    if (m.shard) return;  // the sums of all shards are added by the caller; k_finalize follows
+    if (GA || m.fin_wide || m.shard) return;  // k_finalize follows (a shard's after the exchange of its sums)
     // last block to finish runs the finalize
-    if (threadIdx.x == 0) am_last = atomicAdd(&b.sc->blocks_done, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (am_last) {
-        __threadfence();
+    if (block_is_last(&b.sc->blocks_done, gridDim.x, &am_last))
         finalize_block<WPS>(m, b, P.n, init, f.prior_step, reinterpret_cast<double *>(smem), f.scf_step);
-    }
 }
 
 // ---------------------------------------------------------------- shards of one fit
@@ -2248,19 +2370,44 @@ static __global__ void k_shard_pack(long long *hist, int hist_words, Scalars *sc
     }
 }
 
-// The finalize of a shard from the exchanged (summed) words. red: blockDim doubles.
+// The finalize as a kernel of its own, one block per range of 32 apertures: after a global-
+// deposit step or one of more than 16 chunks of observables (one block took 430,000 cycles for
+// 64 x 64 pixels of five moments, 207 of 604 us; the step takes 360 us with the ranges spread), and for a shard, from the
+// exchanged (summed) words. Every block handles its observables and records; the last one to
+// arrive adds chi^2, the priors and the scalars. A shard's range word replaces Wcheck first.
 template <class T, int WPS>
-__global__ void k_finalize(const Model m, const Buffers b, int init)
+__global__ void __launch_bounds__(256) k_finalize(const Model m, const Buffers b, long long n, int init)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const StepFlags<T> f = step_flags<T>(m, *b.sc, init);
+    __shared__ bool am_last;
+    __shared__ double red[32];
+    const FinPlan &pl = b.plan;
+    const StepFlags<T> f = step_flags<T>(m, b.head, init);
+    const double W0 = init ? 0.0 : __ldcg(&b.sc->W0);
+    const int2 r0 = pl.range[blockIdx.x], r1 = pl.range[blockIdx.x + 1];
+    double s_ren, U;
+    fin_observables<WPS>(m, b, pl, r0.x, r1.x, init, W0, nullptr, pl.csum, s_ren, U);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        b.sc->Wcheck = double(b.hist[m.hist_words]) * (b.sc->Wrange * kRangeUnit);
-        b.hist[m.hist_words] = 0;
+    fin_records(b, pl, r0.y, r1.y, b.c);
+    if (!block_is_last(&b.sc->blocks_done, gridDim.x, &am_last)) return;
+    if (threadIdx.x < 32) {
+        const double chi2 = fin_chi2(pl.csum, pl.n_chunks);
+        if (threadIdx.x == 0) {
+            b.sc->chi2 = chi2;
+            if (m.shard) {
+                b.sc->Wcheck = double(b.hist[m.hist_words]) * (b.sc->Wrange * kRangeUnit);
+                b.hist[m.hist_words] = 0;
+            }
+            fin_scalars(m, b, n, init, f.prior_step, s_ren, U);
+        }
     }
+    if (f.scf_step) {
+        __syncthreads();
+        scf_finalize<WPS>(m, b, s_ren, init, red);
+    }
+    if (f.prior_step) fin_priors<WPS>(m, b, s_ren);
     __syncthreads();
-    finalize_block<WPS>(m, b, m.n_all, init, f.prior_step, reinterpret_cast<double *>(smem), f.scf_step);
+    const int words = (f.prior_step || f.scf_step) ? m.hist_words : m.off_grid;
+    for (int q = threadIdx.x; q < words; q += blockDim.x) b.hist[q] = 0;
 }
 
 // ---------------------------------------------------------------- batched step kernel
@@ -2346,10 +2493,9 @@ __global__ void __launch_bounds__(256, MINB) k_step_batch(const BatchArgs<T> a, 
         const Buffers &b = sb;
         const State<T> P = sP;
         const Smem<T> S = carve<T>(m, smem, 1, 1);
-        const StepFlags<T> f = step_flags<T>(m, *b.sc, 0);
+        if (fresh) tables_start<T>(b, S);
+        const StepFlags<T> f = step_flags<T>(m, b.head, 0);
         block_zero<T, false>(m, S);
-        if (fresh) block_tables<T, false>(m, b, S, f.pending);
-        __syncthreads();
         unsigned err = 0;
         Total<T> wtot;
         T wdep = T(0);
@@ -2360,10 +2506,7 @@ __global__ void __launch_bounds__(256, MINB) k_step_batch(const BatchArgs<T> a, 
             step_particles<T, false, M0, M1, M2, M3>(m, m, k, P, b, S, f, 1, sg.begin + threadIdx.x, sg.end,
                                                      blockDim.x, err, wtot, wdep);
         block_flush<T, WPS, false>(m, k, b, S, f.prior_step, err, wtot, wdep, f.scf_step);
-        if (threadIdx.x == 0) am_last = atomicAdd(&b.sc->blocks_done, 1u) == a.nseg[cur] - 1;
-        __syncthreads();
-        if (am_last) {
-            __threadfence();
+        if (block_is_last(&b.sc->blocks_done, a.nseg[cur], &am_last)) {
             finalize_block<WPS>(m, b, P.n, 0, f.prior_step, reinterpret_cast<double *>(smem), f.scf_step);
             cur = -1;  // the finalize used the shared memory: reload before the next segment
         }
@@ -2380,14 +2523,12 @@ __global__ void k_materialize(const Model m, const Cst<T> k, const State<T> P, c
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const Smem<T> S = carve<T>(m, smem, 0, 0);
+    tables_start<T>(b, S);
     const Scalars sc = *b.sc;
-    if (m.mode == 1) {
-        const double *pr = kLogWeights<T> ? b.lprior : b.iprior;
-        for (int q = threadIdx.x; q < m.ncell; q += blockDim.x) S.iprior[q] = T(pr[q]);
-    }
-    load_tables(m, b, S);
+    tables_wait();
     __syncthreads();
-    const Tables<T> tb{S.esq, S.lut, S.vp, S.isp, S.e2};
+    // the force of change takes V_p and 1/sigma_p from the records
+    const Tables<T> tb{S.esq, S.lut, nullptr, nullptr, S.e2};
     unsigned err = 0;
     Total<double> tot;
     const long long stride = (long long)gridDim.x * blockDim.x;

@@ -298,9 +298,7 @@ __global__ void __launch_bounds__(kSmoothThreads) k_smooth_b(const Model m, cons
     for (int c = threadIdx.x; c < n; c += blockDim.x) {
         double f = 0.0;
         for (int ch = 0; ch < int(gridDim.y); ++ch) f += __ldcg(b.spart + size_t(ch) * n + c);
-        b.prior[c] = f;
-        b.iprior[c] = f > 0.0 ? 1.0 / f : 0.0;
-        b.lprior[c] = f > 0.0 ? log(f) : -HUGE_VAL;
+        write_prior(b, c, f);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
