@@ -386,6 +386,11 @@ static m2m_status build_model(m2m_ctx *ctx, const m2m_potential *pot, const m2m_
     ctx->precision = opt->precision;
     m.wps = ctx->precision == M2M_PREC_FP64 ? 2 : 1;
     m.cache_accel = m.pot != 3 && (ctx->precision == M2M_PREC_FP64 || m.pot == 1) ? 1 : 0;
+    m.int_force = ctx->precision == M2M_PREC_FP64 &&
+                  (m.pot == 2 ? big_range(m.v0 * m.v0) && big_range(m.q * m.q)
+                              : m.pot < 2 && big_range(m.G * m.M) && big_range(m.a) &&
+                                    (m.pot == 0 || (big_range(m.G * m.Ms) && big_range(m.rs))));
+    m.tab_smem = 1;
     m.off_total = m.J * m.wps;
     m.off_grid = (m.J + 1) * m.wps;
     // aperture cache: one 16-bit code per particle (two small groups or one group)
@@ -463,15 +468,17 @@ static m2m_status configure_kernels(m2m_ctx *ctx)
 {
     Model &m = ctx->m;
     // the finalize reuses the start of the dynamic shared memory for a block reduction
-    const size_t smem_shared = step_smem<T>(m);
     int maxsm = 0, smsm = 0;
     CU(cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
+    place_tables<T>(m, size_t(maxsm));
+    const size_t smem_shared = step_smem<T>(m);
     CU(cudaDeviceGetAttribute(&smsm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, ctx->device));
     // block-shared sums while the sums and records fit in shared memory, else global deposits
     if (ctx->deposit == M2M_DEPOSIT_SHARED && smem_shared > size_t(maxsm))
         return fail(ctx, M2M_ERR_ARG, "shared deposit needs %zu B of shared memory (limit %d)", smem_shared, maxsm);
     ctx->global_dep = ctx->deposit == M2M_DEPOSIT_GLOBAL ||
                       (ctx->deposit == M2M_DEPOSIT_AUTO && smem_shared > size_t(maxsm));
+    if (ctx->global_dep) m.tab_smem = smem_bytes<T>(m, 0, 0) <= size_t(maxsm) / 4;
     for (int g = 0; ctx->global_dep && g < m.n_groups; ++g)
         if (m.g[g].geometry == M2M_GEOM_SHELLS)
             return fail(ctx, M2M_ERR_ARG, "shell groups (a_lm) need the shared deposit (%zu B of shared memory, limit %d)",
@@ -539,7 +546,15 @@ static std::vector<unsigned char> host_tables(const m2m_ctx *ctx, const TabLayou
         isp[a] = T(ctx->isp[a]);
     }
     for (int e = 0; e < m.n_edges_total; ++e) esq[e] = T(ctx->edges[e] * ctx->edges[e]);
-    if (sizeof(T) == 8) exp2_table(reinterpret_cast<double *>(h.data() + t.e2));
+    if (sizeof(T) == 8) {
+        static const std::vector<u64> fn = [] {  // made once: long double functions
+            std::vector<u64> f(kExpEntries + 2 * kLnEntries);
+            exp_table(f.data());
+            ln_table(f.data() + kExpEntries);
+            return f;
+        }();
+        std::memcpy(h.data() + t.et, fn.data(), t.bytes - t.et);
+    }
     if (!ctx->lut.empty()) std::memcpy(h.data() + t.lut, ctx->lut.data(), sizeof(unsigned short) * ctx->lut.size());
     return h;
 }
@@ -2036,7 +2051,7 @@ __global__ void __launch_bounds__(256) k_static_observe(const Model m, const Cst
     __shared__ bool am_last;
     for (int q = threadIdx.x; q < 2 * m.J; q += blockDim.x) h[q] = 0;
     __syncthreads();
-    const Tables<double> tb{edges, nullptr, vp, isp, kExp2j};  // edges: squared
+    const StaticTables tb{edges, nullptr, vp, isp, kExp2j};  // edges: squared
     unsigned err = 0;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const double wi = w[i];
@@ -2047,8 +2062,9 @@ __global__ void __launch_bounds__(256) k_static_observe(const Model m, const Cst
             const GroupDesc &G = m.g[g];
             const int p = aperture<kDyn>(G, tb.esq, nullptr, x[i], Y);
             if (p >= 0) {
-                if (G.has_v2 && vlos * vlos > k.v2max) err |= kErrOverflow;
-                group_kernels<kDyn>(G, tb, p, vlos, wi, [&](int j, double v, int cls, int) {
+                const double vv = vlos * vlos;
+                if (G.has_v2 && vv > k.v2max) err |= kErrOverflow;
+                group_kernels<kDyn>(G, tb, p, vlos, vv, wi, [&](int j, double v, int cls, int) {
                     Acc<double>::add(h, m, j, v, cls == kClassMass ? m.fx_w : (cls == kClassVel ? m.fx_v2 : m.fx_gh));
                 });
             }

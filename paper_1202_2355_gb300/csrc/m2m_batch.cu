@@ -76,7 +76,7 @@ static bool group_hot_equal(const GroupDesc &a, const GroupDesc &b)
 static bool hot_equal(const Model &a, const Model &b)
 {
     bool eq = a.pot == b.pot && a.mode == b.mode && a.update_rule == b.update_rule && a.ap_cache == b.ap_cache &&
-              a.cache_accel == b.cache_accel && a.gx_group == b.gx_group && a.J == b.J && a.nslots == b.nslots &&
+              a.cache_accel == b.cache_accel && a.int_force == b.int_force && a.gx_group == b.gx_group && a.J == b.J && a.nslots == b.nslots &&
               a.off_count == b.off_count && a.rec_len == b.rec_len && a.n_groups == b.n_groups &&
               a.win_group == b.win_group && a.win_lo == b.win_lo && a.win_n == b.win_n && a.n_dups == b.n_dups &&
               a.off_dups == b.off_dups;

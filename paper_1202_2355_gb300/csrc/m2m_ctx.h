@@ -159,6 +159,15 @@ inline size_t step_smem(const m2m::Model &m)
     return a > b ? a : b;
 }
 
+// The tables of the FP64 functions stay in global memory where a block-shared step kernel
+// would need more shared memory with them than a block can have.
+template <class T>
+inline void place_tables(m2m::Model &m, size_t limit)
+{
+    m.tab_smem = 1;
+    m.tab_smem = step_smem<T>(m) <= limit ? 1 : 0;
+}
+
 // Resident blocks per SM the step kernels are compiled for (register budget). The
 // batched mixed-precision kernel runs best at 4 blocks of 256 (64 registers; 1.147 ms
 // against 1.176 ms at 5 blocks on the 96-fit workload), the single-fit one at 5.

@@ -14,6 +14,7 @@
 #include <cuda_runtime.h>
 
 #include "fp64_exp.cuh"
+#include "fp64_int.cuh"
 
 namespace m2m {
 
@@ -122,6 +123,9 @@ struct Model {
     // the finalize of a step runs as k_finalize over several blocks instead of in the last
     // block of the step kernel (see configure_kernels)
     int fin_wide;
+    // FP64 mode: the potential's constants are in the range of the integer force factors
+    // (big_range), and whether the tables of the integer functions are in shared memory
+    int int_force, tab_smem;
 };
 
 constexpr unsigned kApNone8 = 0xFFu, kApNone16 = 0xFFFFu;
@@ -201,6 +205,7 @@ struct alignas(16) Cst {
     T dt, hdt, dteps, mu, v2max, fx_w, fx_v2, fx_gh, fx_dv;
     T s_lo, s_den, e_scale, nE, nx;
     T lc_lnr0, lc_dlnr, lc_r0, lc_rmax;
+    T iq2;  // 1/q2
 };
 
 template <class T>
@@ -208,6 +213,7 @@ inline Cst<T> make_cst(const Model &m)
 {
     Cst<T> k;
     k.GM = T(m.G * m.M); k.a = T(m.a); k.GMs = T(m.G * m.Ms); k.rs = T(m.rs);
+    k.iq2 = T(1.0 / (m.q * m.q));
     k.v0sq = T(m.v0 * m.v0); k.r0sq = T(m.r0 * m.r0); k.q2 = T(m.q * m.q);
     k.phi_min = T(m.phi_min); k.hn_phi0 = T(m.rs > 0 ? -m.G * m.Ms / m.rs : 0.0);
     k.sin_i = T(m.sin_i); k.cos_i = T(m.cos_i);
@@ -403,6 +409,15 @@ __host__ __device__ __forceinline__ bool d_finite(float x) { return isfinite(x);
 __host__ __device__ __forceinline__ bool d_finite(double x) { return isfinite(x); }
 
 // ---------------------------------------------------------------- potentials
+
+// a / q^2 of the flattened halo. FP64: the product with 1/q^2 and its exact residual (3 FP64
+// instructions where a division takes 10), the correctly rounded quotient up to rare ties.
+__host__ __device__ __forceinline__ float div_q2(const Cst<float> &k, float a) { return d_div(a, k.q2); }
+__host__ __device__ __forceinline__ double div_q2(const Cst<double> &k, double a)
+{
+    const double t = a * k.iq2;
+    return fma(fma(-t, k.q2, a), k.iq2, t);
+}
 
 // NFW enclosed-mass factor mu(q) = ln(1+q) - q/(1+q), FP64. For small q the two terms
 // cancel: below q = 1e-3 the alternating series sum_k (-1)^k (k-1)/k q^k (Horner).
@@ -616,15 +631,33 @@ __host__ __device__ __forceinline__ T potential(const Model &m, const Cst<T> &k,
 
 // Force factor f of the acceleration at (x, y, z): a = -f (x, y, z) in the spherical
 // potentials (f = g(r)/r with g = G M(<r)/r^2), a = f (x, y, z/q^2) in the flattened log
-// halo (f = -v0^2/D).
+// halo (f = -v0^2/D). lnt: FP64 mode, the logarithm table of the integer force factors
+// (fp64_int.cuh); null takes the library functions. Per particle the Hernquist factor costs 3
+// FP64 instructions so instead of 27 (with the halo 3 instead of about 90).
 template <class T>
-__host__ __device__ __forceinline__ T accel_factor(const Model &m, const Cst<T> &k, T x, T y, T z)
+__host__ __device__ __forceinline__ T accel_factor(const Model &m, const Cst<T> &k, T x, T y, T z,
+                                                   const u64 *lnt = nullptr)
 {
     if (m.pot == 2) {
+        if constexpr (sizeof(T) == 8) {
+            const T D = fma(x, x, fma(y, y, k.r0sq)) + (lnt && m.int_force ? div_q2(k, z * z) : d_div(z * z, k.q2));
+            if (lnt && m.int_force && big_range(D))
+                return -big_double(big_norm(big_mul_raw(big_rcp(big_of(D)), big_of(k.v0sq))));
+            return -d_div(k.v0sq, D);
+        }
         const T D = fma(x, x, fma(y, y, k.r0sq)) + d_div(z * z, k.q2);
         return -d_div(k.v0sq, D);
     }
     const T r2 = fma(x, x, fma(y, y, z * z));
+    if constexpr (sizeof(T) == 8) {
+        if (lnt && m.int_force && big_range(r2)) {
+            Big r, ir;
+            big_rsqrt(big_of(r2), ir, r);
+            Big f = hernquist_big(k.GM, k.a, r, ir);
+            if (m.pot == 1) f = big_add(f, nfw_big(k.GMs, k.rs, r, ir, lnt));
+            return big_double(f);
+        }
+    }
     if (is_zero(r2)) return T(0);
     const T r = d_sqrt(r2);
     const T ra = r + k.a;
@@ -650,7 +683,7 @@ __host__ __device__ __forceinline__ void accel_from(const Model &m, const Cst<T>
     if (m.pot == 2) {
         ax = f * x;
         ay = f * y;
-        az = d_div(f * z, k.q2);
+        az = m.int_force ? div_q2(k, f * z) : d_div(f * z, k.q2);
         return;
     }
     ax = -f * x;
@@ -677,7 +710,7 @@ __host__ __device__ __forceinline__ void accel(const Model &m, const Cst<T> &k, 
 // returns the factor at the end position in f.
 template <class T>
 __device__ __forceinline__ void leapfrog_from(const Model &m, const Cst<T> &k, T &x, T &y, T &z, T &vx, T &vy, T &vz,
-                                              T &f)
+                                              T &f, const u64 *lnt)
 {
     T ax, ay, az;
     accel_from(m, k, f, x, y, z, ax, ay, az);
@@ -687,7 +720,7 @@ __device__ __forceinline__ void leapfrog_from(const Model &m, const Cst<T> &k, T
     x = fma(k.dt, vx, x);
     y = fma(k.dt, vy, y);
     z = fma(k.dt, vz, z);
-    f = accel_factor(m, k, x, y, z);
+    f = accel_factor(m, k, x, y, z, lnt);
     accel_from(m, k, f, x, y, z, ax, ay, az);
     vx = fma(k.hdt, ax, vx);
     vy = fma(k.hdt, ay, vy);
@@ -723,6 +756,15 @@ __device__ __forceinline__ void project(const Cst<T> &k, T y, T z, T vy, T vz, T
     vlos = fma(vy, k.sin_i, vz * k.cos_i);
 }
 
+// x >= 0 truncated to FP32 (0 below its normal range, its largest value above) with integer
+// operations: the conversion would wait for the FP64 pipe.
+__device__ __forceinline__ float float_near(double x)
+{
+    const int hi = __double2hiint(x) - ((1023 - 127) << 20);
+    const unsigned lo = unsigned(__double2loint(x));
+    return hi < (1 << 20) ? 0.f : (hi >= (255 << 20) ? 3.4e38f : __uint_as_float((unsigned(hi) << 3) | (lo >> 29)));
+}
+
 // Aperture of sky point (X, Y) in group G, or -1: half-open annuli
 // [edge_p, edge_p+1) in R = sqrt(X^2 + Y^2), decided on R^2 against squared edges
 // (so the decision can differ from one made on R only within a few ulp of an
@@ -744,7 +786,7 @@ __device__ __forceinline__ int aperture(const GroupDesc &G, const double *esq, c
         if (r < __double_as_longlong(e[0]) || r >= __double_as_longlong(e[G.n_ap])) return -1;
         int p;
         if (G.lut_n > 0) {
-            int b = __float2int_rd((__log2f(__double2float_rn(R2)) - G.l0) * G.lscale);
+            int b = __float2int_rd((__log2f(float_near(R2)) - G.l0) * G.lscale);
             b = b < 0 ? 0 : (b >= G.lut_n ? G.lut_n - 1 : b);
             p = G.lut_identity ? b : int(lut[G.lut_off + b]);
             // the candidate is right but within rounding of an edge or for crowded edges
@@ -814,47 +856,77 @@ struct Tables {
     const T *esq;         // per group squared edges
     const unsigned short *lut;
     const T *vp, *isp;
-    const double *e2;     // FP64 mode: 2^(j/32), j < 32 (exp_tab)
+    const u64 *et, *ln;   // FP64 mode: the tables of exp_int and ln_frac (null without one)
 };
 
-// exp of the kernel values and weights: the ex2-based approximation in mixed mode,
-// the table-driven exp_tab in FP64 mode.
+// Tables of the observables without a context: constant memory instead of a fit's tables.
+struct StaticTables {
+    const double *esq;
+    const unsigned short *lut;
+    const double *vp, *isp;
+    const double *e2;     // 2^(j/32), j < 32 (exp_tab)
+};
+
+// exp of the weights, and exp(-t/2) of the kernel values: the ex2-based approximation in mixed
+// mode, the integer exponential in FP64 mode.
 __device__ __forceinline__ float kexp(const Tables<float> &, float x) { return __expf(x); }
-__device__ __forceinline__ double kexp(const Tables<double> &tb, double x) { return exp_tab(x, tb.e2); }
+__device__ __forceinline__ double kexp(const Tables<double> &tb, double x) { return exp_int(x, tb.et); }
+__device__ __forceinline__ float kexp_mhalf(const Tables<float> &, float t) { return __expf(-0.5f * t); }
+__device__ __forceinline__ double kexp_mhalf(const Tables<double> &tb, double t) { return exp_mhalf(t, tb.et); }
+__device__ __forceinline__ double kexp_mhalf(const StaticTables &tb, double t) { return exp_tab(-0.5 * t, tb.e2); }
+
+// Coefficient of t^k, t = nu^2, in c_n H_n(nu) (n even) or c_n H_n(nu)/nu (n odd), from the
+// explicit sum H_n = n! sum_j (-1)^j (2 nu)^(n-2j) / (j! (n-2j)!).
+__host__ __device__ constexpr double gh_coef(int n, int k)
+{
+    const int j = n / 2 - k, p = n - 2 * j;
+    double v = gh_c(n) * (j % 2 ? -1.0 : 1.0);
+    for (int i = 2; i <= n; ++i) v *= i;
+    for (int i = 2; i <= j; ++i) v /= i;
+    for (int i = 2; i <= p; ++i) v /= i;
+    for (int i = 0; i < p; ++i) v *= 2.0;
+    return v;
+}
+template <int n, class T>
+__device__ __forceinline__ T gh_poly(T t)
+{
+    T s = T(gh_coef(n, n / 2));
+#pragma unroll
+    for (int k = n / 2 - 1; k >= 0; --k) s = fma(s, t, T(gh_coef(n, k)));
+    return s;
+}
 
 // Emits emit(slot, w K_slot, class, kind index in the group) for every kernel of group G
 // at aperture p:
-// surface mass (K = 1), v_los^2, v_los, and the Gauss-Hermite b_n with H_n from the
-// recurrence H_{n+1} = 2 nu H_n - 2 n H_{n-1}, evaluated once up to the group's
-// highest order.
-template <unsigned M, class T, class F>
-__device__ __forceinline__ void group_kernels(const GroupDesc &G, const Tables<T> &tb, int p, T vlos, T w, F &&emit,
+// surface mass (K = 1), v_los^2 (vv), v_los, and the Gauss-Hermite b_n: c_n H_n(nu) as a
+// polynomial in nu^2 times w exp(-nu^2/2), times nu for odd n (8 multiplications and fused
+// multiply-adds for h3 and h4, 15 by the recurrence in n).
+template <unsigned M, class T, class TB, class F>
+__device__ __forceinline__ void group_kernels(const GroupDesc &G, const TB &tb, int p, T vlos, T vv, T w, F &&emit,
                                               T *gexp_out = nullptr)
 {
     using P = GP<M>;
     const int base = G.obs_off + p;
     if (P::mass(G)) emit(base + G.k_mass * G.n_ap, w, kClassMass, G.k_mass);
-    if (P::v2(G)) emit(base + G.k_v2 * G.n_ap, w * vlos * vlos, kClassVel, G.k_v2);
+    if (P::v2(G)) emit(base + G.k_v2 * G.n_ap, w * vv, kClassVel, G.k_v2);
     if (P::v1(G)) emit(base + G.k_v1 * G.n_ap, w * vlos, kClassVel, G.k_v1);
-    const int nmax = P::max_gh(G);
-    if (nmax >= 0) {
+    if (P::max_gh(G) >= 0) {
         const T nu = (vlos - tb.vp[G.ap_off + p]) * tb.isp[G.ap_off + p];
-        const T ge = kexp(tb, T(-0.5) * nu * nu);
+        const T t = nu * nu;
+        const T ge = kexp_mhalf(tb, t);
         if (gexp_out) *gexp_out = ge;
-        const T we = w * ge;
-        T hm1 = T(1), h = T(2) * nu;
-        if (P::gh(G, 0)) emit(base + G.k_gh[0] * G.n_ap, T(gh_c(0)) * we, kClassGH, G.k_gh[0]);
-        if (P::gh(G, 1)) emit(base + G.k_gh[1] * G.n_ap, h * we, kClassGH, G.k_gh[1]);
-#pragma unroll
-        for (int n = 1; n < 6; ++n) {
-            if (n < nmax) {
-                const T hn1 = fma(T(2) * nu, h, -(T(2 * n) * hm1));
-                hm1 = h;
-                h = hn1;
-                if (P::gh(G, n + 1))
-                    emit(base + G.k_gh[n + 1] * G.n_ap, T(gh_c(n + 1)) * h * we, kClassGH, G.k_gh[n + 1]);
-            }
-        }
+        const T we = w * ge, wo = we * nu;
+        auto put = [&](auto N) {
+            constexpr int n = decltype(N)::value;
+            if (P::gh(G, n)) emit(base + G.k_gh[n] * G.n_ap, gh_poly<n>(t) * (n % 2 ? wo : we), kClassGH, G.k_gh[n]);
+        };
+        put(std::integral_constant<int, 0>{});
+        put(std::integral_constant<int, 1>{});
+        put(std::integral_constant<int, 2>{});
+        put(std::integral_constant<int, 3>{});
+        put(std::integral_constant<int, 4>{});
+        put(std::integral_constant<int, 5>{});
+        put(std::integral_constant<int, 6>{});
     }
 }
 
@@ -905,7 +977,7 @@ __device__ __forceinline__ T group_data(const Model &m, const GroupDesc &G, cons
 #pragma unroll
         for (int n = 6; n >= 0; --n)
             if (n <= nmax) poly = fma(poly, nu, r[5 + n]);
-        d = fma(gexp ? *gexp : kexp(tb, T(-0.5) * nu * nu), poly, d);
+        d = fma(gexp ? *gexp : kexp_mhalf(tb, nu * nu), poly, d);
     }
     return d;
 }
@@ -1144,7 +1216,7 @@ __device__ __forceinline__ void group_dkernels(const GroupDesc &G, const Tables<
     if (nmax >= 0) {
         const T is = tb.isp[G.ap_off + p];
         const T nu = (vlos - tb.vp[G.ap_off + p]) * is;
-        const T half = T(0.5) * w * vlos * is * kexp(tb, T(-0.5) * nu * nu);
+        const T half = T(0.5) * w * vlos * is * kexp_mhalf(tb, nu * nu);
         T hm1 = T(0), h = T(1);  // H_(n-1), H_n at n = 0
 #pragma unroll
         for (int n = 0; n <= 6; ++n) {
@@ -1474,6 +1546,7 @@ struct Total;
 template <>
 struct Total<double> {
     long long hi = 0, lo = 0;
+    long long top = 0;  // sum of hi 2^-20, which cannot wrap: the range check
     __device__ void add(double v, double scale)
     {
         long long a, b;
@@ -1485,7 +1558,10 @@ struct Total<double> {
     {
         hi += q.hi;
         lo += q.lo;
+        top += q.hi >> 20;
     }
+    // the deposited weight for the range check (an FP64 sum would take the FP64 pipe)
+    __device__ double range_sum(double, double scale) const { return double(top) * 1048576.0 / scale; }
     __device__ long long word(int q, double) const { return q == 0 ? hi : lo; }
 };
 
@@ -1497,6 +1573,7 @@ struct Total<float> {
     long long s = 0;
     __device__ void add(float v, float scale) { s += __float2ll_rn(v * scale); }
     __device__ void add_fx(const Acc<float>::Fx &q) { s += q.L; }
+    __device__ float range_sum(float wdep, float) const { return wdep; }
     __device__ long long word(int, float) const { return s; }
 };
 
@@ -1579,13 +1656,14 @@ __device__ __forceinline__ T foc_update_log(const Model &m, const Cst<T> &k, con
 
 // The step's tables in the state type T, as one block of global memory per fit that a block
 // of the step kernel copies into shared memory as it is, in 16-byte pieces: the force-of-
-// change records, V_p and 1/sigma_p, 1/prior (ln prior in FP64 mode), the squared edges,
-// 2^(j/32) (FP64 mode) and the annulus lookup. The finalize writes the records and priors in
+// change records, V_p and 1/sigma_p, 1/prior (ln prior in FP64 mode), the squared edges, the
+// annulus lookup and in FP64 mode the tables of the exponential and the logarithm (read from
+// global memory where they are what no longer fits, Model::tab_smem). The finalize writes the records and priors in
 // place; the rest is laid out at creation. (Converting every table from FP64 in every block took
 // 15,000 cycles of a step with 2,700 priors, and 5,800 with 300.) The global-deposit kernel and the
 // weight read-out take the part from the priors on. Offsets in bytes.
 struct TabLayout {
-    int rec, vp, isp, prior, esq, e2, lut, bytes;
+    int rec, vp, isp, prior, esq, lut, et, ln, bytes;
 };
 
 template <class T>
@@ -1598,9 +1676,10 @@ __host__ __device__ inline TabLayout tab_layout(const Model &m)
     t.isp = t.vp + up(sizeof(T) * size_t(m.n_ap_total));
     t.prior = t.isp + up(sizeof(T) * size_t(m.n_ap_total));
     t.esq = t.prior + up(sizeof(T) * size_t(m.ncell));
-    t.e2 = t.esq + up(sizeof(T) * size_t(m.n_edges_total));
-    t.lut = t.e2 + (sizeof(T) == 8 ? 32 * int(sizeof(double)) : 0);
-    t.bytes = t.lut + up(sizeof(unsigned short) * size_t(m.n_lut));
+    t.lut = t.esq + up(sizeof(T) * size_t(m.n_edges_total));
+    t.et = t.lut + up(sizeof(unsigned short) * size_t(m.n_lut));
+    t.ln = t.et + (sizeof(T) == 8 ? kExpEntries * int(sizeof(u64)) : 0);
+    t.bytes = t.ln + (sizeof(T) == 8 && m.pot == 1 ? 2 * kLnEntries * int(sizeof(u64)) : 0);
     return t;
 }
 
@@ -1608,8 +1687,8 @@ template <class T>
 struct Smem {
     void *h;               // fixed-point sums of the block (layout of Acc<T>)
     T *c, *iprior, *esq, *vp, *isp;  // c: the force-of-change records; iprior: 1/prior, or ln prior (FP64)
-    double *e2;            // 2^(j/32) for exp_tab
     unsigned short *lut;
+    const u64 *et, *ln;    // tables of exp_int and ln_frac
     unsigned char *tab;    // start of the copied tables, and the range of them that is copied
     int tab_lo, tab_hi;
 };
@@ -1638,26 +1717,28 @@ template <class T>
 __host__ __device__ inline size_t smem_bytes(const Model &m, int with_hist, int with_rec = 1)
 {
     const TabLayout t = tab_layout<T>(m);
-    return (with_hist ? acc_bytes_padded<T>(m, with_hist) : 0) + size_t(t.bytes - (with_rec ? 0 : t.prior));
+    return (with_hist ? acc_bytes_padded<T>(m, with_hist) : 0) + size_t((m.tab_smem ? t.bytes : t.et) - (with_rec ? 0 : t.prior));
 }
 
 template <class T>
-__device__ __forceinline__ Smem<T> carve(const Model &m, unsigned char *base, int with_hist, int with_rec = 1)
+__device__ __forceinline__ Smem<T> carve(const Model &m, const Buffers &b, unsigned char *base, int with_hist,
+                                         int with_rec = 1)
 {
     const TabLayout t = tab_layout<T>(m);
     Smem<T> s;
     s.h = base;
     s.tab = base + (with_hist ? acc_bytes_padded<T>(m, with_hist) : 0);
     s.tab_lo = with_rec ? 0 : t.prior;
-    s.tab_hi = t.bytes;
+    s.tab_hi = m.tab_smem ? t.bytes : t.et;
     unsigned char *z = s.tab - s.tab_lo;
     s.c = reinterpret_cast<T *>(z + t.rec);
     s.vp = reinterpret_cast<T *>(z + t.vp);
     s.isp = reinterpret_cast<T *>(z + t.isp);
     s.iprior = reinterpret_cast<T *>(z + t.prior);
     s.esq = reinterpret_cast<T *>(z + t.esq);
-    s.e2 = reinterpret_cast<double *>(z + t.e2);
     s.lut = reinterpret_cast<unsigned short *>(z + t.lut);
+    s.et = reinterpret_cast<const u64 *>((m.tab_smem ? z : b.tab) + t.et);
+    s.ln = reinterpret_cast<const u64 *>((m.tab_smem ? z : b.tab) + t.ln);
     return s;
 }
 
@@ -2126,7 +2207,7 @@ __device__ __forceinline__ void step_particles(const Model &m, const Model &mh, 
     // fit's own Model, for the prior binning and the self-consistent potential.
     // the self-consistent potential runs in the generic kernel only (the host picks it)
     constexpr bool kScf = M0 == kDyn;
-    const Tables<T> tb{S.esq, S.lut, GA ? global_vp<T>(b) : S.vp, GA ? global_isp<T>(b) : S.isp, S.e2};
+    const Tables<T> tb{S.esq, S.lut, GA ? global_vp<T>(b) : S.vp, GA ? global_isp<T>(b) : S.isp, S.et, S.ln};
     const T *rec = GA ? global_records<T>(b) : S.c;
     auto deposit = [&](int slot, T v, T scale) {
         if constexpr (GA) global_add(b.hist, slot, v, scale);
@@ -2183,9 +2264,9 @@ __device__ __forceinline__ void step_particles(const Model &m, const Model &mh, 
             T fa;
             if (push) {
                 fa = fa_in;
-                leapfrog_from(mh, k, x, y, z, vx, vy, vz, fa);
+                leapfrog_from(mh, k, x, y, z, vx, vy, vz, fa, tb.ln);
             } else {
-                fa = accel_factor(mh, k, x, y, z);
+                fa = accel_factor(mh, k, x, y, z, tb.ln);
             }
             P.fa[i] = fa;
         } else {
@@ -2212,9 +2293,10 @@ __device__ __forceinline__ void step_particles(const Model &m, const Model &mh, 
                 if (cache) code_out = ap_encode(mh, code_out, g, p);
                 if (p >= 0) {
                     // the v^2 sums' range assumes v^2 <= v2max (energy bound with headroom)
-                    if (GP<M>::v2(G) && gt_nonneg(vlos * vlos, k.v2max)) err |= kErrOverflow;
+                    const T vv = vlos * vlos;
+                    if (GP<M>::v2(G) && gt_nonneg(vv, k.v2max)) err |= kErrOverflow;
                     group_kernels<M>(
-                        G, tb, p, vlos, w,
+                        G, tb, p, vlos, vv, w,
                         [&](int j, T v, int cls, int kk) {
                             const T scale = cls == kClassMass ? k.fx_w : (cls == kClassVel ? k.fx_v2 : k.fx_gh);
                             if constexpr (GA) {
@@ -2245,7 +2327,7 @@ __device__ __forceinline__ void step_particles(const Model &m, const Model &mh, 
             if (cache) P.ap[i] = static_cast<uint16_t>(code_out);
             if (gxc) P.gx[i] = gout;
             wtot.add_fx(wfx);
-            wdep += w;
+            if constexpr (sizeof(T) == 4) wdep += w;
         }
         if (f.prior_step) {
             const int c = prior_cell<T, kScf>(m, k, b.lcE, x, y, z, vx, vy, vz);
@@ -2276,6 +2358,7 @@ __device__ __forceinline__ void block_flush(const Model &m, const Cst<T> &k, con
         if ((threadIdx.x & 31) == 0 && v != 0)
             red_add(b.hist + WPS * m.J + q, v);
     }
+    wdep = wtot.range_sum(wdep, k.fx_w);
     for (int o = 16; o > 0; o >>= 1) wdep += __shfl_xor_sync(0xffffffffu, wdep, o);
     if ((threadIdx.x & 31) == 0 && wdep != T(0)) atomicAdd(&b.sc->Wcheck, double(wdep));
     __syncthreads();
@@ -2325,7 +2408,7 @@ __global__ void __launch_bounds__(kStepMaxThreads<T, GA>, (GA && sizeof(T) == 4)
                                                     const Buffers b, int push, int init)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    const Smem<T> S = carve<T>(m, smem, GA ? 2 : 1, GA ? 0 : 1);
+    const Smem<T> S = carve<T>(m, b, smem, GA ? 2 : 1, GA ? 0 : 1);
     __shared__ bool am_last;
 
     tables_start<T>(b, S);
@@ -2492,7 +2575,7 @@ __global__ void __launch_bounds__(256, MINB) k_step_batch(const BatchArgs<T> a, 
         }
         const Buffers &b = sb;
         const State<T> P = sP;
-        const Smem<T> S = carve<T>(m, smem, 1, 1);
+        const Smem<T> S = carve<T>(m, b, smem, 1, 1);
         if (fresh) tables_start<T>(b, S);
         const StepFlags<T> f = step_flags<T>(m, b.head, 0);
         block_zero<T, false>(m, S);
@@ -2522,13 +2605,13 @@ __global__ void k_materialize(const Model m, const Cst<T> k, const State<T> P, c
                               long long *acc)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    const Smem<T> S = carve<T>(m, smem, 0, 0);
+    const Smem<T> S = carve<T>(m, b, smem, 0, 0);
     tables_start<T>(b, S);
     const Scalars sc = *b.sc;
     tables_wait();
     __syncthreads();
     // the force of change takes V_p and 1/sigma_p from the records
-    const Tables<T> tb{S.esq, S.lut, nullptr, nullptr, S.e2};
+    const Tables<T> tb{S.esq, S.lut, nullptr, nullptr, S.et, S.ln};
     unsigned err = 0;
     Total<double> tot;
     const long long stride = (long long)gridDim.x * blockDim.x;
