@@ -445,16 +445,12 @@ static typename StepKernel<T>::Fn step_fn() { return k_step<T, WPS, kMinBlocks<T
 template <class T, int WPS, bool GA>
 static typename StepKernel<T>::Fn pick_step(const Model &m)
 {
-    // the self-consistent potential is compiled into the generic kernel only
-    if (m.pot == 3) return step_fn<T, WPS, GA, kDyn, kDyn, kDyn, kDyn>();
-    unsigned mk[4] = {0, 0, 0, 0};
-    for (int g = 0; g < m.n_groups; ++g) mk[g] = group_mask(m.g[g]);
-    constexpr unsigned kin1 = kBitV2 | bit_gh(4), kin2 = kBitV2 | bit_gh(3) | bit_gh(4);
-    constexpr unsigned map = kBitPix | kBitMass | bit_gh(1) | bit_gh(2) | bit_gh(3) | bit_gh(4);
-    if (m.n_groups == 2 && mk[0] == kBitMass && mk[1] == kin1) return step_fn<T, WPS, GA, kBitMass, kin1, 0u, 0u>();
-    if (m.n_groups == 2 && mk[0] == kBitMass && mk[1] == kin2) return step_fn<T, WPS, GA, kBitMass, kin2, 0u, 0u>();
-    if (m.n_groups == 1 && mk[0] == map) return step_fn<T, WPS, GA, map, 0u, 0u, 0u>();
-    return step_fn<T, WPS, GA, kDyn, kDyn, kDyn, kDyn>();
+    switch (step_shape(m)) {
+    case kShapeKin1: return step_fn<T, WPS, GA, kBitMass, kKin1, 0u, 0u>();
+    case kShapeKin2: return step_fn<T, WPS, GA, kBitMass, kKin2, 0u, 0u>();
+    case kShapeMap: return step_fn<T, WPS, GA, kMapMask, 0u, 0u, 0u>();
+    default: return step_fn<T, WPS, GA, kDyn, kDyn, kDyn, kDyn>();
+    }
 }
 
 template <class T>
@@ -515,7 +511,7 @@ static m2m_status configure_kernels(m2m_ctx *ctx)
         m.win_group = best;
         // 1 KB per block is reserved by the runtime; 1 KB more covers the carve's alignment
         const long long per_block = std::min<long long>(smsm / rb, maxsm) - 2048 - (long long)smem_bytes<T>(m, 0, 0);
-        const long long slot_bytes = sizeof(T) == 8 ? 16 : 12;
+        const long long slot_bytes = 3 * sizeof(int);
         if (per_block > 0) m.win_n = int(std::min<long long>(m.g[best].n_ap, per_block / (slot_bytes * m.g[best].n_kinds)));
         m.win_lo = (m.g[best].n_ap - m.win_n) / 2;  // until the load places it
     }
@@ -570,7 +566,7 @@ static std::vector<ObsRow> plan_rows(const m2m_ctx *ctx)
         for (int p0 = 0; p0 < G.n_ap; p0 += 32)
             for (int k = 0; k < G.n_kinds; ++k)
                 for (int q = 0; q < 32; ++q) {
-                    ObsRow r{0.0, 0.0, 0.0, 0.0, 1.0, -1, 0};
+                    ObsRow r{0.0, 0.0, 0.0, 0.0, 1.0, 1.0, -1, 0};
                     if (p0 + q < G.n_ap) {
                         r.j = G.obs_off + k * G.n_ap + p0 + q;
                         r.iscale = ctx->obs_iscale.empty() ? 1.0 : ctx->obs_iscale[r.j];
@@ -578,6 +574,7 @@ static std::vector<ObsRow> plan_rows(const m2m_ctx *ctx)
                         r.cw = r.post / ctx->sig[r.j];
                         r.Y = ctx->Y[r.j];
                         r.sig = ctx->sig[r.j];
+                        r.isig = 1.0 / r.sig;
                     }
                     rows.push_back(r);
                 }
@@ -818,6 +815,7 @@ m2m_status create_impl(const m2m_potential *pot, const m2m_observables *obs,
     }
     if (s == M2M_OK) s = upload_tables(ctx);
     if (s == M2M_OK) s = smooth_setup(ctx);
+    if (s == M2M_OK) s = persist_setup(ctx);
     if (s != M2M_OK) {
         g_create_error = ctx->err;
         m2m_destroy(ctx);
@@ -850,13 +848,13 @@ Buffers buffers(m2m_ctx *c)
     return b;
 }
 
-static int grid_for(m2m_ctx *c)
+int grid_for(m2m_ctx *c, int bps)
 {
     // whole waves of one block per SM, up to the resident ones (the kernel shares the particles
     // out evenly over the blocks in whole warps); a fit of fewer warps than SMs takes a block per
     // warp. With ceil(n / block) blocks a 20,000-particle FP64 fit used 79 of the 152 SMs.
     const long long units = (c->n + 31) / 32, wave = (long long)c->nsm * c->block;
-    long long g = c->nsm * std::min<long long>(c->bps, (c->n + wave - 1) / wave);
+    long long g = c->nsm * std::min<long long>(bps, (c->n + wave - 1) / wave);
     if (units < g) g = units;
     // no block may process more than kMaxParticlesPerBlock particles (exact 32-bit sums)
     const long long floor_g = (c->n + kMaxParticlesPerBlock - 1) / kMaxParticlesPerBlock;
@@ -875,7 +873,7 @@ static void launch_finalize(m2m_ctx *c, int init)
 template <class T, int WPS>
 static void launch_step(m2m_ctx *c, int push, int init)
 {
-    step_kernel<T>(c)<<<grid_for(c), c->block, c->smem_step, c->stream>>>(c->m, make_cst<T>(c->m), state<T>(c),
+    step_kernel<T>(c)<<<grid_for(c, c->bps), c->block, c->smem_step, c->stream>>>(c->m, make_cst<T>(c->m), state<T>(c),
                                                                               buffers(c), push, init);
     if (c->m.fin_wide && !c->m.shard) launch_finalize<T, WPS>(c, init);
 }
@@ -981,6 +979,8 @@ static m2m_status finish_load(m2m_ctx *ctx, const double *dx, const double *dy, 
     const m2m_status rs = set_scales(ctx);
     if (rs != M2M_OK) return rs;
     CU(cudaMemsetAsync(ctx->d_hist, 0, sizeof(long long) * exchange_words(ctx), ctx->stream));
+    const m2m_status ps = persist_reset(ctx);
+    if (ps != M2M_OK) return ps;
     Scalars sc0{};
     sc0.Wrange = 9.2233720368547758e18 / m.fx_w;
     sc0.ups = ctx->scf_ups0;
@@ -1138,6 +1138,9 @@ extern "C" m2m_status m2m_step(m2m_ctx *ctx, int64_t nsteps)
         CU(cudaGetLastError());
         return M2M_OK;
     }
+    // two steps or more of a fit that can: one launch for many (a single step finalizes in its
+    // last block, without a meeting)
+    if (nsteps > 1 && persist_fits(ctx)) return persist_steps(ctx, nsteps);
     int64_t left = nsteps;
     if (left >= kGraphSteps && !ctx->graph) {
         m2m_status s = build_graph(ctx);
@@ -1159,6 +1162,7 @@ m2m_status check_device_errors(m2m_ctx *ctx)
     CU(cudaStreamSynchronize(ctx->stream));
     if (sc.err & kErrNegWeight) return fail(ctx, M2M_ERR_NEG_WEIGHT, "the force of change made a weight negative");
     if (sc.err & kErrOverflow) return fail(ctx, M2M_ERR_OVERFLOW, "a deposit left the fixed-point range");
+    if (sc.err & kErrTimeout) return fail(ctx, M2M_ERR_TIMEOUT, "a bounded device wait expired");
     if (sc.err & kErrNonFinite) return fail(ctx, M2M_ERR_NONFINITE, "a weight became non-finite");
     if (sc.err) return fail(ctx, M2M_ERR_CUDA, "device error word %u", sc.err);
     return M2M_OK;
@@ -1660,6 +1664,7 @@ extern "C" m2m_status m2m_load_state(m2m_ctx *ctx, const char *path)
     }
     CU(cudaMemcpy(ctx->d_sc, p, sizeof(Scalars), cudaMemcpyHostToDevice));
     CU(cudaMemset(ctx->d_hist, 0, sizeof(long long) * m.hist_words));
+    if ((s = persist_reset(ctx)) != M2M_OK) return s;
     k_head<<<1, 32, 0, ctx->stream>>>(m, ctx->d_sc, ctx->d_head);
     CU(cudaGetLastError());
     CU(cudaStreamSynchronize(ctx->stream));
@@ -1943,6 +1948,7 @@ void destroy_impl(m2m_ctx *ctx)
     free_dev(ctx->d_yraw); free_dev(ctx->d_delta); free_dev(ctx->d_prior_count);
     free_dev(ctx->d_hist); free_dev(ctx->d_acc); free_dev(ctx->d_sc); free_dev(ctx->d_pwin);
     smooth_free(ctx);
+    persist_free(ctx);
     if (ctx->own_stream && ctx->stream) cudaStreamDestroy(ctx->stream);
     delete ctx;
 }
@@ -2047,9 +2053,9 @@ __global__ void __launch_bounds__(256) k_static_observe(const Model m, const Cst
                                                         long long *hist, StaticStats *st, double *out)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    long long *h = reinterpret_cast<long long *>(smem);
+    unsigned *h = reinterpret_cast<unsigned *>(smem);
     __shared__ bool am_last;
-    for (int q = threadIdx.x; q < 2 * m.J; q += blockDim.x) h[q] = 0;
+    for (int q = threadIdx.x; q < 3 * m.J; q += blockDim.x) h[q] = 0;
     __syncthreads();
     const StaticTables tb{edges, nullptr, vp, isp, kExp2j};  // edges: squared
     unsigned err = 0;
@@ -2065,15 +2071,17 @@ __global__ void __launch_bounds__(256) k_static_observe(const Model m, const Cst
                 const double vv = vlos * vlos;
                 if (G.has_v2 && vv > k.v2max) err |= kErrOverflow;
                 group_kernels<kDyn>(G, tb, p, vlos, vv, wi, [&](int j, double v, int cls, int) {
-                    Acc<double>::add(h, m, j, v, cls == kClassMass ? m.fx_w : (cls == kClassVel ? m.fx_v2 : m.fx_gh));
+                    Acc<double>::add(h, j, v, cls == kClassMass ? m.fx_w : (cls == kClassVel ? m.fx_v2 : m.fx_gh));
                 });
             }
         });
     }
     if (err) atomicOr(&st->err, err);
     __syncthreads();
-    for (int q = threadIdx.x; q < 2 * m.J; q += blockDim.x)
-        if (h[q] != 0) atomicAdd(reinterpret_cast<unsigned long long *>(hist + q), static_cast<unsigned long long>(h[q]));
+    for (int q = threadIdx.x; q < 2 * m.J; q += blockDim.x) {
+        const long long v = Acc<double>::word(h, q >> 1, q & 1);
+        if (v != 0) red_add(hist + q, v);
+    }
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) am_last = atomicAdd(&st->done, 1u) == gridDim.x - 1;
@@ -2227,7 +2235,7 @@ extern "C" m2m_status m2m_observe_static(const m2m_observables *obs, int64_t n, 
     m.fx_w = pow2_floor(two62 / Wb);
     m.fx_v2 = pow2_floor(two62 / (Wb * (m.v2max > 1.0 ? m.v2max : 1.0)));
     m.fx_gh = pow2_floor(two62 / (Wb * 1.5));
-    const size_t smem = sizeof(long long) * 2 * size_t(J);
+    const size_t smem = sizeof(unsigned) * 3 * size_t(J);
     CS(cudaFuncSetAttribute(k_static_observe, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
     int occ = 0;
     CS(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_static_observe, 256, smem));

@@ -101,13 +101,12 @@ static void *batch_pick(const std::vector<m2m_ctx *> &sub, bool &bank)
         for (int g = 0; same && g < m0.n_groups; ++g)
             if (group_mask(c->m.g[g]) != mk[g]) same = false;
     }
-    constexpr unsigned kin1 = kBitV2 | bit_gh(4), kin2 = kBitV2 | bit_gh(3) | bit_gh(4);
-    constexpr unsigned map = kBitPix | kBitMass | bit_gh(1) | bit_gh(2) | bit_gh(3) | bit_gh(4);
-    if (same && m0.n_groups == 2 && mk[0] == kBitMass && mk[1] == kin1)
-        return batch_fn<T, WPS, kBitMass, kin1, 0u, 0u>(bank);
-    if (same && m0.n_groups == 2 && mk[0] == kBitMass && mk[1] == kin2)
-        return batch_fn<T, WPS, kBitMass, kin2, 0u, 0u>(bank);
-    if (same && m0.n_groups == 1 && mk[0] == map) return batch_fn<T, WPS, map, 0u, 0u, 0u>(bank);
+    switch (same ? step_shape(m0) : kShapeAny) {
+    case kShapeKin1: return batch_fn<T, WPS, kBitMass, kKin1, 0u, 0u>(bank);
+    case kShapeKin2: return batch_fn<T, WPS, kBitMass, kKin2, 0u, 0u>(bank);
+    case kShapeMap: return batch_fn<T, WPS, kMapMask, 0u, 0u, 0u>(bank);
+    default: break;
+    }
     return batch_fn<T, WPS, kDyn, kDyn, kDyn, kDyn>(bank);
 }
 

@@ -65,6 +65,13 @@ struct m2m_ctx {
     long long wout_cap = 0;
     bool loaded = false;
 
+    // several steps per launch (m2m_persist.cu); ksteps null: not for this fit
+    void *ksteps = nullptr;
+    size_t smem_steps = 0;
+    int steps_own = 0, steps_bps = 0;
+    long long *d_hist2 = nullptr;
+    void *d_meet = nullptr;
+
     cudaGraphExec_t graph = nullptr;
     int graph_steps = 0;
     std::string err;
@@ -129,6 +136,14 @@ m2m_status smooth_setup(m2m_ctx *ctx);
 void smooth_free(m2m_ctx *ctx);
 void smooth_launch(m2m_ctx *ctx);
 
+// several steps per launch (m2m_persist.cu)
+m2m_status persist_setup(m2m_ctx *ctx);
+bool persist_fits(m2m_ctx *ctx);
+m2m_status persist_reset(m2m_ctx *ctx);
+m2m_status persist_steps(m2m_ctx *ctx, int64_t nsteps);
+void persist_free(m2m_ctx *ctx);
+int grid_for(m2m_ctx *ctx, int bps);  // blocks of a step kernel at most bps of which share an SM
+
 // batch runtime (m2m_batch.cu)
 m2m_status batch_step(m2m_ctx *ctx, int64_t nsteps);
 m2m_status batch_synchronize(m2m_ctx *ctx);
@@ -188,4 +203,19 @@ inline unsigned group_mask(const m2m::GroupDesc &G)
     if (G.geometry == 1) mk |= m2m::kBitPix;
     if (G.geometry == 2) mk |= m2m::kBitShell;
     return mk;
+}
+
+// The compiled observable shapes: mass annuli and v2, h4 annuli; mass annuli and v2, h3, h4
+// annuli; one pixel group of mass, h1 .. h4; anything else.
+enum { kShapeAny = 0, kShapeKin1 = 1, kShapeKin2 = 2, kShapeMap = 3 };
+constexpr unsigned kKin1 = m2m::kBitV2 | m2m::bit_gh(4), kKin2 = kKin1 | m2m::bit_gh(3);
+constexpr unsigned kMapMask = m2m::kBitPix | m2m::kBitMass | m2m::bit_gh(1) | m2m::bit_gh(2) | m2m::bit_gh(3) | m2m::bit_gh(4);
+inline int step_shape(const m2m::Model &m)
+{
+    // the self-consistent potential is compiled into the generic kernel only
+    if (m.pot == 3 || m.n_groups > 2) return kShapeAny;
+    const unsigned m0 = group_mask(m.g[0]), m1 = m.n_groups > 1 ? group_mask(m.g[1]) : 0u;
+    if (m0 == m2m::kBitMass && m1 == kKin1) return kShapeKin1;
+    if (m0 == m2m::kBitMass && m1 == kKin2) return kShapeKin2;
+    return m0 == kMapMask && m1 == 0u ? kShapeMap : kShapeAny;
 }

@@ -26,7 +26,7 @@ constexpr int kKindV1 = 2;  // internal: first moment, used only to build target
 constexpr int kKindGH0 = 10;
 constexpr int kKindAlm0 = 100;  // a_lm on shells: kKindAlm0 + l (l + 1) + m
 
-enum : unsigned { kErrNonFinite = 1u, kErrNegWeight = 2u, kErrOverflow = 4u, kErrIndex = 8u };
+enum : unsigned { kErrNonFinite = 1u, kErrNegWeight = 2u, kErrOverflow = 4u, kErrIndex = 8u, kErrTimeout = 16u };
 
 struct GroupDesc {
     int geometry;   // 0 annuli, 1 pixels, 2 shells (3-D radial grid of the a_lm, eq. alm)
@@ -305,8 +305,8 @@ __host__ __device__ __forceinline__ bool keeps_accel(const Model &m)
 // sum_k coef_k c_(j0 + k stride) over the kinds of its group, with the factors laid out here
 // (see upload_plan), and only the elements that are ever non-zero are listed.
 struct ObsRow {
-    double iscale, post, cw, Y, sig;  // 1/fixed-point scale; factor of the raw sum; post / sig; data
-    int j, pad;                       // observable, -1 for the padding of a chunk
+    double iscale, post, cw, Y, sig, isig;  // 1/fixed-point scale; factor of the raw sum; post / sig; data
+    int j, pad;                             // observable, -1 for the padding of a chunk
 };
 struct RecElem {
     int dst, j0, stride, nk;  // element of the records; its terms
@@ -1449,28 +1449,36 @@ __device__ __forceinline__ void fx2(double v, double scale, long long &hi, long 
     }
 }
 
-// Mixed mode: round(v*scale) (the scaling by a power of two is exact) in one 64-bit
-// conversion, added to the block sums as three 32-bit limbs (see Acc<float>).
-__device__ __forceinline__ long long limbs_value(long long hi, long long mid, long long lo)
-{
-    return hi * 4294967296ll + mid * 65536ll + lo;
-}
-
-// Block-shared sums. FP64 mode: the two int64 words of each slot, added with
-// 64-bit shared atomics. Mixed mode: three int32 limbs per slot added with native
-// 32-bit shared atomics; at most kMaxParticlesPerBlock particles per block keep the
-// sums of mid and lo (each term in [0, 2^16)) below 2^31, and |sum of hi| < 2^31
-// follows from the fixed-point range. The block flush recombines the limbs into the
-// int64 word exactly.
+// Block-shared sums. Shared memory adds 32-bit integers natively, 64-bit ones only by a loop
+// around a compare-and-swap that runs once per lane of a warp that meets on a slot, so a sum is
+// kept in three 32-bit words.
+// FP64 mode: the words of a 96-bit integer, modulo 2^96. The low word is added first, the old
+// value it returns gives the carry, and so on up; the top word is added only where it and the
+// carry are not zero together (for small values of either sign: -x has it all ones and the carry
+// makes it 0), so a deposit is two shared atomics. (The 64-bit loops took a third of a small
+// fit's step: 20,000 particles 22.9 -> 20.5 us a step.)
+// Mixed mode: the fields of one 64-bit integer L = hi 2^32 + mid 2^16 + lo, mid, lo in [0, 2^16)
+// and hi signed, added without carries (three atomics that return nothing; two words with a
+// carry are 4 % slower at 2M particles, the returned value being waited for). At most
+// kMaxParticlesPerBlock particles per block keep the sums of mid and lo below 2^31, and |sum of
+// hi| < 2^31 follows from the fixed-point range.
 constexpr long long kMaxParticlesPerBlock = 32768;
+
+// Adds v and the carry c to *w; returns the carry out.
+__device__ __forceinline__ unsigned add_word(unsigned *w, unsigned v, unsigned c)
+{
+    const unsigned a = v + c;
+    const unsigned old = atomicAdd(w, a);
+    return (old + a < a || a < c) ? 1u : 0u;
+}
 
 template <class T>
 struct Acc;
 
 template <>
 struct Acc<double> {
-    static __host__ __device__ size_t bytes(const Model &m) { return sizeof(long long) * size_t(m.hist_words); }
-    // the fixed-point value of v * scale (two words)
+    static __host__ __device__ size_t bytes(const Model &m) { return sizeof(int) * (3 * size_t(m.nslots) + size_t(m.ncell)); }
+    // the fixed-point value of v * scale: hi + lo 2^-32
     struct Fx {
         long long hi, lo;
     };
@@ -1482,33 +1490,30 @@ struct Acc<double> {
     }
     __device__ static void put(void *base, int slot, const Fx &q)
     {
-        long long *h = static_cast<long long *>(base);
-        atomicAdd(reinterpret_cast<unsigned long long *>(h + 2 * slot), static_cast<unsigned long long>(q.hi));
-        if (q.lo) atomicAdd(reinterpret_cast<unsigned long long *>(h + 2 * slot + 1), static_cast<unsigned long long>(q.lo));
+        unsigned *h = static_cast<unsigned *>(base) + 3 * slot;
+        unsigned c = add_word(h, unsigned(q.lo), 0u);
+        c = add_word(h + 1, unsigned(q.hi), c);
+        const unsigned top = unsigned(static_cast<unsigned long long>(q.hi) >> 32) + c;
+        if (top) atomicAdd(h + 2, top);
     }
-    __device__ static void add(void *base, const Model &, int slot, double v, double scale)
+    __device__ static void add(void *base, int slot, double v, double scale)
     {
         if (is_zero(v)) return;
         put(base, slot, fx(v, scale));
     }
-    __device__ static void count(void *base, const Model &m, int c)
+    // word wd (0: integer part, 1: fraction) of a slot of the block's sums
+    __device__ static long long word(const void *base, int slot, int wd)
     {
-        atomicAdd(reinterpret_cast<unsigned long long *>(static_cast<long long *>(base) + m.off_count + c), 1ull);
+        const unsigned *h = static_cast<const unsigned *>(base) + 3 * slot;
+        if (wd == 1) return static_cast<long long>(h[0]);
+        return static_cast<long long>((static_cast<unsigned long long>(h[2]) << 32) | h[1]);
     }
-    // global word k of the block's sums
-    __device__ static long long word(const void *base, const Model &, int k) { return static_cast<const long long *>(base)[k]; }
 };
 
 template <>
 struct Acc<float> {
-    static __host__ __device__ size_t bytes(const Model &m)
-    {
-        return sizeof(int) * (3 * size_t(m.nslots) + size_t(m.ncell)) + 8;
-    }
-    // round(v*scale) as L = hi 2^32 + mid 2^16 + lo with mid, lo in [0, 2^16) and hi signed:
-    // the two's-complement fields of one 64-bit conversion. Per block the lo and mid sums
-    // stay below 32768 * 65535 < 2^31, and the hi sum within the fixed-point range.
-    // the fixed-point value of v * scale (one 64-bit integer)
+    static __host__ __device__ size_t bytes(const Model &m) { return sizeof(int) * (3 * size_t(m.nslots) + size_t(m.ncell)); }
+    // the fixed-point value of v * scale: one 64-bit integer, rounded to nearest
     struct Fx {
         long long L;
     };
@@ -1522,22 +1527,20 @@ struct Acc<float> {
         atomicAdd(h + 2, static_cast<int>(q.L & 0xFFFF));
     }
     // a zero adds zeros: cheaper than the branch around it
-    __device__ static void add(void *base, const Model &, int slot, float v, float scale)
+    __device__ static void add(void *base, int slot, float v, float scale) { put(base, slot, fx(v, scale)); }
+    __device__ static long long word(const void *base, int slot, int)
     {
-        put(base, slot, fx(v, scale));
-    }
-    __device__ static void count(void *base, const Model &m, int c)
-    {
-        atomicAdd(static_cast<int *>(base) + 3 * m.nslots + c, 1);
-    }
-    __device__ static long long word(const void *base, const Model &m, int k)
-    {
-        const int *h = static_cast<const int *>(base);
-        if (k >= m.off_count) return static_cast<long long>(h[3 * m.nslots + (k - m.off_count)]);
-        const int *q = h + 3 * k;
-        return limbs_value(q[0], q[1], q[2]);
+        const int *q = static_cast<const int *>(base) + 3 * slot;
+        return q[0] * 4294967296ll + q[1] * 65536ll + q[2];
     }
 };
+
+// Particle counts of the cells, behind the sums.
+template <class T>
+__device__ __forceinline__ unsigned *acc_counts(void *base, const Model &m)
+{
+    return static_cast<unsigned *>(base) + 3 * m.nslots;
+}
 
 // Per-thread running total of the deposited weight, in the same fixed point.
 template <class T>
@@ -1561,7 +1564,8 @@ struct Total<double> {
         top += q.hi >> 20;
     }
     // the deposited weight for the range check (an FP64 sum would take the FP64 pipe)
-    __device__ double range_sum(double, double scale) const { return double(top) * 1048576.0 / scale; }
+    __device__ long long range_sum(double) const { return top; }
+    __device__ static double range_value(long long v, double scale) { return double(v) * (1048576.0 * (1.0 / scale)); }
     __device__ long long word(int q, double) const { return q == 0 ? hi : lo; }
 };
 
@@ -1573,7 +1577,8 @@ struct Total<float> {
     long long s = 0;
     __device__ void add(float v, float scale) { s += __float2ll_rn(v * scale); }
     __device__ void add_fx(const Acc<float>::Fx &q) { s += q.L; }
-    __device__ float range_sum(float wdep, float) const { return wdep; }
+    __device__ float range_sum(float wdep) const { return wdep; }
+    __device__ static double range_value(float v, float) { return double(v); }
     __device__ long long word(int, float) const { return s; }
 };
 
@@ -1699,7 +1704,7 @@ template <class T>
 __host__ __device__ inline size_t window_bytes(const Model &m)
 {
     const size_t slots = m.win_n > 0 ? size_t(m.g[m.win_group].n_kinds) * m.win_n : 0;
-    return slots * (sizeof(T) == 8 ? 2 * sizeof(long long) : 3 * sizeof(int));
+    return slots * 3 * sizeof(int);
 }
 
 // hist: 0 no block sums, 1 all (Acc<T>), 2 the aperture window of the global deposit
@@ -1742,15 +1747,20 @@ __device__ __forceinline__ Smem<T> carve(const Model &m, const Buffers &b, unsig
     return s;
 }
 
-// Starts the copy of a fit's tables into shared memory (asynchronous 16-byte copies; the
-// caller waits with tables_wait and then synchronises the block).
+// Starts the copy of bytes [lo, hi) (multiples of 16) of a fit's tables into shared memory
+// (asynchronous 16-byte copies; the caller waits with tables_wait and then synchronises the block).
+template <class T>
+__device__ __forceinline__ void tables_range(const Buffers &b, const Smem<T> &s, int lo, int hi)
+{
+    const unsigned dst = static_cast<unsigned>(__cvta_generic_to_shared(s.tab)) + unsigned(lo - s.tab_lo);
+    const unsigned char *src = b.tab + lo;
+    for (int q = 16 * int(threadIdx.x); q < hi - lo; q += 16 * int(blockDim.x))
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + q), "l"(src + q) : "memory");
+}
 template <class T>
 __device__ __forceinline__ void tables_start(const Buffers &b, const Smem<T> &s)
 {
-    const unsigned dst = static_cast<unsigned>(__cvta_generic_to_shared(s.tab));
-    const unsigned char *src = b.tab + s.tab_lo;
-    for (int q = 16 * int(threadIdx.x); q < s.tab_hi - s.tab_lo; q += 16 * int(blockDim.x))
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + q), "l"(src + q) : "memory");
+    tables_range<T>(b, s, s.tab_lo, s.tab_hi);
 }
 __device__ __forceinline__ void tables_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
@@ -1869,11 +1879,11 @@ __device__ __forceinline__ void write_prior(const Buffers &b, int c, double pr)
 }
 
 template <int WPS>
-__device__ void window_priors(const Model &m, const Buffers &b, double s_ren)
+__device__ void window_priors(const Model &m, const Buffers &b, long long *hist, double s_ren)
 {
     constexpr int NQ = WPS + 1;
     const int nE = m.nE, nx = m.nx, nc = m.ncell, hE = m.pwin_E, hx = m.pwin_x;
-    unsigned long long *H = reinterpret_cast<unsigned long long *>(b.hist);
+    unsigned long long *H = reinterpret_cast<unsigned long long *>(hist);
     unsigned long long *cum = b.pwin;
     auto at = [&](int q, int c) -> unsigned long long * {
         return q == 0 ? H + m.off_count + c : H + WPS * (m.J + 1 + c) + (q - 1);
@@ -1946,47 +1956,72 @@ static __global__ void k_head(const Model m, const Scalars *sc, StepHead *head)
     *head = h;
 }
 
-// The scale that renormalises the weights of this step, and their total U (stored units).
+// The total weight of a step (stored units) from its fixed-point sum.
 template <int WPS>
-__device__ __forceinline__ double renorm_scale(const Model &m, const Buffers &b, int init, double W0, double &U)
+__device__ __forceinline__ double total_weight(const Model &m, const long long *hist)
 {
-    U = fx_read<WPS>(b.hist, m.J) * (1.0 / m.fx_w);  // fx_w is a power of two: exact
-    return (!init && m.renormalize && U > 0.0) ? W0 / U : 1.0;
+    return fx_read<WPS>(hist, m.J) * (1.0 / m.fx_w);  // fx_w is a power of two: exact
+}
+
+// The scale W0/U that renormalises the weights of this step, in integers: every thread forms it,
+// and as FP64 instructions its division would queue for the narrow pipe.
+template <int WPS>
+__device__ __forceinline__ double renorm_scale(const Model &m, const long long *hist, int init, double W0)
+{
+    const long long hi = __ldcg(hist + WPS * m.J), lo = WPS == 2 ? __ldcg(hist + WPS * m.J + 1) : 0;
+    if (init || !m.renormalize) return 1.0;
+    const long long t = hi + (lo >> 32);
+    if (t > 0 && big_range(W0) && big_range(m.fx_w)) {
+        const int z = __clzll(t);
+        const u64 f = u64(lo) << 32;  // the fraction below t
+        const Big U{(u64(t) << z) | (z ? f >> (64 - z) : 0), 63 - z - big_of(m.fx_w).e};
+        return big_double(big_norm(big_mul_raw(big_rcp(U), big_of(W0))));
+    }
+    const double U = total_weight<WPS>(m, hist);
+    return U > 0.0 ? W0 / U : 1.0;
 }
 
 // The observables of chunks [ch0, ch1) from the fixed-point sums: smoothing (eq. myts),
 // Delta_j (eq. delta), coefficients c_j into b.c and cs (if given, J doubles of shared memory);
 // csum[chunk]: the chunk's sum of Delta_j^2. A warp per chunk. What does not depend on the
-// sums is loaded before them.
+// sums is loaded before them. ys: the block's own copy of ytil in shared memory, or null
+// (Buffers::ytil); store: whether this block writes the fit's arrays.
 template <int WPS>
-__device__ __forceinline__ void fin_observables(const Model &m, const Buffers &b, const FinPlan &pl, int ch0, int ch1,
-                                                int init, double W0, double *cs, double *csum, double &s_ren, double &U)
+__device__ __forceinline__ void fin_observables(const Model &m, const Buffers &b, const long long *hist, int ch0, int ch1,
+                                                int init, double W0, double *cs, double *csum, double &s_ren,
+                                                double *ys = nullptr, bool store = true)
 {
+    const FinPlan &pl = b.plan;
     const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     ObsRow r;
     double h = 0.0, old = 0.0;
     auto fetch = [&](int ch) {
         r = pl.rows[32 * ch + lane];
         if (r.j >= 0) {
-            h = fx_read<WPS>(b.hist, r.j);
-            old = b.ytil[r.j];
+            h = fx_read<WPS>(hist, r.j);
+            old = ys ? ys[r.j] : b.ytil[r.j];
         }
     };
     int ch = ch0 + int(threadIdx.x >> 5);
     if (ch < ch1) fetch(ch);
-    s_ren = renorm_scale<WPS>(m, b, init, W0, U);
+    s_ren = renorm_scale<WPS>(m, hist, init, W0);
     for (; ch < ch1; ch += nw) {
         double d = 0.0;
         if (r.j >= 0) {
             const double raw = h * r.iscale * s_ren * r.post;
             const double yt = init ? raw : old + m.alpha * (raw - old);
-            d = (yt - r.Y) / r.sig;
+            const double a = yt - r.Y;  // a / sig: the product with 1/sig and its exact residual
+            const double q = a * r.isig;
+            d = fma(fma(-q, r.sig, a), r.isig, q);
             const double cj = d * r.cw;
-            b.yraw[r.j] = raw;
-            b.ytil[r.j] = yt;
-            b.delta[r.j] = d;
-            b.c[r.j] = cj;
+            if (ys) ys[r.j] = yt;
             if (cs) cs[r.j] = cj;
+            if (store) {
+                b.yraw[r.j] = raw;
+                b.ytil[r.j] = yt;
+                b.delta[r.j] = d;
+                b.c[r.j] = cj;
+            }
         }
         double d2 = d * d;
         if (ch + nw < ch1) fetch(ch + nw);
@@ -1995,23 +2030,32 @@ __device__ __forceinline__ void fin_observables(const Model &m, const Buffers &b
     }
 }
 
-// The record elements [e0, e1) from the coefficients c.
-__device__ __forceinline__ void fin_records(const Buffers &b, const FinPlan &pl, int e0, int e1, const double *c)
+// The record elements [e0, e1) from the coefficients c; rs: also into the block's records in
+// shared memory, if given.
+template <class T = double>
+__device__ __forceinline__ void fin_records(const Buffers &b, int e0, int e1, const double *c, T *rs = nullptr,
+                                            bool store = true)
 {
+    const FinPlan &pl = b.plan;
     for (int e = e0 + int(threadIdx.x); e < e1; e += blockDim.x) {
         const RecElem el = pl.elems[e];
         double v = 0.0;
         for (int k = 0; k < el.nk; ++k) v += pl.coef[size_t(k) * pl.n_elems + e] * c[el.j0 + k * el.stride];
-        b.rec[el.dst] = v;
-        if (b.recf) b.recf[el.dst] = float(v);
+        if (rs) rs[el.dst] = T(v);
+        if (store) {
+            b.rec[el.dst] = v;
+            if (b.recf) b.recf[el.dst] = float(v);
+        }
     }
 }
 
-// chi^2 from the chunk sums, in chunk order over 32 lanes (one warp).
+// chi^2 from the chunk sums, in chunk order over 32 lanes (one warp). L2: the sums are in
+// global memory, from several blocks.
+template <bool L2>
 __device__ __forceinline__ double fin_chi2(const double *csum, int n)
 {
     double v = 0.0;
-    for (int q = int(threadIdx.x & 31); q < n; q += 32) v += csum[q];
+    for (int q = int(threadIdx.x & 31); q < n; q += 32) v += L2 ? __ldcg(csum + q) : csum[q];
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
@@ -2042,18 +2086,20 @@ __device__ __forceinline__ void fin_scalars(const Model &m, const Buffers &b, lo
     *b.head = h;
 }
 
-// Update steps: the cell means (Sec. 2.3.1) or window means from the cells' sums.
+// Update steps: the cell means (Sec. 2.3.1) or window means from the cells' sums, by block
+// `blk` of `blks` (the windows by the first).
 template <int WPS>
-__device__ __forceinline__ void fin_priors(const Model &m, const Buffers &b, double s_ren)
+__device__ __forceinline__ void fin_priors(const Model &m, const Buffers &b, long long *hist, double s_ren, int blk = 0,
+                                           int blks = 1)
 {
     if (m.pwin_E > 0 || m.pwin_x > 0) {
-        window_priors<WPS>(m, b, s_ren);
+        if (blk == 0) window_priors<WPS>(m, b, hist, s_ren);
         return;
     }
     const double ifx = 1.0 / m.fx_w;
-    for (int q = threadIdx.x; q < m.ncell; q += blockDim.x) {
-        const long long cnt = __ldcg(b.hist + m.off_count + q);
-        const double sum = fx_read<WPS>(b.hist, m.J + 1 + q) * ifx * s_ren;
+    for (int q = blk * blockDim.x + threadIdx.x; q < m.ncell; q += blks * blockDim.x) {
+        const long long cnt = __ldcg(hist + m.off_count + q);
+        const double sum = fx_read<WPS>(hist, m.J + 1 + q) * ifx * s_ren;
         const double pr = cnt > 0 ? sum / double(cnt) : 0.0;  // mean weight of the cell
         b.prior_count[q] = cnt;
         if (m.smooth) b.prior_raw[q] = pr;  // the smoothing kernels turn the raw means into the priors
@@ -2075,20 +2121,21 @@ __device__ void finalize_block(const Model &m, const Buffers &b, long long n, in
     const FinPlan &pl = b.plan;
     const double W0 = init ? 0.0 : __ldcg(&b.sc->W0);
     double *csum = cs + m.J;
-    double s_ren, U;
-    fin_observables<WPS>(m, b, pl, 0, pl.n_chunks, init, W0, cs, csum, s_ren, U);
+    double s_ren;
+    fin_observables<WPS>(m, b, b.hist, 0, pl.n_chunks, init, W0, cs, csum, s_ren);
     __syncthreads();
-    if (int(threadIdx.x) == int(blockDim.x) - 32) fin_scalars(m, b, n, init, prior_step, s_ren, U);
+    if (int(threadIdx.x) == int(blockDim.x) - 32)
+        fin_scalars(m, b, n, init, prior_step, s_ren, total_weight<WPS>(m, b.hist));
     if (threadIdx.x < 32) {
-        const double chi2 = fin_chi2(csum, pl.n_chunks);
+        const double chi2 = fin_chi2<false>(csum, pl.n_chunks);
         if (threadIdx.x == 0) b.sc->chi2 = chi2;
     }
-    fin_records(b, pl, 0, pl.n_elems, cs);
+    fin_records(b, 0, pl.n_elems, cs);
     if (scf_step) {
         __syncthreads();
         scf_finalize<WPS>(m, b, s_ren, init, cs);
     }
-    if (prior_step) fin_priors<WPS>(m, b, s_ren);
+    if (prior_step) fin_priors<WPS>(m, b, b.hist, s_ren);
     __syncthreads();
     const int words = (prior_step || scf_step) ? m.hist_words : m.off_grid;
     for (int q = threadIdx.x; q < words; q += blockDim.x) b.hist[q] = 0;
@@ -2211,7 +2258,7 @@ __device__ __forceinline__ void step_particles(const Model &m, const Model &mh, 
     const T *rec = GA ? global_records<T>(b) : S.c;
     auto deposit = [&](int slot, T v, T scale) {
         if constexpr (GA) global_add(b.hist, slot, v, scale);
-        else Acc<T>::add(S.h, mh, slot, v, scale);
+        else Acc<T>::add(S.h, slot, v, scale);
     };
     // the next particle's state is loaded while the current one is processed
     const bool need_cell = f.pending && mh.mode == 1;
@@ -2285,7 +2332,7 @@ __device__ __forceinline__ void step_particles(const Model &m, const Model &mh, 
                 if (GP<M>::shells(G)) {  // never cached; never in the global-deposit kernel
                     shell_kernels(G, tb, x, y, z, w, [&](int j, T v, int, int) {
                         if constexpr (GA) global_add(b.hist, j, v, k.fx_gh);
-                        else Acc<T>::add(S.h, mh, j, v, k.fx_gh);
+                        else Acc<T>::add(S.h, j, v, k.fx_gh);
                     });
                     return;
                 }
@@ -2302,13 +2349,13 @@ __device__ __forceinline__ void step_particles(const Model &m, const Model &mh, 
                             if constexpr (GA) {
                                 const unsigned a = unsigned(p - mh.win_lo);
                                 if (g == mh.win_group && a < unsigned(mh.win_n))
-                                    Acc<T>::add(S.h, mh, kk * mh.win_n + int(a), v, scale);
+                                    Acc<T>::add(S.h, kk * mh.win_n + int(a), v, scale);
                                 else
                                     global_add(b.hist, j, v, scale);
                             } else if (cls == kClassMass) {  // v is w (the kernel is 1)
                                 Acc<T>::put(S.h, j, wfx);
                             } else {
-                                Acc<T>::add(S.h, mh, j, v, scale);
+                                Acc<T>::add(S.h, j, v, scale);
                             }
                         },
                         gxc && g == mh.gx_group ? &gout : nullptr);
@@ -2333,7 +2380,7 @@ __device__ __forceinline__ void step_particles(const Model &m, const Model &mh, 
             const int c = prior_cell<T, kScf>(m, k, b.lcE, x, y, z, vx, vy, vz);
             deposit(m.J + 1 + c, w, k.fx_w);
             if constexpr (GA) red_add(b.hist + m.off_count + c, 1);
-            else Acc<T>::count(S.h, m, c);
+            else atomicAdd(acc_counts<T>(S.h, m) + c, 1u);
             P.cell[i] = static_cast<uint16_t>(c);
         }
         P.x[i] = x; P.y[i] = y; P.z[i] = z;
@@ -2345,22 +2392,23 @@ __device__ __forceinline__ void step_particles(const Model &m, const Model &mh, 
 // Adds the block's sums, its total weight and its error bits to the fit's global
 // sums and scalars. Called by every thread of the block.
 template <class T, int WPS, bool GA>
-__device__ __forceinline__ void block_flush(const Model &m, const Cst<T> &k, const Buffers &b, const Smem<T> &S,
-                                            int prior_step, unsigned err, const Total<T> &wtot, T wdep,
-                                            int scf_step = 0)
+__device__ __forceinline__ void block_flush(const Model &m, const Cst<T> &k, Scalars *sc, long long *hist, double *wcheck,
+                                            const Smem<T> &S, int prior_step, unsigned err, const Total<T> &wtot, T wdep,
+                                            int scf_step)
 {
-    if (err) atomicOr(&b.sc->err, err);
+    if (err) atomicOr(&sc->err, err);
     // the total weight went into registers: one global atomic per warp and word
 #pragma unroll
     for (int q = 0; q < WPS; ++q) {
         long long v = wtot.word(q, k.fx_w);
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         if ((threadIdx.x & 31) == 0 && v != 0)
-            red_add(b.hist + WPS * m.J + q, v);
+            red_add(hist + WPS * m.J + q, v);
     }
-    wdep = wtot.range_sum(wdep, k.fx_w);
-    for (int o = 16; o > 0; o >>= 1) wdep += __shfl_xor_sync(0xffffffffu, wdep, o);
-    if ((threadIdx.x & 31) == 0 && wdep != T(0)) atomicAdd(&b.sc->Wcheck, double(wdep));
+    auto chk = wtot.range_sum(wdep);
+    for (int o = 16; o > 0; o >>= 1) chk += __shfl_xor_sync(0xffffffffu, chk, o);
+    if ((threadIdx.x & 31) == 0 && chk != 0)
+        atomicAdd(wcheck, Total<T>::range_value(chk, k.fx_w));
     __syncthreads();
     if (GA) {  // the aperture window's sums go to their observables' global words
         const GroupDesc &G = m.g[m.win_group < 0 ? 0 : m.win_group];
@@ -2368,16 +2416,23 @@ __device__ __forceinline__ void block_flush(const Model &m, const Cst<T> &k, con
         for (int q = threadIdx.x; q < WPS * slots; q += blockDim.x) {
             const int slot = q / WPS, wd = q - slot * WPS;
             const int kk = slot / m.win_n, a = slot - kk * m.win_n;
-            const long long v = Acc<T>::word(S.h, m, q);
+            const long long v = Acc<T>::word(S.h, slot, wd);
             const int j = G.obs_off + kk * G.n_ap + m.win_lo + a;
-            if (v != 0) red_add(b.hist + WPS * j + wd, v);
+            if (v != 0) red_add(hist + WPS * j + wd, v);
         }
     }
-    const int words = GA ? 0 : ((prior_step || scf_step) ? m.hist_words : m.off_grid);
+    const bool all = prior_step || scf_step;
+    const int words = GA ? 0 : WPS * (all ? m.nslots : m.J);
     for (int q = threadIdx.x; q < words; q += blockDim.x) {
-        if (q >= WPS * m.J && q < WPS * (m.J + 1)) continue;  // the total is already global
-        const long long v = Acc<T>::word(S.h, m, q);
-        if (v != 0) red_add(b.hist + q, v);
+        const int slot = q / WPS;
+        if (slot == m.J) continue;  // the total is already global
+        const long long v = Acc<T>::word(S.h, slot, q - slot * WPS);
+        if (v != 0) red_add(hist + q, v);
+    }
+    if (!GA && all) {
+        const unsigned *cnt = acc_counts<T>(S.h, m);
+        for (int q = threadIdx.x; q < m.ncell; q += blockDim.x)
+            if (cnt[q]) red_add(hist + m.off_count + q, static_cast<long long>(cnt[q]));
     }
     __syncthreads();
 }
@@ -2425,7 +2480,7 @@ __global__ void __launch_bounds__(kStepMaxThreads<T, GA>, (GA && sizeof(T) == 4)
     Total<T> wtot;
     T wdep = T(0);  // floating-point twin of wtot, for the fixed-point range check
     step_particles<T, GA, M0, M1, M2, M3>(m, m, k, P, b, S, f, push, lo + threadIdx.x, hi, blockDim.x, err, wtot, wdep);
-    block_flush<T, WPS, GA>(m, k, b, S, f.prior_step, err, wtot, wdep, f.scf_step);
+    block_flush<T, WPS, GA>(m, k, b.sc, b.hist, &b.sc->Wcheck, S, f.prior_step, err, wtot, wdep, f.scf_step);
     if (GA || m.fin_wide || m.shard) return;  // k_finalize follows (a shard's after the exchange of its sums)
     // last block to finish runs the finalize
     if (block_is_last(&b.sc->blocks_done, gridDim.x, &am_last))
@@ -2467,27 +2522,27 @@ __global__ void __launch_bounds__(256) k_finalize(const Model m, const Buffers b
     const StepFlags<T> f = step_flags<T>(m, b.head, init);
     const double W0 = init ? 0.0 : __ldcg(&b.sc->W0);
     const int2 r0 = pl.range[blockIdx.x], r1 = pl.range[blockIdx.x + 1];
-    double s_ren, U;
-    fin_observables<WPS>(m, b, pl, r0.x, r1.x, init, W0, nullptr, pl.csum, s_ren, U);
+    double s_ren;
+    fin_observables<WPS>(m, b, b.hist, r0.x, r1.x, init, W0, nullptr, pl.csum, s_ren);
     __syncthreads();
-    fin_records(b, pl, r0.y, r1.y, b.c);
+    fin_records(b, r0.y, r1.y, b.c);
     if (!block_is_last(&b.sc->blocks_done, gridDim.x, &am_last)) return;
     if (threadIdx.x < 32) {
-        const double chi2 = fin_chi2(pl.csum, pl.n_chunks);
+        const double chi2 = fin_chi2<true>(pl.csum, pl.n_chunks);
         if (threadIdx.x == 0) {
             b.sc->chi2 = chi2;
             if (m.shard) {
                 b.sc->Wcheck = double(b.hist[m.hist_words]) * (b.sc->Wrange * kRangeUnit);
                 b.hist[m.hist_words] = 0;
             }
-            fin_scalars(m, b, n, init, f.prior_step, s_ren, U);
+            fin_scalars(m, b, n, init, f.prior_step, s_ren, total_weight<WPS>(m, b.hist));
         }
     }
     if (f.scf_step) {
         __syncthreads();
         scf_finalize<WPS>(m, b, s_ren, init, red);
     }
-    if (f.prior_step) fin_priors<WPS>(m, b, s_ren);
+    if (f.prior_step) fin_priors<WPS>(m, b, b.hist, s_ren);
     __syncthreads();
     const int words = (f.prior_step || f.scf_step) ? m.hist_words : m.off_grid;
     for (int q = threadIdx.x; q < words; q += blockDim.x) b.hist[q] = 0;
@@ -2588,7 +2643,7 @@ __global__ void __launch_bounds__(256, MINB) k_step_batch(const BatchArgs<T> a, 
         else
             step_particles<T, false, M0, M1, M2, M3>(m, m, k, P, b, S, f, 1, sg.begin + threadIdx.x, sg.end,
                                                      blockDim.x, err, wtot, wdep);
-        block_flush<T, WPS, false>(m, k, b, S, f.prior_step, err, wtot, wdep, f.scf_step);
+        block_flush<T, WPS, false>(m, k, b.sc, b.hist, &b.sc->Wcheck, S, f.prior_step, err, wtot, wdep, f.scf_step);
         if (block_is_last(&b.sc->blocks_done, a.nseg[cur], &am_last)) {
             finalize_block<WPS>(m, b, P.n, 0, f.prior_step, reinterpret_cast<double *>(smem), f.scf_step);
             cur = -1;  // the finalize used the shared memory: reload before the next segment

@@ -54,3 +54,65 @@ def test_chunks_of_the_finalize(n_ap):
     wl.groups = [Group("annuli", ["mass"], [0.05], edges=_edges(n_ap)), wl.groups[1]]
     wl.params = dict(wl.params, eps=1e-6)
     _check(wl, O.from_workload(wl))
+
+
+def _same(a, b):
+    for u, v in zip(a, b):
+        assert np.array_equal(u, v)
+
+
+def _read(f):
+    yt, y = f.observables()
+    pos, vel = f.state()
+    g, cnt, cells = f.priors()
+    return yt, y, f.weights(), pos, vel, g, cnt, cells, np.array([f.chi2(), f.step_count()])
+
+
+CASES = {
+    "c1": dict(wl="c1", n=3001),
+    "c1_mixed": dict(wl="c1", n=40_001, precision="mixed"),
+    "window": dict(wl="c2", n=20_000, prior=dict(nE=90, nx=30, window=(1, 1), update_every=7), precision="mixed"),
+    "every_step": dict(wl="c2", n=5000, prior=dict(update_every=1)),
+    "gwr_euler_relax": dict(wl="c1", n=700, prior=dict(mode="gwr"), params=dict(update_rule="euler", n_relax=9, eps=1e-5)),
+    "nfw": dict(wl="c3", n=2500, precision="fp64", params=dict(eps=1e-5)),
+    "one": dict(wl="c1", n=1, params=dict(eps=1e-6)),
+    "wide_block": dict(wl="c1", n=9000, kw=dict(block=64, blocks_per_sm=1)),
+}
+
+
+def _fit(case, targets):
+    from paper_1202_2355_gb300 import binding as B
+    wl = W.make(case["wl"], n=case["n"], n_target=100_000)
+    obs, Y, sig = targets(case["wl"])
+    f = B.fit_from_workload(wl, Y, sig, obs.Vp, obs.sp, precision=case.get("precision", "fp64"),
+                            prior=dict(wl.prior, **dict(dict(update_every=5), **case.get("prior", {}))),
+                            params=dict(wl.params, **dict(dict(eps=1e-4), **case.get("params", {}))), **case.get("kw", {}))
+    f.load(wl.model)
+    return f
+
+
+@pytest.fixture(scope="module")
+def targets():
+    made = {}
+
+    def get(name):
+        if name not in made:
+            made[name] = O.from_workload(W.make(name, n=16, n_target=100_000))
+        return made[name]
+    return get
+
+
+@pytest.mark.parametrize("name", sorted(CASES))
+def test_many_steps_per_launch_are_the_same_steps(name, targets):
+    """step(k) runs k steps in one launch, step(1) a launch and a finalize per step: the same
+    bits, in any mixture, and with two fits taking turns on their own streams."""
+    one, many, other = (_fit(CASES[name], targets) for _ in range(3))
+    for _ in range(83):
+        one.step(1)
+    for k in (2, 1, 70, 10):
+        many.step(k)
+        other.step(k)
+    _same(_read(one), _read(many))
+    _same(_read(one), _read(other))
+    for f in (one, many, other):
+        f.close()
