@@ -187,6 +187,15 @@ __host__ __device__ __forceinline__ Big big_add(const Big &a, const Big &b)
 // that of the product if its top bit is set (see big_norm).
 __host__ __device__ __forceinline__ Big big_mul_raw(const Big &a, const Big &b) { return Big{mulhi_u(a.m, b.m), a.e + b.e + 1}; }
 
+__host__ __device__ __forceinline__ int big_clz(u64 v)
+{
+#ifdef __CUDA_ARCH__
+    return __clzll(i64(v));
+#else
+    return __builtin_clzll(v);
+#endif
+}
+
 // Up to three leading zeros shifted out.
 __host__ __device__ __forceinline__ Big big_norm(Big a)
 {
@@ -305,17 +314,18 @@ __host__ __device__ __forceinline__ i64 ln_frac(u64 m, const u64 *t)
     return i64(t[2 * j + 1]) + z + (mulhi_s(z2, g) >> 9);
 }
 
-// G M_s mu(r/r_s) / r^3 of the NFW halo, mu(q) = ln(1+q) - q/(1+q). With t = r/(r + r_s) = q/(1+q)
-// and u = 1 - t = r_s/(r + r_s): mu = -ln u - t, both terms in fixed point (2^-62 while u > 1/2,
-// 2^-56 beyond); below t = 2^-7, where they cancel, the series t^2 (1/2 + t/3 + t^2/4 + ..).
-__host__ __device__ __forceinline__ Big nfw_big(double gms, double rs, const Big &r, const Big &ir, const u64 *t)
+// The NFW terms at q = r/r_s: mu = ln(1+q) - q/(1+q) and, if l1 is not null, ln(1+q). With
+// t = r/(r + r_s) = q/(1+q) and u = 1 - t = r_s/(r + r_s): mu = -ln u - t, both terms in fixed point
+// (2^-62 while u > 1/2, 2^-56 beyond); below t = 2^-7, where they cancel, the series
+// t^2 (1/2 + t/3 + t^2/4 + ..). ln(1+q) = mu + t.
+__host__ __device__ __forceinline__ Big nfw_mu_big(double rs, const Big &r, const u64 *tab, Big *l1 = nullptr)
 {
     const Big B = big_of(rs);
     const Big w = big_rcp(big_add(r, B));
-    const Big q = big_norm(big_mul_raw(r, w)), u = big_norm(big_mul_raw(B, w));
+    const Big t = big_norm(big_mul_raw(r, w)), u = big_norm(big_mul_raw(B, w));
     Big mu;
-    if (q.e < -7) {
-        const double x = big_double(q);
+    if (t.e < -7) {
+        const double x = big_double(t);
         double s = 1.0 / 9.0;
         s = fma(x, s, 1.0 / 8.0);
         s = fma(x, s, 1.0 / 7.0);
@@ -324,26 +334,68 @@ __host__ __device__ __forceinline__ Big nfw_big(double gms, double rs, const Big
         s = fma(x, s, 1.0 / 4.0);
         s = fma(x, s, 1.0 / 3.0);
         s = fma(x, s, 0.5);
-        mu = big_norm(big_mul_raw(big_mul_raw(q, q), big_of(s)));
+        mu = big_norm(big_mul_raw(big_mul_raw(t, t), big_of(s)));
     } else {
-        const i64 ln = ln_frac(u.m, t);
+        const i64 ln = ln_frac(u.m, tab);
         i64 v;
         int sc;
         if (u.e >= -1) {  // -ln u = ln 2 - ln(2 u)
-            v = 3196577161300663915ll - ln - i64(q.m >> (1 - q.e));  // scale 2^62: t = m 2^(e - 63)
+            v = 3196577161300663915ll - ln - i64(t.m >> (1 - t.e));  // scale 2^62: t = m 2^(e - 63)
             sc = 62;
         } else {
-            v = i64(-u.e) * 49946518145322874ll - (ln >> 6) - i64(q.m >> (7 - q.e));  // scale 2^56
+            v = i64(-u.e) * 49946518145322874ll - (ln >> 6) - i64(t.m >> (7 - t.e));  // scale 2^56
             sc = 56;
         }
-#ifdef __CUDA_ARCH__
-        const int lz = __clzll(v);
-#else
-        const int lz = __builtin_clzll(v);
-#endif
+        const int lz = big_clz(u64(v));
         mu = Big{u64(v) << lz, 63 - lz - sc};
     }
-    return big_norm(big_mul_raw(big_norm(big_mul_raw(big_mul_raw(big_mul_raw(ir, ir), ir), big_of(gms))), mu));
+    if (l1) *l1 = big_add(t, mu);
+    return mu;
+}
+
+// G M_s mu(r/r_s) / r^3 of the NFW halo.
+__host__ __device__ __forceinline__ Big nfw_big(double gms, double rs, const Big &r, const Big &ir, const u64 *tab)
+{
+    return big_norm(big_mul_raw(big_norm(big_mul_raw(big_mul_raw(big_mul_raw(ir, ir), ir), big_of(gms))),
+                                nfw_mu_big(rs, r, tab)));
+}
+
+// ---------------------------------------------------------------- plain functions
+//
+// FP64 square root, quotient and logarithm on the integer pipe for the arguments of the prior
+// binning (the library's for anything out of range).
+
+__host__ __device__ __forceinline__ double sqrt_int(double x)
+{
+    if (!big_range(x)) return sqrt(x);
+    Big r, ir;
+    big_rsqrt(big_of(x), ir, r);
+    return big_double(r);
+}
+
+// a / b for b > 0
+__host__ __device__ __forceinline__ double div_int(double a, double b)
+{
+    const double p = of_bits(bits_of(a) & 0x7fffffffffffffffll);
+    if (!big_range(p) || !big_range(b)) return a / b;
+    const double q = big_double(big_norm(big_mul_raw(big_rcp(big_of(b)), big_of(p))));
+    return of_bits(bits_of(q) | (bits_of(a) & i64(1ull << 63)));
+}
+
+// ln x: within 2^-61 of it for 1/2 <= x < 2 and 2^-55 beyond.
+__host__ __device__ __forceinline__ double log_int(double x, const u64 *tab)
+{
+    if (!big_range(x)) return log(x);
+    const Big b = big_of(x);
+    const i64 ln = ln_frac(b.m, tab);
+    const bool near1 = b.e == 0 || b.e == -1;
+    i64 v = near1 ? (b.e ? ln - 3196577161300663915ll : ln) : i64(b.e) * 24973259072661437ll + (ln >> 7);  // 2^62, 2^55
+    if (v == 0) return 0.0;
+    const bool neg = v < 0;
+    if (neg) v = -v;
+    const int lz = big_clz(u64(v));
+    const double r = big_double(Big{u64(v) << lz, 63 - lz - (near1 ? 62 : 55)});
+    return neg ? -r : r;
 }
 
 }  // namespace m2m

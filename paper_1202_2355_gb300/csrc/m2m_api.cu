@@ -386,10 +386,7 @@ static m2m_status build_model(m2m_ctx *ctx, const m2m_potential *pot, const m2m_
     ctx->precision = opt->precision;
     m.wps = ctx->precision == M2M_PREC_FP64 ? 2 : 1;
     m.cache_accel = m.pot != 3 && (ctx->precision == M2M_PREC_FP64 || m.pot == 1) ? 1 : 0;
-    m.int_force = ctx->precision == M2M_PREC_FP64 &&
-                  (m.pot == 2 ? big_range(m.v0 * m.v0) && big_range(m.q * m.q)
-                              : m.pot < 2 && big_range(m.G * m.M) && big_range(m.a) &&
-                                    (m.pot == 0 || (big_range(m.G * m.Ms) && big_range(m.rs))));
+    m.int_force = ctx->precision == M2M_PREC_FP64 && int_force_ok(m);
     m.tab_smem = 1;
     m.off_total = m.J * m.wps;
     m.off_grid = (m.J + 1) * m.wps;
@@ -496,6 +493,7 @@ static m2m_status configure_kernels(m2m_ctx *ctx)
     const size_t red = size_t(ctx->block) * sizeof(double);
     m.win_group = 0;
     m.win_lo = m.win_n = 0;
+    m.cells_smem = 0;
     if (ctx->global_dep) {
         // an aperture window of the largest group keeps block-shared sums, as large as the
         // blocks that registers and threads allow on an SM (or blocks_per_sm) leave room for
@@ -512,7 +510,10 @@ static m2m_status configure_kernels(m2m_ctx *ctx)
         // 1 KB per block is reserved by the runtime; 1 KB more covers the carve's alignment
         const long long per_block = std::min<long long>(smsm / rb, maxsm) - 2048 - (long long)smem_bytes<T>(m, 0, 0);
         const long long slot_bytes = 3 * sizeof(int);
-        if (per_block > 0) m.win_n = int(std::min<long long>(m.g[best].n_ap, per_block / (slot_bytes * m.g[best].n_kinds)));
+        // the prior grid first (up to half of the room: its cells are the most contended sums)
+        m.cells_smem = 16ll * m.ncell <= per_block / 2;
+        const long long room = per_block - (m.cells_smem ? 16ll * m.ncell : 0);
+        if (room > 0) m.win_n = int(std::min<long long>(m.g[best].n_ap, room / (slot_bytes * m.g[best].n_kinds)));
         m.win_lo = (m.g[best].n_ap - m.win_n) / 2;  // until the load places it
     }
     ctx->smem_step = ctx->global_dep ? std::max(smem_bytes<T>(m, 2, 0), red) : smem_shared;
@@ -529,6 +530,18 @@ static m2m_status configure_kernels(m2m_ctx *ctx)
     return M2M_OK;
 }
 
+// The tables of the integer functions: exp, then ln (made once: long double arithmetic).
+const std::vector<u64> &fn_tables()
+{
+    static const std::vector<u64> fn = [] {
+        std::vector<u64> f(kExpEntries + 2 * kLnEntries);
+        exp_table(f.data());
+        ln_table(f.data() + kExpEntries);
+        return f;
+    }();
+    return fn;
+}
+
 // The host image of the step's tables (records and priors zero).
 template <class T>
 static std::vector<unsigned char> host_tables(const m2m_ctx *ctx, const TabLayout &t)
@@ -543,13 +556,7 @@ static std::vector<unsigned char> host_tables(const m2m_ctx *ctx, const TabLayou
     }
     for (int e = 0; e < m.n_edges_total; ++e) esq[e] = T(ctx->edges[e] * ctx->edges[e]);
     if (sizeof(T) == 8) {
-        static const std::vector<u64> fn = [] {  // made once: long double functions
-            std::vector<u64> f(kExpEntries + 2 * kLnEntries);
-            exp_table(f.data());
-            ln_table(f.data() + kExpEntries);
-            return f;
-        }();
-        std::memcpy(h.data() + t.et, fn.data(), t.bytes - t.et);
+        std::memcpy(h.data() + t.et, fn_tables().data(), t.bytes - t.et);
     }
     if (!ctx->lut.empty()) std::memcpy(h.data() + t.lut, ctx->lut.data(), sizeof(unsigned short) * ctx->lut.size());
     return h;
@@ -726,6 +733,11 @@ static m2m_status upload_tables(m2m_ctx *ctx)
         CU(cudaMemset(ctx->d_head, 0, sizeof(StepHead)));
     }
     if ((s = up(ctx->d_lcE, ctx->lcE)) != M2M_OK) return s;
+    if (ctx->precision == M2M_PREC_MIXED && !ctx->lcE.empty()) {
+        const std::vector<float> f(ctx->lcE.begin(), ctx->lcE.end());
+        CU(cudaMalloc(&ctx->d_lcEf, sizeof(float) * f.size()));
+        CU(cudaMemcpy(ctx->d_lcEf, f.data(), sizeof(float) * f.size(), cudaMemcpyHostToDevice));
+    }
     if (m.pot == 3) {
         if ((s = up(ctx->d_scf_r, ctx->scf_r)) != M2M_OK) return s;
         const size_t nt = size_t(m.scf_n + 1) * m.scf_nlm * 2;
@@ -837,7 +849,7 @@ extern "C" m2m_status m2m_create(const m2m_potential *pot, const m2m_observables
 Buffers buffers(m2m_ctx *c)
 {
     Buffers b;
-    b.tab = c->d_tab; b.head = c->d_head; b.Vp = c->d_Vp; b.isp = c->d_isp; b.Vpf = c->d_Vpf; b.ispf = c->d_ispf; b.lcE = c->d_lcE;
+    b.tab = c->d_tab; b.head = c->d_head; b.Vp = c->d_Vp; b.isp = c->d_isp; b.Vpf = c->d_Vpf; b.ispf = c->d_ispf; b.lcE = c->d_lcE; b.lcEf = c->d_lcEf;
     b.ipriorf = c->d_ipriorf;
     b.sig = c->d_sig; b.obs_kind = c->d_kind; b.plan = c->plan;
     b.c = c->d_c; b.rec = c->d_rec; b.recf = c->d_recf; b.prior = c->d_prior; b.iprior = c->d_iprior;
@@ -1940,7 +1952,7 @@ void destroy_impl(m2m_ctx *ctx)
     if (ctx->precision == M2M_PREC_MIXED) {  // in FP64 mode these are parts of d_tab
         free_dev(ctx->d_Vp); free_dev(ctx->d_isp); free_dev(ctx->d_rec); free_dev(ctx->d_lprior);
     }
-    free_dev(ctx->d_tab); free_dev(ctx->d_head); free_dev(ctx->d_plan); free_dev(ctx->d_lcE);
+    free_dev(ctx->d_tab); free_dev(ctx->d_head); free_dev(ctx->d_plan); free_dev(ctx->d_lcE); free_dev(ctx->d_lcEf);
     free_dev(ctx->d_scf_r); free_dev(ctx->d_scf_tab); free_dev(ctx->d_scf_tabf); free_dev(ctx->d_scf_coef);
     free_dev(ctx->d_sig);
     free_dev(ctx->d_kind); free_dev(ctx->d_c); free_dev(ctx->d_prior); free_dev(ctx->d_iprior);

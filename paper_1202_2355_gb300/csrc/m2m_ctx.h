@@ -42,7 +42,7 @@ struct m2m_ctx {
     unsigned char *d_tab = nullptr;
     m2m::StepHead *d_head = nullptr;
     double *d_Vp = nullptr, *d_isp = nullptr, *d_lcE = nullptr;
-    float *d_Vpf = nullptr, *d_ispf = nullptr, *d_ipriorf = nullptr;
+    float *d_Vpf = nullptr, *d_ispf = nullptr, *d_ipriorf = nullptr, *d_lcEf = nullptr;
     m2m::FinPlan plan{};
     unsigned char *d_plan = nullptr;  // the plan's arrays in one allocation, its rows first
     double *d_sig = nullptr;
@@ -122,6 +122,7 @@ m2m_status create_impl(const m2m_potential *pot, const m2m_observables *obs, con
                        double mu, double alpha, const m2m_options *opt, int internal, m2m_ctx **out);
 m2m_status check_device_errors(m2m_ctx *ctx);
 m2m::Buffers buffers(m2m_ctx *c);
+const std::vector<m2m::u64> &fn_tables();  // exp, then ln (fp64_int.cuh)
 void destroy_impl(m2m_ctx *ctx);
 
 // The (E, x) grid fields of a model (nE, nx, spacing, signed L_z, s_lo, s_den, ncell)
@@ -161,6 +162,15 @@ inline m2m::State<T> state(m2m_ctx *c)
     s.gx = sizeof(T) == 8 ? reinterpret_cast<T *>(c->gx) : nullptr;
     s.n = c->n;
     return s;
+}
+
+// Whether the potential's constants are in the range of the integer FP64 functions.
+inline bool int_force_ok(const m2m::Model &m)
+{
+    using m2m::big_range;
+    if (m.pot == 2) return big_range(m.v0 * m.v0) && big_range(m.q * m.q);
+    return m.pot < 2 && big_range(m.G * m.M) && big_range(m.a) &&
+           (m.pot == 0 || (big_range(m.G * m.Ms) && big_range(m.rs)));
 }
 
 // Shared memory of a block-shared step kernel: sums and tables, and at least what the

@@ -126,6 +126,8 @@ struct Model {
     // FP64 mode: the potential's constants are in the range of the integer force factors
     // (big_range), and whether the tables of the integer functions are in shared memory
     int int_force, tab_smem;
+    // global-deposit kernel: the prior grid's sums are block-shared
+    int cells_smem;
 };
 
 constexpr unsigned kApNone8 = 0xFFu, kApNone16 = 0xFFFFu;
@@ -326,6 +328,7 @@ struct Buffers {
     const double *Vp, *isp;          // per aperture V_p and 1/sigma_p
     const float *Vpf, *ispf;         // FP32 copies of V_p and 1/sigma_p (mixed mode)
     const double *lcE;               // E_c table
+    const float *lcEf;               // FP32 copy of it (mixed mode)
     const double *sig;
     const int *obs_kind;             // per observable: kind
     FinPlan plan;                    // the order of the finalize
@@ -601,8 +604,35 @@ __device__ __forceinline__ void scf_accel(const Model &m, const Cst<T> &k, T x, 
 // SCF: whether the code of the self-consistent potential is compiled in (only the generic
 // step kernel and the helpers around it need it; the kernels specialised to an observable
 // shape run the other potentials without its registers).
+// -phi of the spherical potentials at r (ir = 1/r), G M/(r + a) + G M_s ln(1 + r/r_s)/r, and, if
+// vc2 is not null, v_c^2 = G M r/(r + a)^2 + G M_s mu/r.
+__host__ __device__ __forceinline__ Big well_big(const Model &m, const Cst<double> &k, const Big &r, const Big &ir,
+                                                 const u64 *ln, Big *vc2)
+{
+    const Big gz = big_norm(big_mul_raw(big_rcp(big_add(r, big_of(k.a))), big_of(k.GM)));
+    Big w = gz;
+    if (vc2) {
+        const Big z = big_rcp(big_add(r, big_of(k.a)));
+        *vc2 = big_norm(big_mul_raw(big_mul_raw(gz, z), r));
+    }
+    if (m.pot == 1) {
+        Big l1;
+        const Big mu = nfw_mu_big(k.rs, r, ln, &l1);
+        const Big h = big_norm(big_mul_raw(ir, big_of(k.GMs)));
+        w = big_add(w, big_norm(big_mul_raw(h, l1)));
+        if (vc2) *vc2 = big_add(*vc2, big_norm(big_mul_raw(h, mu)));
+    }
+    return w;
+}
+
+// fn: FP64 mode, the tables of the integer functions (null: the library's).
+struct FnTables {
+    const u64 *et, *ln;
+};
+
 template <class T, bool SCF = true>
-__host__ __device__ __forceinline__ T potential(const Model &m, const Cst<T> &k, T x, T y, T z)
+__host__ __device__ __forceinline__ T potential(const Model &m, const Cst<T> &k, T x, T y, T z,
+                                                FnTables fn = FnTables{nullptr, nullptr})
 {
 #ifdef __CUDA_ARCH__
     if constexpr (SCF) {
@@ -612,6 +642,14 @@ __host__ __device__ __forceinline__ T potential(const Model &m, const Cst<T> &k,
     if (m.pot == 2) {
         const T D = fma(x, x, fma(y, y, k.r0sq)) + d_div(z * z, k.q2);
         return T(0.5) * k.v0sq * d_log(D);
+    }
+    if constexpr (sizeof(T) == 8) {
+        const T r2 = fma(x, x, fma(y, y, z * z));
+        if (fn.ln && m.int_force && big_range(r2)) {
+            Big r, ir;
+            big_rsqrt(big_of(r2), ir, r);
+            return -big_double(well_big(m, k, r, ir, fn.ln, nullptr));
+        }
     }
     const T r = d_sqrt(fma(x, x, fma(y, y, z * z)));
     T phi = -d_div(k.GM, r + k.a);
@@ -1238,8 +1276,18 @@ __device__ __forceinline__ void group_dkernels(const GroupDesc &G, const Tables<
 // NFW halo (shared by its potential and its enclosed mass); the flattened log halo
 // through accel and potential.
 template <class T, bool SCF = true>
-__host__ __device__ __forceinline__ void circ_terms(const Model &m, const Cst<T> &k, T R, T &vc2, T &phi)
+__host__ __device__ __forceinline__ void circ_terms(const Model &m, const Cst<T> &k, T R, T &vc2, T &phi,
+                                                    FnTables fn = FnTables{nullptr, nullptr})
 {
+    if constexpr (sizeof(T) == 8) {
+        if (m.pot < 2 && fn.ln && m.int_force && big_range(R)) {
+            const Big r = big_of(R);
+            Big v;
+            phi = -big_double(well_big(m, k, r, big_rcp(r), fn.ln, &v));
+            vc2 = big_double(v);
+            return;
+        }
+    }
     if (m.pot >= 2) {
         T ax, ay, az;
         accel<T, SCF>(m, k, R, T(0), T(0), ax, ay, az);
@@ -1271,27 +1319,50 @@ __host__ __device__ __forceinline__ void circ_terms(const Model &m, const Cst<T>
 
 // Energy of the circular orbit of radius R in the equatorial plane: phi(R) + v_c^2/2.
 template <class T, bool SCF = true>
-__host__ __device__ __forceinline__ T circ_energy(const Model &m, const Cst<T> &k, T R)
+__host__ __device__ __forceinline__ T circ_energy(const Model &m, const Cst<T> &k, T R,
+                                                  FnTables fn = FnTables{nullptr, nullptr})
 {
     T vc2, phi;
-    circ_terms<T, SCF>(m, k, R, vc2, phi);
+    circ_terms<T, SCF>(m, k, R, vc2, phi, fn);
     return phi + T(0.5) * vc2;
 }
 
 // Lc(E): closed form for the Hernquist potential (E_c = -(u+1)/(2u^2) GM/a with
 // u = R/a + 1), otherwise the host table of E_c(ln R) bracketed by binary search,
 // interpolated, and refined by secant steps on E_c(R) = E.
+// Square root, quotient (b > 0), exponential and logarithm of the prior binning: FP64 on the
+// integer pipe where fn has the tables.
+__device__ __forceinline__ float p_sqrt(float x, FnTables) { return d_sqrt(x); }
+__device__ __forceinline__ double p_sqrt(double x, FnTables fn) { return fn.et ? sqrt_int(x) : sqrt(x); }
+__device__ __forceinline__ float p_div(float a, float b, FnTables) { return d_div(a, b); }
+__device__ __forceinline__ double p_div(double a, double b, FnTables fn) { return fn.et ? div_int(a, b) : a / b; }
+__device__ __forceinline__ float p_exp(float x, FnTables) { return d_exp(x); }
+__device__ __forceinline__ double p_exp(double x, FnTables fn) { return fn.et ? exp_int(x, fn.et) : exp(x); }
+__device__ __forceinline__ float p_log(float x, FnTables) { return d_log(x); }
+__device__ __forceinline__ double p_log(double x, FnTables fn) { return fn.ln ? log_int(x, fn.ln) : log(x); }
+
+// The E_c table in the state type: FP64, or its FP32 copy (a conversion of each of the twenty
+// values a search reads would go through the FP64 pipe).
+template <class T>
+using LcTable = T;
+template <class T>
+__device__ __forceinline__ const T *lc_table(const Buffers &b);
+template <>
+__device__ __forceinline__ const double *lc_table<double>(const Buffers &b) { return b.lcE; }
+template <>
+__device__ __forceinline__ const float *lc_table<float>(const Buffers &b) { return b.lcEf; }
+
 template <class T, bool SCF = true>
-__device__ T circular_L(const Model &m, const Cst<T> &k, const double *lcE, T E)
+__device__ T circular_L(const Model &m, const Cst<T> &k, const LcTable<T> *lcE, T E, FnTables fn)
 {
     if (m.pot < 2 && !(E < T(0))) return T(0);
     if (m.lc_closed) {
         const T e = E * k.e_scale;
         if (!(e > T(-1))) return T(0);
-        const T u = d_div(T(-1) - d_sqrt(T(1) - T(8) * e), T(4) * e);
+        const T u = p_div(T(1) + p_sqrt(T(1) - T(8) * e, fn), T(-4) * e, fn);
         const T R = k.a * (u - T(1));
         const T ra = R + k.a;
-        return d_div(R * d_sqrt(k.GM * R), ra);
+        return p_div(R * p_sqrt(k.GM * R, fn), ra, fn);
     }
     if (!(E > k.phi_min)) return T(0);
     const int n = m.lc_n;
@@ -1350,15 +1421,15 @@ __device__ T circular_L(const Model &m, const Cst<T> &k, const double *lcE, T E)
             R = d_exp(fminf(fmaxf(lnr, ylo), ylo + k.lc_dlnr));
         } else {
             const T e0 = T(__ldg(lcE + lo)), e1 = T(__ldg(lcE + hi));
-            const T fr = d_div(E - e0, e1 - e0);
-            R = d_exp(k.lc_lnr0 + (T(lo) + fr) * k.lc_dlnr);
+            const T fr = p_div(E - e0, e1 - e0, fn);
+            R = p_exp(k.lc_lnr0 + (T(lo) + fr) * k.lc_dlnr, fn);
             // secant refinement, starting from the table segment's slope
-            const T Ra = d_exp(k.lc_lnr0 + T(lo) * k.lc_dlnr);
-            const T Rb = d_exp(k.lc_lnr0 + T(hi) * k.lc_dlnr);
-            T r0 = R, f0 = circ_energy<T, SCF>(m, k, r0) - E;
-            T r1 = r0 - f0 * d_div(Rb - Ra, e1 - e0);
+            const T Ra = p_exp(k.lc_lnr0 + T(lo) * k.lc_dlnr, fn);
+            const T Rb = p_exp(k.lc_lnr0 + T(hi) * k.lc_dlnr, fn);
+            T r0 = R, f0 = circ_energy<T, SCF>(m, k, r0, fn) - E;
+            T r1 = r0 - f0 * p_div(Rb - Ra, e1 - e0, fn);
             for (int it = 0; it < 3; ++it) {
-                const T f1 = circ_energy<T, SCF>(m, k, r1) - E;
+                const T f1 = circ_energy<T, SCF>(m, k, r1, fn) - E;
                 if (f1 == f0) break;
                 const T r2 = r1 - f1 * d_div(r1 - r0, f1 - f0);
                 r0 = r1;
@@ -1369,36 +1440,36 @@ __device__ T circular_L(const Model &m, const Cst<T> &k, const double *lcE, T E)
         }
     }
     T vc2, phi;
-    circ_terms<T, SCF>(m, k, R, vc2, phi);
-    return R * d_sqrt(vc2);
+    circ_terms<T, SCF>(m, k, R, vc2, phi, fn);
+    return R * p_sqrt(vc2, fn);
 }
 
 // Cell k*nx + l of a particle: E bin from the chosen spacing (clamped), circularity
 // bin from x = L/Lc(E) (x = Lz/Lc(E) on [-1, 1] for the signed variant, clamped).
 template <class T, bool SCF = true>
-__device__ __forceinline__ int prior_cell(const Model &m, const Cst<T> &k, const double *lcE, T x, T y, T z,
-                                          T vx, T vy, T vz)
+__device__ __forceinline__ int prior_cell(const Model &m, const Cst<T> &k, const LcTable<T> *lcE, T x, T y, T z,
+                                          T vx, T vy, T vz, FnTables fn)
 {
-    const T E = fma(T(0.5), fma(vx, vx, fma(vy, vy, vz * vz)), potential<T, SCF>(m, k, x, y, z));
+    const T E = fma(T(0.5), fma(vx, vx, fma(vy, vy, vz * vz)), potential<T, SCF>(m, k, x, y, z, fn));
     const T Lz = fma(x, vy, -(y * vx));
     T L;
     if (m.signed_lz) {
         L = Lz;
     } else {
         const T Lx = fma(y, vz, -(z * vy)), Ly = fma(z, vx, -(x * vz));
-        L = d_sqrt(fma(Lx, Lx, fma(Ly, Ly, Lz * Lz)));
+        L = p_sqrt(fma(Lx, Lx, fma(Ly, Ly, Lz * Lz)), fn);
     }
-    const T Lc = circular_L<T, SCF>(m, k, lcE, E);
-    T xc = (Lc > T(0)) ? d_div(L, Lc) : T(0);
+    const T Lc = circular_L<T, SCF>(m, k, lcE, E, fn);
+    T xc = (Lc > T(0)) ? p_div(L, Lc, fn) : T(0);
     const T xmin = m.signed_lz ? T(-1) : T(0);
     xc = xc < xmin ? xmin : (xc > T(1) ? T(1) : xc);
     T f;
-    if (m.e_spacing == 0) f = (E >= T(0)) ? T(1) : d_div(d_log(-E) - k.s_lo, k.s_den);
-    else if (m.e_spacing == 1) f = d_div(d_exp(E) - k.s_lo, k.s_den);
-    else f = d_div(E - k.s_lo, k.s_den);
+    if (m.e_spacing == 0) f = (E >= T(0)) ? T(1) : p_div(p_log(-E, fn) - k.s_lo, k.s_den, fn);
+    else if (m.e_spacing == 1) f = p_div(p_exp(E, fn) - k.s_lo, k.s_den, fn);
+    else f = p_div(E - k.s_lo, k.s_den, fn);
     const T fk = d_floor(f * k.nE);
     const int kb = !(fk >= T(0)) ? 0 : (fk >= k.nE ? m.nE - 1 : int(fk));
-    const T fl = d_floor(d_div(xc - xmin, T(1) - xmin) * k.nx);
+    const T fl = d_floor(p_div(xc - xmin, T(1) - xmin, fn) * k.nx);
     const int lb = !(fl >= T(0)) ? 0 : (fl >= k.nx ? m.nx - 1 : int(fl));
     return kb * m.nx + lb;
 }
@@ -1536,10 +1607,12 @@ struct Acc<float> {
 };
 
 // Particle counts of the cells, behind the sums.
-template <class T>
+__host__ __device__ inline int cell_slots(const Model &m);
+template <class T, bool GA = false>
 __device__ __forceinline__ unsigned *acc_counts(void *base, const Model &m)
 {
-    return static_cast<unsigned *>(base) + 3 * m.nslots;
+    const int slots = GA ? cell_slots(m) + (m.win_n > 0 ? m.g[m.win_group].n_kinds * m.win_n : 0) : m.nslots;
+    return static_cast<unsigned *>(base) + 3 * slots;
 }
 
 // Per-thread running total of the deposited weight, in the same fixed point.
@@ -1684,7 +1757,7 @@ __host__ __device__ inline TabLayout tab_layout(const Model &m)
     t.lut = t.esq + up(sizeof(T) * size_t(m.n_edges_total));
     t.et = t.lut + up(sizeof(unsigned short) * size_t(m.n_lut));
     t.ln = t.et + (sizeof(T) == 8 ? kExpEntries * int(sizeof(u64)) : 0);
-    t.bytes = t.ln + (sizeof(T) == 8 && m.pot == 1 ? 2 * kLnEntries * int(sizeof(u64)) : 0);
+    t.bytes = t.ln + (sizeof(T) == 8 && m.pot < 2 ? 2 * kLnEntries * int(sizeof(u64)) : 0);
     return t;
 }
 
@@ -1698,13 +1771,16 @@ struct Smem {
     int tab_lo, tab_hi;
 };
 
-// Block sums of the global-deposit kernel's aperture window: one slot per kind and
-// window aperture, laid out as Acc<T> slots.
+// Block sums of the global-deposit kernel, laid out as Acc<T> slots: the cells of the prior
+// grid with their counts behind the slots (where they fit, Model::cells_smem), and the aperture
+// window, one slot per kind and window aperture. (With the cells in global memory a prior update of
+// 8M particles on 800 cells took 2.3 ms, ten times the other steps.)
+__host__ __device__ inline int cell_slots(const Model &m) { return m.cells_smem ? m.ncell : 0; }
 template <class T>
 __host__ __device__ inline size_t window_bytes(const Model &m)
 {
-    const size_t slots = m.win_n > 0 ? size_t(m.g[m.win_group].n_kinds) * m.win_n : 0;
-    return slots * 3 * sizeof(int);
+    const size_t slots = (m.win_n > 0 ? size_t(m.g[m.win_group].n_kinds) * m.win_n : 0) + cell_slots(m);
+    return (slots * 3 + cell_slots(m)) * sizeof(int);
 }
 
 // hist: 0 no block sums, 1 all (Acc<T>), 2 the aperture window of the global deposit
@@ -2349,7 +2425,7 @@ __device__ __forceinline__ void step_particles(const Model &m, const Model &mh, 
                             if constexpr (GA) {
                                 const unsigned a = unsigned(p - mh.win_lo);
                                 if (g == mh.win_group && a < unsigned(mh.win_n))
-                                    Acc<T>::add(S.h, kk * mh.win_n + int(a), v, scale);
+                                    Acc<T>::add(S.h, cell_slots(mh) + kk * mh.win_n + int(a), v, scale);
                                 else
                                     global_add(b.hist, j, v, scale);
                             } else if (cls == kClassMass) {  // v is w (the kernel is 1)
@@ -2377,10 +2453,11 @@ __device__ __forceinline__ void step_particles(const Model &m, const Model &mh, 
             if constexpr (sizeof(T) == 4) wdep += w;
         }
         if (f.prior_step) {
-            const int c = prior_cell<T, kScf>(m, k, b.lcE, x, y, z, vx, vy, vz);
-            deposit(m.J + 1 + c, w, k.fx_w);
-            if constexpr (GA) red_add(b.hist + m.off_count + c, 1);
-            else atomicAdd(acc_counts<T>(S.h, m) + c, 1u);
+            const int c = prior_cell<T, kScf>(m, k, lc_table<T>(b), x, y, z, vx, vy, vz, FnTables{tb.et, m.pot < 2 ? tb.ln : nullptr});
+            if (GA && m.cells_smem) Acc<T>::add(S.h, c, w, k.fx_w);
+            else deposit(m.J + 1 + c, w, k.fx_w);
+            if (GA && !m.cells_smem) red_add(b.hist + m.off_count + c, 1);
+            else atomicAdd(acc_counts<T, GA>(S.h, m) + c, 1u);
             P.cell[i] = static_cast<uint16_t>(c);
         }
         P.x[i] = x; P.y[i] = y; P.z[i] = z;
@@ -2416,7 +2493,7 @@ __device__ __forceinline__ void block_flush(const Model &m, const Cst<T> &k, Sca
         for (int q = threadIdx.x; q < WPS * slots; q += blockDim.x) {
             const int slot = q / WPS, wd = q - slot * WPS;
             const int kk = slot / m.win_n, a = slot - kk * m.win_n;
-            const long long v = Acc<T>::word(S.h, slot, wd);
+            const long long v = Acc<T>::word(S.h, cell_slots(m) + slot, wd);
             const int j = G.obs_off + kk * G.n_ap + m.win_lo + a;
             if (v != 0) red_add(hist + WPS * j + wd, v);
         }
@@ -2429,8 +2506,14 @@ __device__ __forceinline__ void block_flush(const Model &m, const Cst<T> &k, Sca
         const long long v = Acc<T>::word(S.h, slot, q - slot * WPS);
         if (v != 0) red_add(hist + q, v);
     }
-    if (!GA && all) {
-        const unsigned *cnt = acc_counts<T>(S.h, m);
+    if (GA && all)
+        for (int q = threadIdx.x; q < WPS * cell_slots(m); q += blockDim.x) {
+            const int slot = q / WPS;
+            const long long v = Acc<T>::word(S.h, slot, q - slot * WPS);
+            if (v != 0) red_add(hist + WPS * (m.J + 1) + q, v);
+        }
+    if ((!GA || m.cells_smem) && all) {
+        const unsigned *cnt = acc_counts<T, GA>(S.h, m);
         for (int q = threadIdx.x; q < m.ncell; q += blockDim.x)
             if (cnt[q]) red_add(hist + m.off_count + q, static_cast<long long>(cnt[q]));
     }

@@ -152,13 +152,13 @@ __global__ void __launch_bounds__(kDiagThreads) k_kin_sums(const SphBins g, cons
 // First pass over the (E, x) grid: each particle's cell, the cell's weight and count.
 template <class T>
 __global__ void __launch_bounds__(kDiagThreads) k_grid_sums(const Model m, const Cst<double> k, const double *lcE,
-                                                            const Particles<T> p, DiagScales sc, int *cell,
+                                                            const Particles<T> p, DiagScales sc, FnTables fn, int *cell,
                                                             long long *wsum, unsigned long long *counts)
 {
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < p.n;
          i += (long long)gridDim.x * blockDim.x) {
         const int c = prior_cell<double>(m, k, lcE, double(p.x[i]), double(p.y[i]), double(p.z[i]),
-                                         double(p.vx[i]), double(p.vy[i]), double(p.vz[i]));
+                                         double(p.vx[i]), double(p.vy[i]), double(p.vz[i]), fn);
         cell[i] = c;
         fx_add(wsum + 2 * c, p.w[i], sc.w);
         atomicAdd(counts + c, 1ull);
@@ -375,12 +375,19 @@ extern "C" m2m_status m2m_diag_grid(m2m_ctx *ctx, const m2m_prior_grid *grid, in
     CU(cudaMemsetAsync(d_cnt, 0, sizeof(unsigned long long) * ncell, ctx->stream));
     if (np > 0) {
         const Cst<double> kd = make_cst<double>(m);
+        // FP64 arithmetic whatever the fit's precision: the integer functions of the prior binning
+        const std::vector<u64> &tab = fn_tables();
+        u64 *d_fn = nullptr;
+        CU(S.get(&d_fn, tab.size()));
+        CU(cudaMemcpyAsync(d_fn, tab.data(), sizeof(u64) * tab.size(), cudaMemcpyHostToDevice, ctx->stream));
+        const FnTables fn{d_fn, m.pot < 2 ? d_fn + kExpEntries : nullptr};
+        m.int_force = int_force_ok(m);
         const int gr = grid_of(ctx, np);
         if (src.kind == 2) {
-            k_grid_sums<float><<<gr, kDiagThreads, 0, ctx->stream>>>(m, kd, ctx->d_lcE, src.f, sc, d_cell, d_ws, d_cnt);
+            k_grid_sums<float><<<gr, kDiagThreads, 0, ctx->stream>>>(m, kd, ctx->d_lcE, src.f, sc, fn, d_cell, d_ws, d_cnt);
             k_grid_dev<<<gr, kDiagThreads, 0, ctx->stream>>>(np, d_cell, src.f.w, d_ws, d_cnt, sc, d_wd);
         } else {
-            k_grid_sums<double><<<gr, kDiagThreads, 0, ctx->stream>>>(m, kd, ctx->d_lcE, src.d, sc, d_cell, d_ws, d_cnt);
+            k_grid_sums<double><<<gr, kDiagThreads, 0, ctx->stream>>>(m, kd, ctx->d_lcE, src.d, sc, fn, d_cell, d_ws, d_cnt);
             k_grid_dev<<<gr, kDiagThreads, 0, ctx->stream>>>(np, d_cell, src.d.w, d_ws, d_cnt, sc, d_wd);
         }
         CU(cudaGetLastError());
