@@ -209,7 +209,7 @@ typedef struct {
     void *stream;                  /* cudaStream_t to run on; NULL: the library creates one */
     int32_t block;                 /* threads per block of the step kernel, a multiple of 32: at most
                                       256, or 1024 for the mixed-precision global-deposit kernel;
-                                      0: 256 (512 for the global-deposit kernel) */
+                                      0: 256 (1024 for the mixed global-deposit kernel) */
     int32_t blocks_per_sm;         /* resident blocks per SM; 0: as many as fit. With global
                                       deposits it also sizes the aperture window (a share of
                                       the SM's shared memory per block) */

@@ -484,9 +484,11 @@ static m2m_status configure_kernels(m2m_ctx *ctx)
     for (int g = 0; g < m.n_groups; ++g) chunks += m.g[g].n_kinds * ((m.g[g].n_ap + 31) / 32);
     m.fin_wide = ctx->global_dep || chunks > 16;
     const int max_block = ctx->global_dep ? kStepMaxThreads<T, true> : kStepMaxThreads<T, false>;
-    // 512 threads in two blocks per SM was the fastest shape of the mixed-precision
-    // global-deposit kernel on 64x64 maps (1024 x 1 and 256 x 4 were 8-10 % slower)
-    if (ctx->block == 0) ctx->block = std::min(max_block, 512);
+    // One block of 1024 threads an SM for the mixed global-deposit kernel: its shared memory then
+    // holds the sums of all of a 64 x 64 map of five moments (two words each). us per step at 8M
+    // particles: 1024 x 1 208, 768 x 1 243, 512 x 2 (three fifths of the map each) 253, 256 x 4 261;
+    // at 300,000: 31.1, 33.2, 34.4, 33.9.
+    if (ctx->block == 0) ctx->block = max_block;
     if (ctx->block % 32 != 0 || ctx->block < 32 || ctx->block > max_block)
         return fail(ctx, M2M_ERR_ARG, "block must be a multiple of 32, <= %d", max_block);
     ctx->kstep = reinterpret_cast<void *>(ctx->global_dep ? pick_step<T, WPS, true>(m) : pick_step<T, WPS, false>(m));
@@ -509,7 +511,7 @@ static m2m_status configure_kernels(m2m_ctx *ctx)
         m.win_group = best;
         // 1 KB per block is reserved by the runtime; 1 KB more covers the carve's alignment
         const long long per_block = std::min<long long>(smsm / rb, maxsm) - 2048 - (long long)smem_bytes<T>(m, 0, 0);
-        const long long slot_bytes = 3 * sizeof(int);
+        const long long slot_bytes = WinAcc<T>::kWords * sizeof(int);
         // the prior grid first (up to half of the room: its cells are the most contended sums)
         m.cells_smem = 16ll * m.ncell <= per_block / 2;
         const long long room = per_block - (m.cells_smem ? 16ll * m.ncell : 0);

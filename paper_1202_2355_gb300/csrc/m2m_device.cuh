@@ -1606,13 +1606,44 @@ struct Acc<float> {
     }
 };
 
+// Sums of the global-deposit kernel's shared slots (n of them), where space decides how much
+// of a map has block-shared sums: FP64 as above, mixed two 32-bit words modulo 2^64 with a carry,
+// those of one significance together (two thirds of the space of the three limbs, and one or
+// two atomics each deposit).
+template <class T>
+struct WinAcc : Acc<T> {
+    static constexpr int kWords = 3;
+    __device__ static void add(void *base, int, int slot, T v, T scale) { Acc<T>::add(base, slot, v, scale); }
+    __device__ static long long word(const void *base, int, int slot, int wd) { return Acc<T>::word(base, slot, wd); }
+};
+template <>
+struct WinAcc<float> : Acc<float> {
+    static constexpr int kWords = 2;
+    __device__ static void add(void *base, int n, int slot, float v, float scale)
+    {
+        const long long L = fx(v, scale).L;
+        unsigned *h = static_cast<unsigned *>(base) + slot;
+        const unsigned c = add_word(h, unsigned(L), 0u);
+        const unsigned top = unsigned(static_cast<unsigned long long>(L) >> 32) + c;
+        if (top) atomicAdd(h + n, top);
+    }
+    __device__ static long long word(const void *base, int n, int slot, int)
+    {
+        const unsigned *h = static_cast<const unsigned *>(base) + slot;
+        return static_cast<long long>((static_cast<unsigned long long>(h[n]) << 32) | h[0]);
+    }
+};
+
 // Particle counts of the cells, behind the sums.
-__host__ __device__ inline int cell_slots(const Model &m);
+__host__ __device__ inline int cell_slots(const Model &m) { return m.cells_smem ? m.ncell : 0; }
+__host__ __device__ inline int ga_slots(const Model &m)
+{
+    return cell_slots(m) + (m.win_n > 0 ? m.g[m.win_group].n_kinds * m.win_n : 0);
+}
 template <class T, bool GA = false>
 __device__ __forceinline__ unsigned *acc_counts(void *base, const Model &m)
 {
-    const int slots = GA ? cell_slots(m) + (m.win_n > 0 ? m.g[m.win_group].n_kinds * m.win_n : 0) : m.nslots;
-    return static_cast<unsigned *>(base) + 3 * slots;
+    return static_cast<unsigned *>(base) + (GA ? WinAcc<T>::kWords * ga_slots(m) : 3 * m.nslots);
 }
 
 // Per-thread running total of the deposited weight, in the same fixed point.
@@ -1775,12 +1806,10 @@ struct Smem {
 // grid with their counts behind the slots (where they fit, Model::cells_smem), and the aperture
 // window, one slot per kind and window aperture. (With the cells in global memory a prior update of
 // 8M particles on 800 cells took 2.3 ms, ten times the other steps.)
-__host__ __device__ inline int cell_slots(const Model &m) { return m.cells_smem ? m.ncell : 0; }
 template <class T>
 __host__ __device__ inline size_t window_bytes(const Model &m)
 {
-    const size_t slots = (m.win_n > 0 ? size_t(m.g[m.win_group].n_kinds) * m.win_n : 0) + cell_slots(m);
-    return (slots * 3 + cell_slots(m)) * sizeof(int);
+    return (size_t(ga_slots(m)) * WinAcc<T>::kWords + cell_slots(m)) * sizeof(int);
 }
 
 // hist: 0 no block sums, 1 all (Acc<T>), 2 the aperture window of the global deposit
@@ -2425,7 +2454,7 @@ __device__ __forceinline__ void step_particles(const Model &m, const Model &mh, 
                             if constexpr (GA) {
                                 const unsigned a = unsigned(p - mh.win_lo);
                                 if (g == mh.win_group && a < unsigned(mh.win_n))
-                                    Acc<T>::add(S.h, cell_slots(mh) + kk * mh.win_n + int(a), v, scale);
+                                    WinAcc<T>::add(S.h, ga_slots(mh), cell_slots(mh) + kk * mh.win_n + int(a), v, scale);
                                 else
                                     global_add(b.hist, j, v, scale);
                             } else if (cls == kClassMass) {  // v is w (the kernel is 1)
@@ -2454,7 +2483,7 @@ __device__ __forceinline__ void step_particles(const Model &m, const Model &mh, 
         }
         if (f.prior_step) {
             const int c = prior_cell<T, kScf>(m, k, lc_table<T>(b), x, y, z, vx, vy, vz, FnTables{tb.et, m.pot < 2 ? tb.ln : nullptr});
-            if (GA && m.cells_smem) Acc<T>::add(S.h, c, w, k.fx_w);
+            if (GA && m.cells_smem) WinAcc<T>::add(S.h, ga_slots(m), c, w, k.fx_w);
             else deposit(m.J + 1 + c, w, k.fx_w);
             if (GA && !m.cells_smem) red_add(b.hist + m.off_count + c, 1);
             else atomicAdd(acc_counts<T, GA>(S.h, m) + c, 1u);
@@ -2493,7 +2522,7 @@ __device__ __forceinline__ void block_flush(const Model &m, const Cst<T> &k, Sca
         for (int q = threadIdx.x; q < WPS * slots; q += blockDim.x) {
             const int slot = q / WPS, wd = q - slot * WPS;
             const int kk = slot / m.win_n, a = slot - kk * m.win_n;
-            const long long v = Acc<T>::word(S.h, cell_slots(m) + slot, wd);
+            const long long v = WinAcc<T>::word(S.h, ga_slots(m), cell_slots(m) + slot, wd);
             const int j = G.obs_off + kk * G.n_ap + m.win_lo + a;
             if (v != 0) red_add(hist + WPS * j + wd, v);
         }
@@ -2509,7 +2538,7 @@ __device__ __forceinline__ void block_flush(const Model &m, const Cst<T> &k, Sca
     if (GA && all)
         for (int q = threadIdx.x; q < WPS * cell_slots(m); q += blockDim.x) {
             const int slot = q / WPS;
-            const long long v = Acc<T>::word(S.h, slot, q - slot * WPS);
+            const long long v = WinAcc<T>::word(S.h, ga_slots(m), slot, q - slot * WPS);
             if (v != 0) red_add(hist + WPS * (m.J + 1) + q, v);
         }
     if ((!GA || m.cells_smem) && all) {
@@ -2537,7 +2566,7 @@ __device__ __forceinline__ bool block_is_last(unsigned *counter, unsigned blocks
 
 // Threads per block the step kernel is compiled for. The mixed-precision global-deposit
 // kernel runs up to 1024 threads in one block per SM, so that one aperture window takes
-// the whole shared memory of the SM.
+// the whole shared memory of the SM (DRAM and L2 see the deposits once per block).
 template <class T, bool GA>
 constexpr int kStepMaxThreads = (GA && sizeof(T) == 4) ? 1024 : 256;
 
