@@ -160,6 +160,8 @@ static m2m_status build_model(m2m_ctx *ctx, const m2m_potential *pot, const m2m_
         G.geometry = S.geometry;
         G.n_ap = S.n_ap;
         G.n_kinds = S.n_kinds;
+        m.alm_lmax[g] = 0;
+        std::memset(m.alm_k[g], -1, sizeof m.alm_k[g]);
         if (S.n_ap < 1) return fail(ctx, M2M_ERR_ARG, "group %d: n_ap must be >= 1", g);
         if (S.n_kinds < 1 || S.n_kinds > kMaxKinds) return fail(ctx, M2M_ERR_ARG, "group %d: n_kinds must be 1..%d", g, kMaxKinds);
         G.obs_off = J;
@@ -254,6 +256,8 @@ static m2m_status build_model(m2m_ctx *ctx, const m2m_potential *pot, const m2m_
                 G.alm_m[k] = (signed char)mm;
                 G.alm_norm[k] = nrm;
                 G.alm_norm_f[k] = float(nrm);
+                m.alm_k[g][lm] = (signed char)k;
+                m.alm_lmax[g] = std::max(m.alm_lmax[g], l);
                 for (int p = 0; p < S.n_ap; ++p) {
                     ctx->obs_kind.push_back(kind);
                     ctx->obs_post.push_back(1.0);
@@ -742,7 +746,7 @@ static m2m_status upload_tables(m2m_ctx *ctx)
     }
     if (m.pot == 3) {
         if ((s = up(ctx->d_scf_r, ctx->scf_r)) != M2M_OK) return s;
-        const size_t nt = size_t(m.scf_n + 1) * m.scf_nlm * 2;
+        const size_t nt = size_t(m.scf_n + 1) * (m.scf_nlm + m.scf_lmax + 1) * 2;  // intervals, then the x axis
         free_dev(ctx->d_scf_tab);
         free_dev(ctx->d_scf_tabf);
         free_dev(ctx->d_scf_coef);
@@ -915,7 +919,8 @@ static void launch_step_timed(m2m_ctx *c, cudaEvent_t *ev)
 static size_t elem_size(const m2m_ctx *c) { return c->precision == M2M_PREC_FP64 ? 8 : 4; }
 
 // x, y, z, vx, vy, vz, w and, where the step keeps it, the force factor of the acceleration
-static int state_arrays(const m2m_ctx *c) { return c->m.cache_accel ? 8 : 7; }
+// (the self-consistent potential: its three components)
+static int state_arrays(const m2m_ctx *c) { return c->m.pot == 3 ? 10 : (c->m.cache_accel ? 8 : 7); }
 
 static m2m_status ensure_capacity(m2m_ctx *ctx, long long n)
 {

@@ -67,7 +67,7 @@ static bool group_hot_equal(const GroupDesc &a, const GroupDesc &b)
     for (int n = 0; eq && n < 7; ++n) eq = a.k_gh[n] == b.k_gh[n];
     for (int q = 0; eq && q < a.n_kinds; ++q)
         eq = a.kinds[q] == b.kinds[q] && a.alm_l[q] == b.alm_l[q] && a.alm_m[q] == b.alm_m[q] &&
-             a.alm_norm[q] == b.alm_norm[q] && a.alm_norm_f[q] == b.alm_norm_f[q];
+             a.alm_norm[q] == b.alm_norm[q] && a.alm_norm_f[q] == b.alm_norm_f[q];  // (and so alm_k, alm_lmax)
     return eq;
 }
 

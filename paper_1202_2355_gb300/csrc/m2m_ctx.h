@@ -157,6 +157,7 @@ inline m2m::State<T> state(m2m_ctx *c)
     s.x = (T *)c->st[0]; s.y = (T *)c->st[1]; s.z = (T *)c->st[2];
     s.vx = (T *)c->st[3]; s.vy = (T *)c->st[4]; s.vz = (T *)c->st[5]; s.w = (T *)c->st[6];
     s.fa = (T *)c->st[7];
+    s.ax = (T *)c->st[7]; s.ay = (T *)c->st[8]; s.az = (T *)c->st[9];
     s.cell = c->cell;
     s.ap = c->ap;
     s.gx = sizeof(T) == 8 ? reinterpret_cast<T *>(c->gx) : nullptr;

@@ -128,6 +128,9 @@ struct Model {
     int int_force, tab_smem;
     // global-deposit kernel: the prior grid's sums are block-shared
     int cells_smem;
+    // shell groups: highest l, and the kind of each (l, m) (index l (l + 1) + m) or -1
+    int alm_lmax[kMaxGroups];
+    signed char alm_k[kMaxGroups][56];
 };
 
 constexpr unsigned kApNone8 = 0xFFu, kApNone16 = 0xFFFFu;
@@ -258,7 +261,7 @@ struct Scalars {
 struct alignas(16) StepHead {
     int pending, prior_step, scf_step;
     float wscale, iwhat;      // mixed mode: weight scale, 1/flat prior (0 when it reads 0)
-    int pad;
+    int fresh;                // the self-consistent potential was rebuilt since the last push
     double lwscale, lwhat;    // FP64 mode: ln of both
 };
 
@@ -266,6 +269,7 @@ template <class T>
 struct State {
     T *x, *y, *z, *vx, *vy, *vz, *w;
     T *fa;            // force factor of the acceleration at the current positions (Model::cache_accel)
+    T *ax, *ay, *az;  // self-consistent potential: the acceleration itself
     uint16_t *cell;
     uint16_t *ap;     // cached apertures (Model::ap_cache), null without the cache
     T *gx;            // cached exp(-nu^2/2) of Model::gx_group (FP64 mode), else null
@@ -291,8 +295,8 @@ constexpr bool kLogWeights = sizeof(T) == 8;
 template <class T>
 constexpr bool kCacheAccel = sizeof(T) == 8;
 
-// The self-consistent potential is not of the force-factor form: its acceleration is
-// evaluated at both ends of the step.
+// The self-consistent potential is not of the force-factor form: its three components are
+// kept, and formed anew after a step that rebuilt the expansion (StepHead::fresh).
 template <class T>
 __host__ __device__ __forceinline__ bool keeps_accel(const Model &m)
 {
@@ -467,6 +471,19 @@ __host__ __device__ __forceinline__ void nfw_logs(float q, float &l1, float &mu)
     }
 }
 
+// 1/n of a small integer, 1 <= n <= 6 (a division in the inner recurrences otherwise).
+template <class T>
+__device__ __forceinline__ T inv_small(int n)
+{
+    return n == 1 ? T(1) : n == 2 ? T(0.5) : n == 3 ? T(1.0 / 3.0) : n == 4 ? T(0.25) : n == 5 ? T(0.2) : T(1.0 / 6.0);
+}
+
+// Square root and quotient (b > 0) of the shell geometry: on the integer pipe in FP64.
+__device__ __forceinline__ float g_sqrt(float x) { return d_sqrt(x); }
+__device__ __forceinline__ double g_sqrt(double x) { return sqrt_int(x); }
+__device__ __forceinline__ float g_div(float a, float b) { return d_div(a, b); }
+__device__ __forceinline__ double g_div(double a, double b) { return div_int(a, b); }
+
 // ---------------------------------------------------------------- self-consistent potential
 //
 // The stellar potential of pot 3 (Sec. 6) is the multipole expansion of the particles'
@@ -512,8 +529,8 @@ __device__ T scf_field(const Model &m, T x, T y, T z, T *g)
     const int j = scf_interval(m, r2);
     const T *tab = scf_table<T>(m) + size_t(j) * m.scf_nlm * 2;
     const bool inner = j > 0;  // then r >= r_0 > 0
-    const T ir2 = inner ? T(1) / r2 : T(0);
-    const T ir = inner ? d_sqrt(ir2) : T(0);
+    const T ir2 = inner ? g_div(T(1), r2) : T(0);
+    const T ir = inner ? g_sqrt(ir2) : T(0);
     const int L = m.scf_lmax;
     T phi = T(0), gx = T(0), gy = T(0), gz = T(0);
     T cm = T(1), sm = T(0), cm1 = T(0), sm1 = T(0);  // (x + iy)^m and (x + iy)^(m-1)
@@ -525,7 +542,7 @@ __device__ T scf_field(const Model &m, T x, T y, T z, T *g)
         T irl = irm;
         for (int l = mm; l <= L; ++l) {
             if (l > mm) {  // the recurrence in l
-                const T a = T(2 * l - 1), bq = T(l + mm - 1), il = T(1) / T(l - mm);
+                const T a = T(2 * l - 1), bq = T(l + mm - 1), il = inv_small<T>(l - mm);
                 const T tn = (a * z * t1 - bq * r2 * t0) * il;
                 const T tnz = (a * (t1 + z * t1z) - bq * r2 * t0z) * il;
                 const T tnr = (a * z * t1r - bq * (t0 + r2 * t0r)) * il;
@@ -594,11 +611,37 @@ __device__ __forceinline__ void scf_accel(const Model &m, const Cst<T> &k, T x, 
 {
     T g[3];
     scf_field<T>(m, x, y, z, g);
-    const T D = fma(x, x, fma(y, y, k.r0sq)) + d_div(z * z, k.q2);
-    const T f = -d_div(k.v0sq, D);
+    const T D = fma(x, x, fma(y, y, k.r0sq)) + g_div(z * z, k.q2);
+    const T f = -g_div(k.v0sq, D);
     ax = fma(f, x, -g[0]);
     ay = fma(f, y, -g[1]);
-    az = d_div(f * z, k.q2) - g[2];
+    az = g_div(f * z, k.q2) - g[2];
+}
+
+// Energy and v_c^2 of the circular orbit of radius R on the x axis of the self-consistent
+// potential. There theta = pi/2 and phi = 0, so within an interval of the grid phi_star is
+// sum_l A_l R^-(l+1) + B_l R^l, with A_l, B_l summed over m by the finalize (scf_axis), and its
+// derivative R d/dR follows term by term: some ten operations per l where the field takes a
+// hundred per (l, m), in the bisection for Lc(E) that runs 60 times per particle and update.
+template <class T>
+__device__ __forceinline__ T scf_circ(const Model &m, const Cst<T> &k, T R, T &vc2)
+{
+    const T R2 = R * R;
+    const int j = scf_interval(m, R2);
+    const double *ax = m.scf_tab + size_t(m.scf_n + 1) * m.scf_nlm * 2 + size_t(j) * (m.scf_lmax + 1) * 2;
+    const T iR = j > 0 ? g_div(T(1), R) : T(0);
+    T phi = T(0), v = T(0), a = iR, p = T(1);
+    for (int l = 0; l <= m.scf_lmax; ++l) {
+        const T ta = T(__ldcg(ax + 2 * l)) * a, tb = T(__ldcg(ax + 2 * l + 1)) * p;
+        phi += ta + tb;
+        v += T(l) * tb - T(l + 1) * ta;
+        a *= iR;
+        p *= R;
+    }
+    const T D = R2 + k.r0sq;
+    phi += T(0.5) * k.v0sq * d_log(D);
+    vc2 = v + g_div(k.v0sq * R2, D);
+    return phi + T(0.5) * vc2;
 }
 
 // SCF: whether the code of the self-consistent potential is compiled in (only the generic
@@ -766,18 +809,26 @@ __device__ __forceinline__ void leapfrog_from(const Model &m, const Cst<T> &k, T
 }
 
 // One kick-drift-kick leap-frog step.
-template <class T, bool SCF = true>
+template <class T>
 __device__ __forceinline__ void leapfrog(const Model &m, const Cst<T> &k, T &x, T &y, T &z, T &vx, T &vy, T &vz)
 {
-    T ax, ay, az;
-    accel<T, SCF>(m, k, x, y, z, ax, ay, az);
+    T f = accel_factor(m, k, x, y, z);
+    leapfrog_from(m, k, x, y, z, vx, vy, vz, f, nullptr);
+}
+
+// The same from the acceleration (ax, ay, az) at the start, which becomes that at the end
+// (the self-consistent potential).
+template <class T>
+__device__ __forceinline__ void leapfrog_scf(const Model &m, const Cst<T> &k, T &x, T &y, T &z, T &vx, T &vy, T &vz,
+                                             T &ax, T &ay, T &az)
+{
     vx = fma(k.hdt, ax, vx);
     vy = fma(k.hdt, ay, vy);
     vz = fma(k.hdt, az, vz);
     x = fma(k.dt, vx, x);
     y = fma(k.dt, vy, y);
     z = fma(k.dt, vz, z);
-    accel<T, SCF>(m, k, x, y, z, ax, ay, az);
+    accel<T, true>(m, k, x, y, z, ax, ay, az);
     vx = fma(k.hdt, ax, vx);
     vy = fma(k.hdt, ay, vy);
     vz = fma(k.hdt, az, vz);
@@ -1050,11 +1101,11 @@ __device__ __forceinline__ int shell_cic(const GroupDesc &G, const T *esq, T r2,
         if (e[mid] <= r2) lo = mid;
         else hi = mid;
     }
-    const T r = d_sqrt(r2), ra = d_sqrt(e[lo]), rb = d_sqrt(e[hi]);
+    const T r = g_sqrt(r2), ra = g_sqrt(e[lo]), rb = g_sqrt(e[hi]);
     const T d = rb - ra;
     p0 = lo;
-    g0 = d_div(rb - r, d);
-    g1 = d_div(r - ra, d);
+    g0 = g_div(rb - r, d);
+    g1 = g_div(r - ra, d);
     return 2;
 }
 
@@ -1065,65 +1116,69 @@ __device__ __forceinline__ void shell_angles(T x, T y, T z, T &ct, T &st, T &cp,
 {
     // explicit fused forms: the same rounding in every kernel that inlines this
     const T R2 = fma(x, x, y * y);
-    const T R = d_sqrt(R2), r = d_sqrt(fma(z, z, R2));
+    const T R = g_sqrt(R2), r = g_sqrt(fma(z, z, R2));
     const bool c = r > T(0), a = R > T(0);
-    ct = c ? d_div(z, r) : T(1);
-    st = c ? d_div(R, r) : T(0);
-    cp = a ? d_div(x, R) : T(1);
-    sp = a ? d_div(y, R) : T(0);
+    ct = c ? g_div(z, r) : T(1);
+    st = c ? g_div(R, r) : T(0);
+    cp = a ? g_div(x, R) : T(1);
+    sp = a ? g_div(y, R) : T(0);
 }
 
-// Y_lm of kind kk of a shell group.
-template <class T>
-__device__ __forceinline__ T shell_ylm(const GroupDesc &G, int kk, T ct, T st, T cp, T sp)
+// f(kk, Y_lm) for every kind kk of shell group g: one sweep over l for each |m| (every P_l^m once,
+// for the cosine and the sine; a sweep per kind takes three times as many FP64 instructions
+// for l <= 4).
+template <class T, class F>
+__device__ __forceinline__ void shell_sweep(const Model &m, int g, const GroupDesc &G, T ct, T st, T cp, T sp, F &&f)
 {
-    const int l = G.alm_l[kk], m = G.alm_m[kk], am = m < 0 ? -m : m;
-    T pmm = T(1);
-    for (int i = 1; i <= am; ++i) pmm *= T(2 * i - 1) * st;
-    T plm = pmm;
-    if (l > am) {
-        T p0 = pmm, p1 = ct * T(2 * am + 1) * pmm;
-        for (int ll = am + 2; ll <= l; ++ll) {
-            const T p2 = d_div(fma(ct * T(2 * ll - 1), p1, -(T(ll + am - 1) * p0)), T(ll - am));
-            p0 = p1;
-            p1 = p2;
+    const int L = m.alm_lmax[g];
+    T cm = T(1), sm = T(0), pmm = T(1);
+    for (int mm = 0; mm <= L; ++mm) {
+        T p0 = T(0), p1 = pmm;
+        for (int l = mm; l <= L; ++l) {
+            if (l > mm) {
+                const T p2 = fma(ct * T(2 * l - 1), p1, -(T(l + mm - 1) * p0)) * inv_small<T>(l - mm);
+                p0 = p1;
+                p1 = p2;
+            }
+            for (int v = 0; v < (mm > 0 ? 2 : 1); ++v) {
+                const int kk = m.alm_k[g][l * (l + 1) + (v == 0 ? mm : -mm)];
+                if (kk < 0) continue;
+                const T nrm = sizeof(T) == 8 ? T(G.alm_norm[kk]) : T(G.alm_norm_f[kk]);
+                f(kk, nrm * p1 * (v == 0 ? cm : sm));
+            }
         }
-        plm = p1;
+        const T cn = fma(cm, cp, -(sm * sp));
+        sm = fma(sm, cp, cm * sp);
+        cm = cn;
+        pmm *= T(2 * mm + 1) * st;
     }
-    T c = T(1), s = T(0);
-    for (int i = 0; i < am; ++i) {
-        const T c2 = fma(c, cp, -(s * sp));
-        s = fma(s, cp, c * sp);
-        c = c2;
-    }
-    const T nrm = sizeof(T) == 8 ? T(G.alm_norm[kk]) : T(G.alm_norm_f[kk]);
-    return nrm * plm * (m > 0 ? c : (m < 0 ? s : T(1)));
 }
 
 // emit(slot, w K_slot, class, kind index) for every a_lm of the group at the particle's
 // one or two grid points.
 template <class T, class F>
-__device__ __forceinline__ void shell_kernels(const GroupDesc &G, const Tables<T> &tb, T x, T y, T z, T w, F &&emit)
+__device__ __forceinline__ void shell_kernels(const Model &m, int g, const Tables<T> &tb, T x, T y, T z, T w, F &&emit)
 {
+    const GroupDesc &G = m.g[g];
     int p0 = 0;
     T g0 = T(0), g1 = T(0);
     const int np = shell_cic(G, tb.esq, fma(z, z, fma(x, x, y * y)), p0, g0, g1);
     if (np == 0) return;
     T ct, st, cp, sp;
     shell_angles(x, y, z, ct, st, cp, sp);
-    for (int kk = 0; kk < G.n_kinds; ++kk) {
-        const T v = w * shell_ylm(G, kk, ct, st, cp, sp);
+    shell_sweep(m, g, G, ct, st, cp, sp, [&](int kk, T Y) {
+        const T v = w * Y;
         const int j = G.obs_off + kk * G.n_ap + p0;
         emit(j, g0 * v, kClassGH, kk);
         if (np == 2) emit(j + 1, g1 * v, kClassGH, kk);
-    }
+    });
 }
 
 // sum_j K_j c_j over the group's a_lm: the records of a shell group hold c_j per kind.
 template <class T>
-__device__ __forceinline__ T shell_data(const Model &m, const GroupDesc &G, const Tables<T> &tb, const T *rec, T x,
-                                        T y, T z)
+__device__ __forceinline__ T shell_data(const Model &m, int g, const Tables<T> &tb, const T *rec, T x, T y, T z)
 {
+    const GroupDesc &G = m.g[g];
     int p0 = 0;
     T g0 = T(0), g1 = T(0);
     const int np = shell_cic(G, tb.esq, fma(z, z, fma(x, x, y * y)), p0, g0, g1);
@@ -1132,11 +1187,10 @@ __device__ __forceinline__ T shell_data(const Model &m, const GroupDesc &G, cons
     shell_angles(x, y, z, ct, st, cp, sp);
     const T *r0 = rec + (G.ap_off + p0) * m.rec_len;
     T d0 = T(0), d1 = T(0);
-    for (int kk = 0; kk < G.n_kinds; ++kk) {
-        const T Y = shell_ylm(G, kk, ct, st, cp, sp);
+    shell_sweep(m, g, G, ct, st, cp, sp, [&](int kk, T Y) {
         d0 = fma(Y, r0[kk], d0);
         if (np == 2) d1 = fma(Y, r0[m.rec_len + kk], d1);
-    }
+    });
     return fma(g0, d0, g1 * d1);
 }
 
@@ -1149,7 +1203,7 @@ __device__ __forceinline__ T data_term(const Model &m, const Tables<T> &tb, cons
         constexpr unsigned M = decltype(P)::mask;
         const GroupDesc &G = m.g[g];
         if (GP<M>::shells(G)) {
-            data += shell_data(m, G, tb, rec, x, y, z);
+            data += shell_data(m, g, tb, rec, x, y, z);
             return;
         }
         const int p = aperture<M>(G, tb.esq, tb.lut, X, Y);
@@ -1218,7 +1272,7 @@ __device__ __forceinline__ void scf_deposit(const Model &m, T x, T y, T z, T w, 
         T p0 = T(0), p1 = pmm;
         for (int l = mm; l <= L; ++l) {
             if (l > mm) {
-                const T p2 = d_div(fma(ct * T(2 * l - 1), p1, -(T(l + mm - 1) * p0)), T(l - mm));
+                const T p2 = fma(ct * T(2 * l - 1), p1, -(T(l + mm - 1) * p0)) * inv_small<T>(l - mm);
                 p0 = p1;
                 p1 = p2;
             }
@@ -1374,19 +1428,19 @@ __device__ T circular_L(const Model &m, const Cst<T> &k, const LcTable<T> *lcE, 
         // so E_c(R) = E may have no root below phi(0) and is not smooth: Lc(E) by plain
         // bisection, from [0, 1] doubled until it brackets the root (no circular orbit
         // below E_c(0) = phi(0)).
-        if (!(E > circ_energy<T, SCF>(m, k, T(0)))) return T(0);
+        T v = T(0);
+        if (!(E > scf_circ(m, k, T(0), v))) return T(0);
         T hi = T(1), lo = T(0);
-        while (hi < T(1e15) && circ_energy<T, SCF>(m, k, hi) <= E) hi *= T(2);
+        while (hi < T(1e15) && scf_circ(m, k, hi, v) <= E) hi *= T(2);
         for (int it = 0; it < 400; ++it) {
             const T mid = T(0.5) * (lo + hi);
             if (!(mid > lo) || !(mid < hi)) break;
-            if (circ_energy<T, SCF>(m, k, mid) <= E) lo = mid;
+            if (scf_circ(m, k, mid, v) <= E) lo = mid;
             else hi = mid;
         }
         R = T(0.5) * (lo + hi);
-        T vc2, phi;
-        circ_terms<T, SCF>(m, k, R, vc2, phi);
-        return R * d_sqrt(vc2);
+        scf_circ(m, k, R, v);
+        return R * d_sqrt(v);
     }
     if (!(E > T(__ldg(lcE)))) {
         R = k.lc_r0;
@@ -1965,6 +2019,29 @@ __device__ void scf_finalize(const Model &m, const Buffers &b, double s_ren, int
         }
     }
     __syncthreads();
+    // the x axis (see scf_circ): R_lm(R, 0, 0) = N_lm T_lm(0, R^2) R^m = c_lm R^l for m >= 0, 0 for m < 0
+    const int L = m.scf_lmax;
+    double *axis = m.scf_tab + size_t(n + 1) * nlm * 2;
+    for (int q = threadIdx.x; q < (n + 1) * (L + 1); q += blockDim.x) {
+        const int j = q / (L + 1), l = q % (L + 1);
+        double A = 0.0, B = 0.0, dfac = 1.0;
+        for (int mm = 0; mm <= l; ++mm) {
+            double t0 = 0.0, t1 = dfac;  // T_(q-1), T_q at z = 0, r^2 = 1, from q = mm
+            for (int i = mm + 1; i <= l; ++i) {
+                const double t2 = -double(i + mm - 1) * t0 / double(i - mm);
+                t0 = t1;
+                t1 = t2;
+            }
+            const int idx = l * (l + 1) + mm;
+            const double *tab = m.scf_tab + (size_t(j) * nlm + idx) * 2;
+            A += tab[0] * m.scf_norm[idx] * t1;
+            B += tab[1] * m.scf_norm[idx] * t1;
+            dfac *= double(2 * mm + 1);
+        }
+        axis[2 * q] = A;
+        axis[2 * q + 1] = B;
+    }
+    __syncthreads();
 }
 
 // update steps, and clears the sums for the next step. red: blockDim doubles.
@@ -2036,7 +2113,8 @@ __device__ void window_priors(const Model &m, const Buffers &b, long long *hist,
 }
 
 // The head of step t + 1, from the scalars after step t (one thread).
-__device__ __forceinline__ StepHead next_head(const Model &m, long long t, int pending, double s_ren, double what)
+__device__ __forceinline__ StepHead next_head(const Model &m, long long t, int pending, double s_ren, double what,
+                                              int fresh = 1)
 {
     StepHead h;
     const bool update = (t % m.update_every) == 0;  // step t + 1 is one of 1, 1 + P, ...
@@ -2045,7 +2123,7 @@ __device__ __forceinline__ StepHead next_head(const Model &m, long long t, int p
     h.scf_step = m.pot == 3 && update;
     h.wscale = float(s_ren);
     h.iwhat = what > 0.0 ? float(1.0 / what) : 0.f;
-    h.pad = 0;
+    h.fresh = fresh;
     h.lwscale = log(s_ren);
     h.lwhat = what > 0.0 ? log(what) : -HUGE_VAL;
     return h;
@@ -2167,14 +2245,14 @@ __device__ __forceinline__ double fin_chi2(const double *csum, int n)
 
 // The scalars after the step and the head of the next one (one thread).
 __device__ __forceinline__ void fin_scalars(const Model &m, const Buffers &b, long long n, int init, int prior_step,
-                                            double s_ren, double U)
+                                            int scf_step, double s_ren, double U)
 {
     Scalars &sc = *b.sc;
     const long long t = init ? 0 : __ldcg(&sc.t) + 1;
     const double what = init ? (n > 0 ? U / double(n) : 0.0) : __ldcg(&sc.what_flat);
     // the integer sums wrap beyond their range: the floating-point check sum catches it
     if (!(__ldcg(&sc.Wcheck) <= 0.5 * __ldcg(&sc.Wrange))) atomicOr(&sc.err, kErrOverflow);
-    const StepHead h = next_head(m, t, init ? 0 : (t > m.n_relax ? 1 : 0), s_ren, what);
+    const StepHead h = next_head(m, t, init ? 0 : (t > m.n_relax ? 1 : 0), s_ren, what, scf_step);
     if (init) {
         sc.W0 = U;
         sc.what_flat = what;
@@ -2230,7 +2308,7 @@ __device__ void finalize_block(const Model &m, const Buffers &b, long long n, in
     fin_observables<WPS>(m, b, b.hist, 0, pl.n_chunks, init, W0, cs, csum, s_ren);
     __syncthreads();
     if (int(threadIdx.x) == int(blockDim.x) - 32)
-        fin_scalars(m, b, n, init, prior_step, s_ren, total_weight<WPS>(m, b.hist));
+        fin_scalars(m, b, n, init, prior_step, scf_step, s_ren, total_weight<WPS>(m, b.hist));
     if (threadIdx.x < 32) {
         const double chi2 = fin_chi2<false>(csum, pl.n_chunks);
         if (threadIdx.x == 0) b.sc->chi2 = chi2;
@@ -2308,7 +2386,7 @@ __device__ __forceinline__ void global_add(long long *hist, int slot, float v, f
 // Per-step flags of one fit, read from its scalars at the start of the step.
 template <class T>
 struct StepFlags {
-    int pending, prior_step, scf_step;
+    int pending, prior_step, scf_step, fresh;
     T wscale, lwscale, iwhat_flat;
 };
 
@@ -2321,6 +2399,7 @@ __device__ __forceinline__ StepFlags<T> step_flags(const Model &m, const StepHea
     f.prior_step = init ? 0 : h.prior_step;
     // the self-consistent potential is rebuilt at the load and on the prior schedule
     f.scf_step = init ? m.pot == 3 : h.scf_step;
+    f.fresh = h.fresh;
     if constexpr (kLogWeights<T>) {
         f.wscale = T(1);
         f.lwscale = init ? T(0) : T(h.lwscale);
@@ -2421,8 +2500,23 @@ __device__ __forceinline__ void step_particles(const Model &m, const Model &mh, 
                 fa = accel_factor(mh, k, x, y, z, tb.ln);
             }
             P.fa[i] = fa;
+        } else if (kScf && mh.pot == 3) {
+            if (push) {
+                T ax, ay, az;
+                if (f.fresh) {
+                    accel<T, kScf>(mh, k, x, y, z, ax, ay, az);
+                } else {
+                    ax = P.ax[i];
+                    ay = P.ay[i];
+                    az = P.az[i];
+                }
+                leapfrog_scf(mh, k, x, y, z, vx, vy, vz, ax, ay, az);
+                P.ax[i] = ax;
+                P.ay[i] = ay;
+                P.az[i] = az;
+            }
         } else {
-            if (push) leapfrog<T, kScf>(mh, k, x, y, z, vx, vy, vz);
+            if (push) leapfrog<T>(mh, k, x, y, z, vx, vy, vz);
         }
         if (!is_zero(w)) {
             T Y, vlos;
@@ -2435,7 +2529,7 @@ __device__ __forceinline__ void step_particles(const Model &m, const Model &mh, 
                 constexpr unsigned M = decltype(Pl)::mask;
                 const GroupDesc &G = mh.g[g];
                 if (GP<M>::shells(G)) {  // never cached; never in the global-deposit kernel
-                    shell_kernels(G, tb, x, y, z, w, [&](int j, T v, int, int) {
+                    shell_kernels(mh, g, tb, x, y, z, w, [&](int j, T v, int, int) {
                         if constexpr (GA) global_add(b.hist, j, v, k.fx_gh);
                         else Acc<T>::add(S.h, j, v, k.fx_gh);
                     });
@@ -2647,7 +2741,7 @@ __global__ void __launch_bounds__(256) k_finalize(const Model m, const Buffers b
                 b.sc->Wcheck = double(b.hist[m.hist_words]) * (b.sc->Wrange * kRangeUnit);
                 b.hist[m.hist_words] = 0;
             }
-            fin_scalars(m, b, n, init, f.prior_step, s_ren, total_weight<WPS>(m, b.hist));
+            fin_scalars(m, b, n, init, f.prior_step, f.scf_step, s_ren, total_weight<WPS>(m, b.hist));
         }
     }
     if (f.scf_step) {
