@@ -41,21 +41,58 @@ struct SphBins {
     double r_min, r_max, ln_rmin, ln_span;  // ln(r_max) - ln(r_min)
 };
 
+// The integer part of an FP32 estimate of a bin coordinate whose error is below `err`, or
+// kUnsure where the error could carry it over a bin's edge.
+constexpr int kUnsure = -0x7fffffff;
+__device__ __forceinline__ int sure_floor(float f, float err)
+{
+    const float k = floorf(f);
+    return (f - k > err && f - k < 1.f - err) ? int(k) : kUnsure;
+}
+
+// Every bin is decided in FP64: FP32 gives the bin coordinate to within 1e-5 of the number of
+// bins (logf, atan2f and the conversions of x, y, z are good to a few 1e-7 of it), and only where
+// that leaves an edge in doubt are the FP64 functions evaluated (a few particles in a thousand; they
+// take some 150 FP64 instructions, 16 cycles each).
 __device__ int sph_bin(const SphBins &g, double x, double y, double z)
 {
-    const double r = sqrt(x * x + y * y + z * z);
-    if (!(r < g.r_max)) return -1;
-    int ir = 0;
-    if (r >= g.r_min) {
-        const double f = (log(r) - g.ln_rmin) / g.ln_span;
-        ir = 1 + int(floor(f * (g.n_r - 1)));
-        if (ir > g.n_r - 1) ir = g.n_r - 1;
+    const double r2 = x * x + y * y + z * z;
+    const bool sane = big_range(r2) && r2 > 1e-30 && r2 < 1e30;
+    const float xf = float(x), yf = float(y), zf = float(z), rf = sqrtf(float(r2));
+    const float rmax = float(g.r_max), rmin = float(g.r_min);
+    int ir = kUnsure, ic = kUnsure, ip = kUnsure;
+    if (sane && rf > 1.0001f * rmax) return -1;
+    if (sane && rf < 0.9999f * rmax) {
+        if (rf < 0.9999f * rmin) ir = 0;
+        else if (rf > 1.0001f * rmin) {
+            const float f = (logf(rf) - float(g.ln_rmin)) / float(g.ln_span) * float(g.n_r - 1);
+            const int k = sure_floor(f, 1e-5f * float(g.n_r) * (1.f + (fabsf(float(g.ln_rmin)) + 30.f) / float(g.ln_span) * 0.1f));
+            if (k != kUnsure) ir = 1 + k > g.n_r - 1 ? g.n_r - 1 : 1 + k;
+        }
+        ic = sure_floor((zf / rf + 1.f) * 0.5f * float(g.n_ct), 1e-5f * float(g.n_ct));
+        if (fabsf(xf) + fabsf(yf) > 1e-15f)
+            ip = sure_floor((atan2f(yf, xf) + 3.14159265f) * 0.159154943f * float(g.n_phi), 1e-5f * float(g.n_phi));
     }
-    const double ct = r > 0.0 ? z / r : 1.0;
-    int ic = int(floor((ct + 1.0) * 0.5 * g.n_ct));
+    if (ir == kUnsure) {
+        const double r = sqrt(r2);
+        if (!(r < g.r_max)) return -1;
+        ir = 0;
+        if (r >= g.r_min) {
+            const double f = (log(r) - g.ln_rmin) / g.ln_span;
+            ir = 1 + int(floor(f * (g.n_r - 1)));
+            if (ir > g.n_r - 1) ir = g.n_r - 1;
+        }
+    }
+    if (ic == kUnsure) {
+        const double r = sqrt(r2);
+        const double ct = r > 0.0 ? z / r : 1.0;
+        ic = int(floor((ct + 1.0) * 0.5 * g.n_ct));
+    }
     ic = ic < 0 ? 0 : (ic > g.n_ct - 1 ? g.n_ct - 1 : ic);
-    const double ph = atan2(y, x);
-    int ip = int(floor((ph + 3.14159265358979323846) / (2.0 * 3.14159265358979323846) * g.n_phi));
+    if (ip == kUnsure) {
+        const double ph = atan2(y, x);
+        ip = int(floor((ph + 3.14159265358979323846) / (2.0 * 3.14159265358979323846) * g.n_phi));
+    }
     ip = ip < 0 ? 0 : (ip > g.n_phi - 1 ? g.n_phi - 1 : ip);
     return (ir * g.n_ct + ic) * g.n_phi + ip;
 }
@@ -63,10 +100,10 @@ __device__ int sph_bin(const SphBins &g, double x, double y, double z)
 // v along e_r, e_theta, e_phi; phi = 0 on the z axis and e_r = e_z at the centre.
 __device__ void sph_velocity(double x, double y, double z, double vx, double vy, double vz, double v[3])
 {
-    const double R = sqrt(x * x + y * y);
-    const double r = sqrt(R * R + z * z);
-    const double cp = R > 0.0 ? x / R : 1.0, sp = R > 0.0 ? y / R : 0.0;
-    const double ct = r > 0.0 ? z / r : 1.0, st = r > 0.0 ? R / r : 0.0;
+    const double R = sqrt_int(x * x + y * y);
+    const double r = sqrt_int(R * R + z * z);
+    const double cp = R > 0.0 ? div_int(x, R) : 1.0, sp = R > 0.0 ? div_int(y, R) : 0.0;
+    const double ct = r > 0.0 ? div_int(z, r) : 1.0, st = r > 0.0 ? div_int(R, r) : 0.0;
     v[0] = vx * st * cp + vy * st * sp + vz * ct;
     v[1] = vx * ct * cp + vy * ct * sp - vz * st;
     v[2] = -vx * sp + vy * cp;
@@ -85,15 +122,53 @@ struct DiagScales {
     double w, wv, wv2, dev;
 };
 
-// Adds v to the two-word fixed-point sum at h[0], h[1].
-__device__ __forceinline__ void fx_add(long long *h, double v, double scale)
-{
-    if (v == 0.0) return;
-    long long hi, lo;
-    fx2(v, scale, hi, lo);
-    red_add(h, hi);
-    if (lo) red_add(h + 1, lo);
-}
+// The sums of a binning kernel: SH: in the block's shared memory (three 32-bit words a sum and
+// one a count, Acc<double>), added to the global two-word sums once per block at the end;
+// otherwise added to those directly. A few hundred bins share out millions of particles, and the
+// memory system adds to one address at a time: 2M particles took 3 ms in two grids of 672 and
+// 300 bins that way.
+template <bool SH>
+struct BinSums {
+    unsigned *h;
+    long long *sums;
+    unsigned long long *counts;
+    int n_sums, n_counts;
+    __device__ BinSums(unsigned char *smem, long long *s, unsigned long long *c, long long ns, long long nc)
+        : h(reinterpret_cast<unsigned *>(smem)), sums(s), counts(c), n_sums(int(ns)), n_counts(int(nc))
+    {
+        if (!SH) return;
+        for (int q = threadIdx.x; q < 3 * n_sums + n_counts; q += blockDim.x) h[q] = 0;
+        __syncthreads();
+    }
+    __device__ __forceinline__ void add(long long slot, double v, double scale)
+    {
+        if (SH) {
+            Acc<double>::add(h, int(slot), v, scale);
+            return;
+        }
+        if (v == 0.0) return;
+        long long hi, lo;
+        fx2(v, scale, hi, lo);
+        red_add(sums + 2 * slot, hi);
+        if (lo) red_add(sums + 2 * slot + 1, lo);
+    }
+    __device__ __forceinline__ void count(long long slot)
+    {
+        if (SH) atomicAdd(h + 3 * n_sums + slot, 1u);
+        else atomicAdd(counts + slot, 1ull);
+    }
+    __device__ void flush()
+    {
+        if (!SH) return;
+        __syncthreads();
+        for (int q = threadIdx.x; q < 2 * n_sums; q += blockDim.x) {
+            const long long v = Acc<double>::word(h, q >> 1, q & 1);
+            if (v != 0) red_add(sums + q, v);
+        }
+        for (int q = threadIdx.x; q < n_counts; q += blockDim.x)
+            if (h[3 * n_sums + q]) atomicAdd(counts + q, static_cast<unsigned long long>(h[3 * n_sums + q]));
+    }
+};
 
 // Largest |w| and |v|^2 (as ordered bit patterns of non-negative doubles) and a flag for
 // non-finite input.
@@ -127,10 +202,13 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag_stats(const Particles<T> 
 }
 
 // Per bin: sum w; sum w v_c; sum w v_c^2 (c = r, theta, phi), each two int64 words.
-template <class T>
+template <class T, bool SH>
 __global__ void __launch_bounds__(kDiagThreads) k_kin_sums(const SphBins g, const Particles<T> p, DiagScales sc,
                                                            long long *sums, unsigned long long *counts)
 {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const long long nb = (long long)g.n_r * g.n_ct * g.n_phi;
+    BinSums<SH> S(smem, sums, counts, nb * kKinSums, nb);
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < p.n;
          i += (long long)gridDim.x * blockDim.x) {
         const double x = double(p.x[i]), y = double(p.y[i]), z = double(p.z[i]);
@@ -139,30 +217,34 @@ __global__ void __launch_bounds__(kDiagThreads) k_kin_sums(const SphBins g, cons
         double v[3];
         sph_velocity(x, y, z, double(p.vx[i]), double(p.vy[i]), double(p.vz[i]), v);
         const double w = p.w[i];
-        long long *o = sums + (long long)b * (2 * kKinSums);
-        fx_add(o, w, sc.w);
+        const long long o = (long long)b * kKinSums;
+        S.add(o, w, sc.w);
         for (int c = 0; c < 3; ++c) {
-            fx_add(o + 2 * (1 + c), w * v[c], sc.wv);
-            fx_add(o + 2 * (4 + c), w * v[c] * v[c], sc.wv2);
+            S.add(o + 1 + c, w * v[c], sc.wv);
+            S.add(o + 4 + c, w * v[c] * v[c], sc.wv2);
         }
-        atomicAdd(counts + b, 1ull);
+        S.count(b);
     }
+    S.flush();
 }
 
 // First pass over the (E, x) grid: each particle's cell, the cell's weight and count.
-template <class T>
+template <class T, bool SH>
 __global__ void __launch_bounds__(kDiagThreads) k_grid_sums(const Model m, const Cst<double> k, const double *lcE,
                                                             const Particles<T> p, DiagScales sc, FnTables fn, int *cell,
                                                             long long *wsum, unsigned long long *counts)
 {
+    extern __shared__ __align__(16) unsigned char smem[];
+    BinSums<SH> S(smem, wsum, counts, m.ncell, m.ncell);
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < p.n;
          i += (long long)gridDim.x * blockDim.x) {
         const int c = prior_cell<double>(m, k, lcE, double(p.x[i]), double(p.y[i]), double(p.z[i]),
                                          double(p.vx[i]), double(p.vy[i]), double(p.vz[i]), fn);
         cell[i] = c;
-        fx_add(wsum + 2 * c, p.w[i], sc.w);
-        atomicAdd(counts + c, 1ull);
+        S.add(c, p.w[i], sc.w);
+        S.count(c);
     }
+    S.flush();
 }
 
 // Value of a two-word fixed-point sum.
@@ -172,16 +254,27 @@ __host__ __device__ inline double fx_value(const long long *h, double scale)
 }
 
 // Second pass: squared deviations from the cell means (the means from the exact sums).
-__global__ void __launch_bounds__(kDiagThreads) k_grid_dev(long long n, const int *cell, const double *w,
+template <bool SH>
+__global__ void __launch_bounds__(kDiagThreads) k_grid_dev(long long n, int ncell, const int *cell, const double *w,
                                                            const long long *wsum, const unsigned long long *counts,
                                                            DiagScales sc, long long *wdev2)
 {
+    extern __shared__ __align__(16) unsigned char smem[];
+    BinSums<SH> S(smem, wdev2, nullptr, ncell, 0);
+    // the means once per block, behind the sums (8-byte aligned: 12 ncell rounded up)
+    double *mean = reinterpret_cast<double *>(smem + (12 * size_t(ncell) + 7) / 8 * 8);
+    if (SH) {
+        for (int c = threadIdx.x; c < ncell; c += blockDim.x)
+            mean[c] = counts[c] ? fx_value(wsum + 2 * c, sc.w) / double(counts[c]) : 0.0;
+        __syncthreads();
+    }
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
         const int c = cell[i];
-        const double d = w[i] - fx_value(wsum + 2 * c, sc.w) / double(counts[c]);
-        fx_add(wdev2 + 2 * c, d * d, sc.dev);
+        const double d = w[i] - (SH ? mean[c] : fx_value(wsum + 2 * c, sc.w) / double(counts[c]));
+        S.add(c, d * d, sc.dev);
     }
+    S.flush();
 }
 
 // Device copies of the particles the diagnostics bin, and the scratch they need; freed on
@@ -244,6 +337,25 @@ m2m_status source(m2m_ctx *ctx, int64_t n, const double *pos, const double *vel,
     }
     src.kind = 0;
     src.d = {d, d + n, d + 2 * n, d + 3 * n, d + 4 * n, d + 5 * n, d + 6 * n, n};
+    return M2M_OK;
+}
+
+// Launches a binning kernel: the block-shared form where its `bytes` fit a block (fit: the form
+// in shared memory, else the other), blocks for every SM, or fewer for few particles.
+template <class K, class... A>
+m2m_status bin_launch(m2m_ctx *ctx, K shared, K global, size_t bytes, long long n, A... args)
+{
+    int maxsm = 0;
+    CU(cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
+    const bool sh = bytes <= size_t(maxsm);
+    K fn = sh ? shared : global;
+    if (!sh) bytes = 0;
+    CU(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes)));
+    int occ = 0;
+    CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kDiagThreads, bytes));
+    const long long want = (n + kDiagThreads - 1) / kDiagThreads, cap = (long long)ctx->nsm * (occ > 0 ? occ : 1);
+    fn<<<int(want < 1 ? 1 : (want < cap ? want : cap)), kDiagThreads, bytes, ctx->stream>>>(args...);
+    CU(cudaGetLastError());
     return M2M_OK;
 }
 
@@ -324,9 +436,12 @@ extern "C" m2m_status m2m_diag_kinematics(m2m_ctx *ctx, const m2m_sph_grid *grid
     const SphBins g{grid->n_r, grid->n_phi, grid->n_ct, grid->r_min, grid->r_max, std::log(grid->r_min),
                     std::log(grid->r_max) - std::log(grid->r_min)};
     if (np > 0) {
-        if (src.kind == 2) k_kin_sums<float><<<grid_of(ctx, np), kDiagThreads, 0, ctx->stream>>>(g, src.f, sc, d_sums, d_cnt);
-        else k_kin_sums<double><<<grid_of(ctx, np), kDiagThreads, 0, ctx->stream>>>(g, src.d, sc, d_sums, d_cnt);
-        CU(cudaGetLastError());
+        const size_t bytes = size_t(nb) * (3 * kKinSums + 1) * sizeof(int);
+        s = src.kind == 2 ? bin_launch(ctx, k_kin_sums<float, true>, k_kin_sums<float, false>, bytes, np, g, src.f, sc,
+                                       d_sums, d_cnt)
+                          : bin_launch(ctx, k_kin_sums<double, true>, k_kin_sums<double, false>, bytes, np, g, src.d, sc,
+                                       d_sums, d_cnt);
+        if (s != M2M_OK) return s;
     }
     std::vector<long long> hs(size_t(nb) * 2 * kKinSums);
     CU(cudaMemcpyAsync(hs.data(), d_sums, sizeof(long long) * hs.size(), cudaMemcpyDeviceToHost, ctx->stream));
@@ -382,15 +497,16 @@ extern "C" m2m_status m2m_diag_grid(m2m_ctx *ctx, const m2m_prior_grid *grid, in
         CU(cudaMemcpyAsync(d_fn, tab.data(), sizeof(u64) * tab.size(), cudaMemcpyHostToDevice, ctx->stream));
         const FnTables fn{d_fn, m.pot < 2 ? d_fn + kExpEntries : nullptr};
         m.int_force = int_force_ok(m);
-        const int gr = grid_of(ctx, np);
-        if (src.kind == 2) {
-            k_grid_sums<float><<<gr, kDiagThreads, 0, ctx->stream>>>(m, kd, ctx->d_lcE, src.f, sc, fn, d_cell, d_ws, d_cnt);
-            k_grid_dev<<<gr, kDiagThreads, 0, ctx->stream>>>(np, d_cell, src.f.w, d_ws, d_cnt, sc, d_wd);
-        } else {
-            k_grid_sums<double><<<gr, kDiagThreads, 0, ctx->stream>>>(m, kd, ctx->d_lcE, src.d, sc, fn, d_cell, d_ws, d_cnt);
-            k_grid_dev<<<gr, kDiagThreads, 0, ctx->stream>>>(np, d_cell, src.d.w, d_ws, d_cnt, sc, d_wd);
-        }
-        CU(cudaGetLastError());
+        const size_t bytes = size_t(ncell) * 4 * sizeof(int), dev = (size_t(ncell) * 12 + 7) / 8 * 8 + size_t(ncell) * 8;
+        s = src.kind == 2 ? bin_launch(ctx, k_grid_sums<float, true>, k_grid_sums<float, false>, bytes, np, m, kd,
+                                       static_cast<const double *>(ctx->d_lcE), src.f, sc, fn, d_cell, d_ws, d_cnt)
+                          : bin_launch(ctx, k_grid_sums<double, true>, k_grid_sums<double, false>, bytes, np, m, kd,
+                                       static_cast<const double *>(ctx->d_lcE), src.d, sc, fn, d_cell, d_ws, d_cnt);
+        if (s != M2M_OK) return s;
+        s = bin_launch(ctx, k_grid_dev<true>, k_grid_dev<false>, dev, np, np, int(ncell),
+                       static_cast<const int *>(d_cell), src.kind == 2 ? src.f.w : src.d.w,
+                       static_cast<const long long *>(d_ws), static_cast<const unsigned long long *>(d_cnt), sc, d_wd);
+        if (s != M2M_OK) return s;
     }
     std::vector<long long> hw(size_t(ncell) * 2), hd(size_t(ncell) * 2);
     CU(cudaMemcpyAsync(hw.data(), d_ws, sizeof(long long) * hw.size(), cudaMemcpyDeviceToHost, ctx->stream));

@@ -116,3 +116,42 @@ def test_many_steps_per_launch_are_the_same_steps(name, targets):
     _same(_read(one), _read(other))
     for f in (one, many, other):
         f.close()
+
+
+@pytest.mark.parametrize("grid", [dict(n_r=21, n_phi=8, n_ct=4, r_min=0.05, r_max=20.0),   # sums of a block in shared memory
+                                  dict(n_r=30, n_phi=12, n_ct=12, r_min=1e-3, r_max=1e3),  # beyond it
+                                  dict(n_r=2, n_phi=1, n_ct=1, r_min=1.0, r_max=1.0 + 1e-6)])
+def test_kinematic_bins_beside_their_edges(grid, targets):
+    """Counts and sums of 20,000 particles and of points 1e-9 to either side of every kind of bin
+    edge, where FP32 cannot decide: the oracle's."""
+    from paper_1202_2355_gb300 import synth
+    p = synth.realise_spherical(3, 20_000, W.hernquist_sigma2)
+    r_edges = np.concatenate([[grid["r_min"]], np.exp(np.linspace(math.log(grid["r_min"]), math.log(grid["r_max"]), grid["n_r"]))])
+    rng = np.random.default_rng(5)
+    ext = {k: [] for k in p}
+    for side in (1 - 1e-9, 1 + 1e-9):
+        for r in r_edges * side:
+            for _ in range(3):
+                d = rng.normal(size=3)
+                d *= r / np.linalg.norm(d)
+                for k, v in zip("xyz", d):
+                    ext[k].append(v)
+        for i in range(grid["n_phi"]):
+            ph, z = (-math.pi + 2 * math.pi * (i + 0.5 * (side - 1)) / grid["n_phi"]) * 1.0 + (side - 1), rng.normal()
+            for k, v in zip("xyz", (0.3 * math.cos(ph), 0.3 * math.sin(ph), z)):
+                ext[k].append(v)
+        for i in range(1, grid["n_ct"]):
+            ct = -1 + 2 * i / grid["n_ct"] + (side - 1)
+            for k, v in zip("xyz", (0.5 * math.sqrt(1 - ct * ct), 0.1 * side, 0.51 * ct / max(1e-9, 1.0))):
+                ext[k].append(v)
+    m = len(ext["x"])
+    for k in ("vx", "vy", "vz"):
+        ext[k] = list(rng.normal(size=m))
+    ext["w"] = [1e-5] * m
+    q = {k: np.concatenate([p[k], np.asarray(ext[k])]) for k in p}
+    f = _fit(dict(wl="c1", n=10), targets)
+    s, c = f.diag_kinematics(grid, particles=q)
+    so, co = O.kin_sums(grid, O.ParticleSet(q))
+    f.close()
+    assert np.array_equal(c, co)
+    assert np.all(np.abs(s - so) <= 1e-12 * (np.abs(so).max(axis=0) + 1e-300))
