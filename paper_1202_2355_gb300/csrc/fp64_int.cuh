@@ -210,6 +210,21 @@ __host__ __device__ __forceinline__ Big big_norm(Big a)
     return a;
 }
 
+// a b: the high half of the product of the significands, rounded to nearest; zeros, subnormal or
+// non-finite factors and results near the ends of the range take the FP64 instruction.
+__host__ __device__ __forceinline__ double mul_int(double a, double b)
+{
+    const u64 x = u64(bits_of(a)), y = u64(bits_of(b));
+    const unsigned ex = unsigned(x >> 52) & 0x7ffu, ey = unsigned(y >> 52) & 0x7ffu, e = ex + ey;
+    // ex, ey >= 1 and e - 1023 within 1 .. 2045: both normal, the product too
+    if (ex - 1u >= 2046u || ey - 1u >= 2046u || e - 1024u >= 2044u) return a * b;
+    const u64 m = mulhi_u((x << 11) | (1ull << 63), ((y << 11) | (1ull << 63)));
+    const unsigned up = unsigned(m >> 63);
+    const u64 n = up ? m : m << 1;  // the bit shifted in is below the rounding
+    const u64 r = (n >> 11) + ((n >> 10) & 1);
+    return of_bits(i64((r + (u64(e - 1023u - 1u + up) << 52)) | ((x ^ y) & (1ull << 63))));
+}
+
 // ---------------------------------------------------------------- exp
 //
 // x = N ln2/256 + r, N = 256 e + j, |r| < ln2/512 (1 + 2^-4); exp(x) = 2^e 2^(j/256) (1 + p(r)),

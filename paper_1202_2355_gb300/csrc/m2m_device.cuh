@@ -787,25 +787,38 @@ __host__ __device__ __forceinline__ void accel(const Model &m, const Cst<T> &k, 
     accel_from(m, k, accel_factor(m, k, x, y, z), x, y, z, ax, ay, az);
 }
 
+// v += dt/2 a from the force factor. FP64 forms dt f/2 once (four FP64 instructions instead
+// of six; the spherical potentials, and x, y of the halo).
+__device__ __forceinline__ void kick(const Model &m, const Cst<float> &k, float f, float x, float y, float z, float &vx,
+                                     float &vy, float &vz)
+{
+    float ax, ay, az;
+    accel_from(m, k, f, x, y, z, ax, ay, az);
+    vx = fma(k.hdt, ax, vx);
+    vy = fma(k.hdt, ay, vy);
+    vz = fma(k.hdt, az, vz);
+}
+__device__ __forceinline__ void kick(const Model &m, const Cst<double> &k, double f, double x, double y, double z,
+                                     double &vx, double &vy, double &vz)
+{
+    const double h = m.pot == 2 ? k.hdt * f : -(k.hdt * f);
+    vx = fma(h, x, vx);
+    vy = fma(h, y, vy);
+    vz = fma(m.pot == 2 ? (m.int_force ? div_q2(k, h) : d_div(h, k.q2)) : h, z, vz);
+}
+
 // One kick-drift-kick leap-frog step from the force factor f at the start position;
 // returns the factor at the end position in f.
 template <class T>
 __device__ __forceinline__ void leapfrog_from(const Model &m, const Cst<T> &k, T &x, T &y, T &z, T &vx, T &vy, T &vz,
                                               T &f, const u64 *lnt)
 {
-    T ax, ay, az;
-    accel_from(m, k, f, x, y, z, ax, ay, az);
-    vx = fma(k.hdt, ax, vx);
-    vy = fma(k.hdt, ay, vy);
-    vz = fma(k.hdt, az, vz);
+    kick(m, k, f, x, y, z, vx, vy, vz);
     x = fma(k.dt, vx, x);
     y = fma(k.dt, vy, y);
     z = fma(k.dt, vz, z);
     f = accel_factor(m, k, x, y, z, lnt);
-    accel_from(m, k, f, x, y, z, ax, ay, az);
-    vx = fma(k.hdt, ax, vx);
-    vy = fma(k.hdt, ay, vy);
-    vz = fma(k.hdt, az, vz);
+    kick(m, k, f, x, y, z, vx, vy, vz);
 }
 
 // One kick-drift-kick leap-frog step.
@@ -841,6 +854,11 @@ __device__ __forceinline__ void leapfrog_scf(const Model &m, const Cst<T> &k, T 
 template <class T>
 __device__ __forceinline__ void project(const Cst<T> &k, T y, T z, T vy, T vz, T &Y, T &vlos)
 {
+    if (sizeof(T) == 8 && is_zero(k.sin_i) && k.cos_i == T(1)) {  // face on: the same values, no FP64 instruction
+        Y = y;
+        vlos = vz;
+        return;
+    }
     Y = fma(y, k.cos_i, -(z * k.sin_i));
     vlos = fma(vy, k.sin_i, vz * k.cos_i);
 }
@@ -985,6 +1003,10 @@ __device__ __forceinline__ T gh_poly(T t)
     return s;
 }
 
+// a b of the kernel values: in FP64 on the integer pipe (mul_int), correctly rounded up to ties.
+__device__ __forceinline__ float product(float a, float b) { return a * b; }
+__device__ __forceinline__ double product(double a, double b) { return mul_int(a, b); }
+
 // Emits emit(slot, w K_slot, class, kind index in the group) for every kernel of group G
 // at aperture p:
 // surface mass (K = 1), v_los^2 (vv), v_los, and the Gauss-Hermite b_n: c_n H_n(nu) as a
@@ -997,17 +1019,17 @@ __device__ __forceinline__ void group_kernels(const GroupDesc &G, const TB &tb, 
     using P = GP<M>;
     const int base = G.obs_off + p;
     if (P::mass(G)) emit(base + G.k_mass * G.n_ap, w, kClassMass, G.k_mass);
-    if (P::v2(G)) emit(base + G.k_v2 * G.n_ap, w * vv, kClassVel, G.k_v2);
+    if (P::v2(G)) emit(base + G.k_v2 * G.n_ap, product(w, vv), kClassVel, G.k_v2);
     if (P::v1(G)) emit(base + G.k_v1 * G.n_ap, w * vlos, kClassVel, G.k_v1);
     if (P::max_gh(G) >= 0) {
         const T nu = (vlos - tb.vp[G.ap_off + p]) * tb.isp[G.ap_off + p];
-        const T t = nu * nu;
+        const T t = product(nu, nu);
         const T ge = kexp_mhalf(tb, t);
         if (gexp_out) *gexp_out = ge;
-        const T we = w * ge, wo = we * nu;
+        const T we = product(w, ge), wo = product(we, nu);
         auto put = [&](auto N) {
             constexpr int n = decltype(N)::value;
-            if (P::gh(G, n)) emit(base + G.k_gh[n] * G.n_ap, gh_poly<n>(t) * (n % 2 ? wo : we), kClassGH, G.k_gh[n]);
+            if (P::gh(G, n)) emit(base + G.k_gh[n] * G.n_ap, product(gh_poly<n>(t), n % 2 ? wo : we), kClassGH, G.k_gh[n]);
         };
         put(std::integral_constant<int, 0>{});
         put(std::integral_constant<int, 1>{});
@@ -2539,7 +2561,7 @@ __device__ __forceinline__ void step_particles(const Model &m, const Model &mh, 
                 if (cache) code_out = ap_encode(mh, code_out, g, p);
                 if (p >= 0) {
                     // the v^2 sums' range assumes v^2 <= v2max (energy bound with headroom)
-                    const T vv = vlos * vlos;
+                    const T vv = product(vlos, vlos);
                     if (GP<M>::v2(G) && gt_nonneg(vv, k.v2max)) err |= kErrOverflow;
                     group_kernels<M>(
                         G, tb, p, vlos, vv, w,
