@@ -44,10 +44,14 @@ __host__ __device__ __forceinline__ int mulhi_s32(int a, int b)
     return int((i64(a) * b) >> 32);
 #endif
 }
+// The bits of a double and back, opaque to the compiler's front end: it would turn integer tests
+// of them into FP64 comparisons and sign changes into FP64 arithmetic.
 __host__ __device__ __forceinline__ i64 bits_of(double x)
 {
 #ifdef __CUDA_ARCH__
-    return __double_as_longlong(x);
+    i64 b;
+    asm("mov.b64 %0, %1;" : "=l"(b) : "d"(x));
+    return b;
 #else
     i64 b;
     std::memcpy(&b, &x, 8);
@@ -57,7 +61,9 @@ __host__ __device__ __forceinline__ i64 bits_of(double x)
 __host__ __device__ __forceinline__ double of_bits(i64 b)
 {
 #ifdef __CUDA_ARCH__
-    return __longlong_as_double(b);
+    double x;
+    asm("mov.b64 %0, %1;" : "=d"(x) : "l"(b));
+    return x;
 #else
     double x;
     std::memcpy(&x, &b, 8);
@@ -100,6 +106,12 @@ __host__ __device__ __forceinline__ float seed_rcp(float x)
     return 1.f / x;
 #endif
 }
+
+// The FP64 product of factors out of mul_int's range. Not inlined: the compiler would compute one
+// FP64 instruction ahead of the test and select (it looks cheap, and is 16 cycles of the pipe).
+#ifdef __CUDACC__
+static __device__ __noinline__ double mul_far(double a, double b) { return a * b; }
+#endif
 
 // A positive number m 2^(e - 63) with the top bit of m set.
 struct Big {
@@ -217,7 +229,13 @@ __host__ __device__ __forceinline__ double mul_int(double a, double b)
     const u64 x = u64(bits_of(a)), y = u64(bits_of(b));
     const unsigned ex = unsigned(x >> 52) & 0x7ffu, ey = unsigned(y >> 52) & 0x7ffu, e = ex + ey;
     // ex, ey >= 1 and e - 1023 within 1 .. 2045: both normal, the product too
-    if (ex - 1u >= 2046u || ey - 1u >= 2046u || e - 1024u >= 2044u) return a * b;
+    if (ex - 1u >= 2046u || ey - 1u >= 2046u || e - 1024u >= 2044u) {
+#ifdef __CUDA_ARCH__
+        return mul_far(a, b);
+#else
+        return a * b;
+#endif
+    }
     const u64 m = mulhi_u((x << 11) | (1ull << 63), ((y << 11) | (1ull << 63)));
     const unsigned up = unsigned(m >> 63);
     const u64 n = up ? m : m << 1;  // the bit shifted in is below the rounding
@@ -277,9 +295,11 @@ __host__ __device__ __forceinline__ Big exp_big(double x, const u64 *t)
 // exp(x) in FP64: 0 below -707 (results under ~1e-307), +inf above 709, NaN propagates.
 __host__ __device__ __forceinline__ double exp_int(double x, const u64 *t)
 {
-    if ((bits_of(x) & 0x7fffffffffffffffll) >= 0x4086180000000000ll) {  // |x| >= 707, or NaN
-        if (!(x > -707.0)) return x != x ? x : 0.0;
-        if (x > 709.0) return of_bits(0x7ff0000000000000ll);
+    const i64 b = bits_of(x), p = b & 0x7fffffffffffffffll;
+    if (p >= 0x4086180000000000ll) {  // |x| >= 707, or NaN
+        if (p > 0x7ff0000000000000ll) return x;
+        if (b < 0) return 0.0;
+        if (p > 0x4086280000000000ll) return of_bits(0x7ff0000000000000ll);  // 709
     }
     return big_double(exp_big(x, t));
 }
@@ -289,7 +309,7 @@ __host__ __device__ __forceinline__ double exp_mhalf(double t, const u64 *tab)
 {
     const i64 b = bits_of(t);
     const double x = b > (64ll << 52) ? of_bits((b - (1ll << 52)) | i64(1ull << 63)) : 0.0;  // t < 2^-959 gives 1
-    return exp_int(t != t || b >= (2047ll << 52) ? -t : x, tab);
+    return exp_int(b >= (2047ll << 52) ? of_bits(b | i64(1ull << 63)) : x, tab);  // inf and NaN: negated
 }
 
 // ---------------------------------------------------------------- force factors

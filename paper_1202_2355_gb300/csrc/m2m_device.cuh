@@ -395,21 +395,19 @@ __host__ __device__ __forceinline__ double d_floor(double x) { return floor(x); 
 __host__ __device__ __forceinline__ bool is_zero(float v) { return v == 0.f; }
 __host__ __device__ __forceinline__ bool is_zero(double v)
 {
-#ifdef __CUDA_ARCH__
-    return (__double_as_longlong(v) << 1) == 0;  // +0 or -0
-#else
-    return v == 0.0;
-#endif
+    return (bits_of(v) << 1) == 0;  // +0 or -0
 }
+__host__ __device__ __forceinline__ bool is_one(float v) { return v == 1.f; }
+__host__ __device__ __forceinline__ bool is_one(double v) { return bits_of(v) == 0x3ff0000000000000ll; }
 // a > b for a, b >= 0 (FP64: a positive NaN counts as greater)
 __device__ __forceinline__ bool gt_nonneg(float a, float b) { return a > b; }
 __device__ __forceinline__ bool gt_nonneg(double a, double b)
 {
-    return __double_as_longlong(a) > __double_as_longlong(b);
+    return bits_of(a) > bits_of(b);
 }
 __device__ __forceinline__ bool is_neg_inf(double v)
 {
-    return __double_as_longlong(v) == static_cast<long long>(0xFFF0000000000000ull);
+    return bits_of(v) == static_cast<long long>(0xFFF0000000000000ull);
 }
 
 __host__ __device__ __forceinline__ bool d_finite(float x) { return isfinite(x); }
@@ -854,7 +852,7 @@ __device__ __forceinline__ void leapfrog_scf(const Model &m, const Cst<T> &k, T 
 template <class T>
 __device__ __forceinline__ void project(const Cst<T> &k, T y, T z, T vy, T vz, T &Y, T &vlos)
 {
-    if (sizeof(T) == 8 && is_zero(k.sin_i) && k.cos_i == T(1)) {  // face on: the same values, no FP64 instruction
+    if (sizeof(T) == 8 && is_zero(k.sin_i) && is_one(k.cos_i)) {  // face on: the same values, no FP64 instruction
         Y = y;
         vlos = vz;
         return;
@@ -888,24 +886,24 @@ __device__ __forceinline__ int aperture(const GroupDesc &G, const double *esq, c
 {
     if (!GP<M>::pixels(G)) {
         const double R2 = fma(X, X, Y * Y);
-        const long long r = __double_as_longlong(R2);
+        const long long r = bits_of(R2);
         const double *e = esq + G.edge_off;
-        if (r < __double_as_longlong(e[0]) || r >= __double_as_longlong(e[G.n_ap])) return -1;
+        if (r < bits_of(e[0]) || r >= bits_of(e[G.n_ap])) return -1;
         int p;
         if (G.lut_n > 0) {
             int b = __float2int_rd((__log2f(float_near(R2)) - G.l0) * G.lscale);
             b = b < 0 ? 0 : (b >= G.lut_n ? G.lut_n - 1 : b);
             p = G.lut_identity ? b : int(lut[G.lut_off + b]);
             // the candidate is right but within rounding of an edge or for crowded edges
-            if (r < __double_as_longlong(e[p]) || r >= __double_as_longlong(e[p + 1])) {
-                while (p > 0 && r < __double_as_longlong(e[p])) --p;
-                while (r >= __double_as_longlong(e[p + 1])) ++p;
+            if (r < bits_of(e[p]) || r >= bits_of(e[p + 1])) {
+                while (p > 0 && r < bits_of(e[p])) --p;
+                while (r >= bits_of(e[p + 1])) ++p;
             }
         } else {
             int lo = 0, hi = G.n_ap;  // e[lo] <= R^2 < e[hi]
             while (hi - lo > 1) {
                 const int mid = (lo + hi) >> 1;
-                if (__double_as_longlong(e[mid]) <= r) lo = mid;
+                if (bits_of(e[mid]) <= r) lo = mid;
                 else hi = mid;
             }
             p = lo;
@@ -1562,14 +1560,14 @@ __device__ __forceinline__ int prior_cell(const Model &m, const Cst<T> &k, const
 // high and low 32-bit parts. |v*scale| < 2^62 keeps k <= 42, so m 2^(k-32) < 2^63.
 __device__ __forceinline__ void fx2(double v, double scale, long long &hi, long long &lo)
 {
-    const long long bits = __double_as_longlong(v);
+    const long long bits = bits_of(v);
     const int e = int((bits >> 52) & 0x7FF);
     if (e == 0) {  // zero (and subnormals, below any resolution used here)
         hi = 0;
         lo = 0;
         return;
     }
-    const int se = int((__double_as_longlong(scale) >> 52) & 0x7FF) - 1023;
+    const int se = int((bits_of(scale) >> 52) & 0x7FF) - 1023;
     const unsigned long long m = (static_cast<unsigned long long>(bits) & 0xFFFFFFFFFFFFFull) | (1ull << 52);
     const int k = e - 1075 + se + 32;
     unsigned long long th, tl;
@@ -1832,7 +1830,7 @@ __device__ __forceinline__ T foc_update_log(const Model &m, const Cst<T> &k, con
         un = u + log1p(h);
     }
     // exp_tab overflows above 709 (NaN of either sign is flagged too)
-    const long long ub = __double_as_longlong(un);
+    const long long ub = bits_of(un);
     if ((ub & 0x7fffffffffffffffll) > 0x7ff0000000000000ll || ub > 0x4086280000000000ll) err |= kErrNonFinite;
     return un;
 }
