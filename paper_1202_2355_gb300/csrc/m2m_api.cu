@@ -1174,11 +1174,9 @@ extern "C" m2m_status m2m_step(m2m_ctx *ctx, int64_t nsteps)
     return M2M_OK;
 }
 
-m2m_status check_device_errors(m2m_ctx *ctx)
+// The error latched in a fit's scalars, as a status.
+static m2m_status scalar_errors(m2m_ctx *ctx, const Scalars &sc)
 {
-    Scalars sc;
-    CU(cudaMemcpyAsync(&sc, ctx->d_sc, sizeof sc, cudaMemcpyDeviceToHost, ctx->stream));
-    CU(cudaStreamSynchronize(ctx->stream));
     if (sc.err & kErrNegWeight) return fail(ctx, M2M_ERR_NEG_WEIGHT, "the force of change made a weight negative");
     if (sc.err & kErrOverflow) return fail(ctx, M2M_ERR_OVERFLOW, "a deposit left the fixed-point range");
     if (sc.err & kErrTimeout) return fail(ctx, M2M_ERR_TIMEOUT, "a bounded device wait expired");
@@ -1187,13 +1185,21 @@ m2m_status check_device_errors(m2m_ctx *ctx)
     return M2M_OK;
 }
 
+m2m_status check_device_errors(m2m_ctx *ctx)
+{
+    Scalars sc;
+    CU(cudaMemcpyAsync(&sc, ctx->d_sc, sizeof sc, cudaMemcpyDeviceToHost, ctx->stream));
+    CU(cudaStreamSynchronize(ctx->stream));
+    return scalar_errors(ctx, sc);
+}
+
 extern "C" m2m_status m2m_synchronize(m2m_ctx *ctx)
 {
     if (!ctx) return M2M_ERR_ARG;
     if (!ctx->sub.empty()) return batch_synchronize(ctx);
+    if (ctx->loaded) return check_device_errors(ctx);  // waits for the stream
     CU(cudaStreamSynchronize(ctx->stream));
-    if (!ctx->loaded) return M2M_OK;
-    return check_device_errors(ctx);
+    return M2M_OK;
 }
 
 // ------------------------------------------------------------------ getters
@@ -1441,7 +1447,10 @@ extern "C" m2m_status m2m_get_chi2(m2m_ctx *ctx, double *chi2, int32_t *J, doubl
     Scalars sc;
     CU(cudaMemcpyAsync(&sc, ctx->d_sc, sizeof sc, cudaMemcpyDeviceToHost, ctx->stream));
     if (delta) CU(cudaMemcpyAsync(delta, ctx->d_delta, sizeof(double) * ctx->m.J, cudaMemcpyDeviceToHost, ctx->stream));
-    m2m_status s = m2m_synchronize(ctx);
+    // the scalars hold the error word too: one copy and one wait (a fit watched step by step reads
+    // chi^2 after each: 50 us with the step, 3,001 FP64 particles, 39 so)
+    CU(cudaStreamSynchronize(ctx->stream));
+    const m2m_status s = scalar_errors(ctx, sc);
     if (chi2) *chi2 = sc.chi2;
     if (J) *J = ctx->m.J;
     return s;
