@@ -278,9 +278,9 @@ m2m_status m2m_get_step_count(m2m_ctx *ctx, int64_t *t);
 /* Number of particles currently loaded (0 before the first load). */
 m2m_status m2m_get_particle_count(m2m_ctx *ctx, int64_t *n);
 
-/* Kernel timing. While on, every step-kernel launch (one per step: the
- * finalize runs inside it) is bracketed by CUDA events recorded on the
- * context stream (graph replay is off), and m2m_get_timing returns their
+/* Kernel timing. While on, every step is launched by itself (its pass and its
+ * finalize; no graph replay and no several steps per launch) and bracketed by
+ * CUDA events recorded on the context stream, and m2m_get_timing returns their
  * summed device time in milliseconds and the number of steps timed since
  * timing was switched on. Either output pointer may be NULL. */
 m2m_status m2m_set_timing(m2m_ctx *ctx, int32_t on);

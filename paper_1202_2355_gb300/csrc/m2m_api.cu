@@ -2,10 +2,12 @@
 //
 // A context owns the particle state (structure of arrays in HBM), the
 // observable and prior tables, the fixed-point accumulators and a small block
-// of per-step scalars in device memory. A step is one kernel, k_step: one pass
-// over the particles, whose last block to finish runs the finalize over the
-// observables and prior cells. Every per-step decision is read from device
-// memory, so a chunk of steps is captured once in a CUDA graph and replayed.
+// of per-step scalars in device memory. A step is one pass over the particles and a finalize
+// over the observables and prior cells. Most fits run many steps per launch
+// (m2m_persist.cu). The others take one kernel per step, k_step, whose last block to
+// finish runs the finalize, or k_step and k_finalize for more than 16 chunks of observables;
+// every per-step decision is read from device memory, so a chunk of steps is captured once in
+// a CUDA graph and replayed.
 #include "m2m_ctx.h"
 
 #include <algorithm>
@@ -1159,7 +1161,12 @@ extern "C" m2m_status m2m_step(m2m_ctx *ctx, int64_t nsteps)
     }
     // two steps or more of a fit that can: one launch for many (a single step finalizes in its
     // last block, without a meeting)
-    if (nsteps > 1 && persist_fits(ctx)) return persist_steps(ctx, nsteps);
+    // (plain launches on a stream under capture, as ever)
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (nsteps > 1 && persist_fits(ctx)) {
+        CU(cudaStreamIsCapturing(ctx->stream, &capture));
+        if (capture == cudaStreamCaptureStatusNone) return persist_steps(ctx, nsteps);
+    }
     int64_t left = nsteps;
     if (left >= kGraphSteps && !ctx->graph) {
         m2m_status s = build_graph(ctx);

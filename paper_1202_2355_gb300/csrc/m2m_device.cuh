@@ -2352,7 +2352,8 @@ __device__ void finalize_block(const Model &m, const Buffers &b, long long n, in
 // sums, (d) on prior-update steps the (E, x) cell of every particle with per-cell
 // weight sums and counts. Blocks add their sums to the global sums with integer
 // atomics (exact, so order-independent); the last block to finish runs the
-// finalize. Nothing waits on another block.
+// finalize (or k_finalize follows). Nothing waits on another block here; k_steps, which runs
+// many steps per launch with the same functions, meets once or twice per step.
 //
 // GA (global deposit): for observable sets whose block sums or force-of-change
 // records do not fit in shared memory (e.g. 64 x 64 pixel maps of five moments),

@@ -206,8 +206,7 @@ m2m_status setup(m2m_ctx *ctx)
 
 // The launches of a device run one after another, whatever their streams: two kernels whose
 // blocks wait for their own kind must not share out the SMs between them. Each launch waits for
-// the event of the one before. (A stream under capture takes no part: its graph's launches are
-// ordered by whoever runs it.)
+// the event of the one before.
 struct Turn {
     std::mutex mu;
     cudaEvent_t ev = nullptr;
@@ -230,16 +229,13 @@ m2m_status run(m2m_ctx *ctx, int nsteps)
     const int grid = grid_for(ctx, ctx->steps_bps);
     int spread = (grid + ctx->nsm - 1) / ctx->nsm * b.plan.n_chunks > 8;
     void *args[] = {&m, &k, &P, &b, &h2, &g, &nsteps, &ctx->steps_own, &spread};
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    CU(cudaStreamIsCapturing(ctx->stream, &cap));
     Turn &t = turn_of(ctx->device);
     std::lock_guard<std::mutex> lock(t.mu);
-    const bool ordered = cap == cudaStreamCaptureStatusNone;
-    if (ordered && !t.ev) CU(cudaEventCreateWithFlags(&t.ev, cudaEventDisableTiming));
-    if (ordered) CU(cudaStreamWaitEvent(ctx->stream, t.ev, 0));
+    if (!t.ev) CU(cudaEventCreateWithFlags(&t.ev, cudaEventDisableTiming));
+    CU(cudaStreamWaitEvent(ctx->stream, t.ev, 0));
     CU(cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(ctx->ksteps), dim3(grid), dim3(ctx->block),
                                    args, ctx->smem_steps, ctx->stream));
-    if (ordered) CU(cudaEventRecord(t.ev, ctx->stream));
+    CU(cudaEventRecord(t.ev, ctx->stream));
     return M2M_OK;
 }
 

@@ -155,3 +155,42 @@ def test_kinematic_bins_beside_their_edges(grid, targets):
     f.close()
     assert np.array_equal(c, co)
     assert np.all(np.abs(s - so) <= 1e-12 * (np.abs(so).max(axis=0) + 1e-300))
+
+
+def test_steps_under_capture(targets):
+    """Steps captured into a graph on the caller's stream, replayed: the same steps."""
+    import torch
+    st = torch.cuda.Stream()
+    case = dict(CASES["c1"], kw=dict(stream=st.cuda_stream))
+    a, b = _fit(case, targets), _fit(CASES["c1"], targets)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=st):
+        a.step(3)
+    with torch.cuda.stream(st):
+        g.replay()
+        g.replay()
+    b.step(6)
+    _same(_read(a), _read(b))
+    a.close()
+    b.close()
+
+
+def test_fits_of_several_threads_take_turns(targets):
+    """Two threads step their own fits at the same time: the same bits as alone."""
+    import threading
+    names = ["c1", "nfw"]
+    alone = []
+    for n in names:
+        f = _fit(CASES[n], targets)
+        f.step(200)
+        alone.append(_read(f))
+        f.close()
+    fits = [_fit(CASES[n], targets) for n in names]
+    ts = [threading.Thread(target=lambda f=f: [f.step(20) for _ in range(10)]) for f in fits]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    for f, want in zip(fits, alone):
+        _same(_read(f), want)
+        f.close()
