@@ -59,8 +59,8 @@ FP64_PEAK_TFLOPS = 152 * 4 * 2.07e9 / 1e12
 #                 traffic for arithmetic (acceleration, apertures, exp(-nu^2/2));
 #   flops         FP64 flops the FP64 kernel executes (DFMA = 2, DADD/DMUL = 1: ncu
 #                 sm__sass_thread_inst_executed_op_{dfma,dadd,dmul}_pred_on.sum over
-#                 one step launch / N), including the iterative sqrt, division, log
-#                 and exp;
+#                 one step launch / N); its square root, divisions, exponentials and the
+#                 products of the kernel values run on the integer pipe and are not in it;
 #   method_flops  operations the method itself asks for per particle-step on the
 #                 1M-particle FP64 workload (an FMA counts 2; a square root, a division,
 #                 an exp or a log counts 1): push 31, projection 6, aperture radius 3,
@@ -70,7 +70,7 @@ KERNEL_FIGURES = {
     # method: 7 x 8 B read and written, cell 2 B = 114 B; design: read x..vz, ln w and the
     # force factor (64 B), prior cell, cached apertures and cached exp(-nu^2/2) (2 + 2 + 8 B);
     # write 64 + 2 + 8 B
-    "fp64": {"bytes": 114, "design_bytes": 150, "flops": 151.37, "method_flops": 88},
+    "fp64": {"bytes": 114, "design_bytes": 150, "flops": 60.72, "method_flops": 88},
     # method: 7 x 4 B read and written, cell 2 B = 58 B; design: read 6 coordinates + w
     # (28 B), prior cell and cached apertures (2 + 2 B); write 28 B + 2 B of apertures
     "mixed": {"bytes": 58, "design_bytes": 62, "flops": None},
@@ -85,7 +85,7 @@ ACCEL_BYTES_MIXED = 8
 # the capture); absent: not captured since the kernel last changed. c5: the 12-fit
 # subset of the batch (fits 0, 8, ..., 88), traffic scaled to a full launch by the
 # particle count; c2: the whole 1M-particle fit.
-DRAM_PER_UNIT = {("c5", "mixed"): (63.82, 8_384_798), ("c2", "fp64"): (89.77, 1_000_000)}
+DRAM_PER_UNIT = {("c5", "mixed"): (64.06, 8_384_798), ("c2", "fp64"): (90.02, 1_000_000)}
 
 
 class ClockSampler:
