@@ -28,6 +28,9 @@ using namespace m2m;
 namespace {
 
 constexpr int kPersistSteps = 64;
+// Most chunk-blocks an SM (chunks of observables times blocks an SM) with which every block
+// finalizes for itself (see `spread`): at most so many chunk sums are then in a block's memory.
+constexpr int kOwnChunks = 8;
 constexpr unsigned kPollLimit = 1u << 24;  // about ten seconds of polling
 
 // Scratch of the meetings; all zero between launches.
@@ -70,10 +73,12 @@ __global__ void __launch_bounds__(256, MINB) k_steps(const Model m, const Cst<T>
     __shared__ bool ok, last;
     __shared__ double lw;
     const TabLayout tl = tab_layout<T>(m);
-    // the coefficients and chunk sums of the finalize take the place of the block's sums; own:
-    // offset of the block's smoothed observables
-    double *cs = reinterpret_cast<double *>(smem), *csum = cs + m.J;
-    double *ys = reinterpret_cast<double *>(smem + own);
+    // The coefficients of the finalize take the place of the block's sums (J doubles of the 12 bytes
+    // each of J + 1 slots or more). own: offset of the block's smoothed observables and, behind them,
+    // its chunk sums: up to J of them with single apertures, they do not fit before the tables, which
+    // stay for the steps to come.
+    double *cs = reinterpret_cast<double *>(smem);
+    double *ys = reinterpret_cast<double *>(smem + own), *csum = ys + m.J;
     const FinPlan &pl = b.plan;
 
     tables_start<T>(b, S);
@@ -184,7 +189,8 @@ template <class T, int WPS>
 m2m_status setup(m2m_ctx *ctx)
 {
     const Model &m = ctx->m;
-    const size_t own = (ctx->smem_step + 15) / 16 * 16, smem = own + sizeof(double) * size_t(m.J);
+    const size_t own = (ctx->smem_step + 15) / 16 * 16;
+    const size_t smem = own + sizeof(double) * (size_t(m.J) + std::min(ctx->plan.n_chunks, kOwnChunks));
     int maxsm = 0;
     CU(cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
     if (smem > size_t(maxsm)) return M2M_OK;
@@ -227,7 +233,7 @@ m2m_status run(m2m_ctx *ctx, int nsteps)
     long long *h2 = ctx->d_hist2;
     Meet *g = static_cast<Meet *>(ctx->d_meet);
     const int grid = grid_for(ctx, ctx->steps_bps);
-    int spread = (grid + ctx->nsm - 1) / ctx->nsm * b.plan.n_chunks > 8;
+    int spread = (grid + ctx->nsm - 1) / ctx->nsm * b.plan.n_chunks > kOwnChunks;
     void *args[] = {&m, &k, &P, &b, &h2, &g, &nsteps, &ctx->steps_own, &spread};
     Turn &t = turn_of(ctx->device);
     std::lock_guard<std::mutex> lock(t.mu);
