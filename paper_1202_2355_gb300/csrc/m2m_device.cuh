@@ -1727,7 +1727,10 @@ struct Total;
 template <>
 struct Total<double> {
     long long hi = 0, lo = 0;
-    long long top = 0;  // sum of hi 2^-20, which cannot wrap: the range check
+    // The range check: the sum of hi 2^-20, with 2^43 (the whole range) for each weight whose own
+    // words are out of it. At most kMaxParticlesPerBlock weights meet in a block's sum of it:
+    // it cannot wrap.
+    long long top = 0;
     __device__ void add(double v, double scale)
     {
         long long a, b;
@@ -1735,13 +1738,15 @@ struct Total<double> {
         hi += a;
         lo += b;
     }
-    __device__ void add_fx(const Acc<double>::Fx &q)
+    __device__ void add_fx(const Acc<double>::Fx &q, double w, double scale)
     {
         hi += q.hi;
         lo += q.lo;
-        top += q.hi >> 20;
+        // w scale >= 2^62 on the exponents (infinity and NaN too): fx2 has dropped its high bits
+        const int e = int(bits_of(w) >> 52 & 0x7ff) + int(bits_of(scale) >> 52 & 0x7ff) - 2 * 1023;
+        top += e < 62 ? q.hi >> 20 : 1ll << 43;
     }
-    // the deposited weight for the range check (an FP64 sum would take the FP64 pipe)
+    // the deposited weight for the range check, in units of 2^20 (an FP64 sum would take the FP64 pipe)
     __device__ long long range_sum(double) const { return top; }
     __device__ static double range_value(long long v, double scale) { return double(v) * (1048576.0 * (1.0 / scale)); }
     __device__ long long word(int q, double) const { return q == 0 ? hi : lo; }
@@ -1754,7 +1759,7 @@ template <>
 struct Total<float> {
     long long s = 0;
     __device__ void add(float v, float scale) { s += __float2ll_rn(v * scale); }
-    __device__ void add_fx(const Acc<float>::Fx &q) { s += q.L; }
+    __device__ void add_fx(const Acc<float>::Fx &q, float, float) { s += q.L; }  // the range check: wdep
     __device__ float range_sum(float wdep) const { return wdep; }
     __device__ static double range_value(float v, float) { return double(v); }
     __device__ long long word(int, float) const { return s; }
@@ -2593,7 +2598,7 @@ __device__ __forceinline__ void step_particles(const Model &m, const Model &mh, 
             }
             if (cache) P.ap[i] = static_cast<uint16_t>(code_out);
             if (gxc) P.gx[i] = gout;
-            wtot.add_fx(wfx);
+            wtot.add_fx(wfx, w, k.fx_w);
             if constexpr (sizeof(T) == 4) wdep += w;
         }
         if (f.prior_step) {
@@ -2730,7 +2735,8 @@ constexpr double kRangeUnit = 1.0 / 1099511627776.0;  // 2^-40
 static __global__ void k_shard_pack(long long *hist, int hist_words, Scalars *sc)
 {
     if (threadIdx.x == 0 && blockIdx.x == 0) {
-        hist[hist_words] = llrint(ceil(sc->Wcheck / (sc->Wrange * kRangeUnit)));
+        // up to 2^12 times the range (infinity and NaN too): the words of all shards add up
+        hist[hist_words] = llrint(fmin(ceil(sc->Wcheck / (sc->Wrange * kRangeUnit)), 4503599627370496.0));
         sc->Wcheck = 0.0;
     }
 }
