@@ -836,6 +836,12 @@ m2m_status create_impl(const m2m_potential *pot, const m2m_observables *obs,
     if (s == M2M_OK) s = upload_tables(ctx);
     if (s == M2M_OK) s = smooth_setup(ctx);
     if (s == M2M_OK) s = persist_setup(ctx);
+    if (s == M2M_OK) {
+        // the copies and fills of the setup are on the default stream, which the fit's own is not
+        // ordered after (and a copy from pageable memory may return before it is done)
+        cudaError_t e = cudaStreamSynchronize(cudaStreamLegacy);
+        if (e != cudaSuccess) s = fail(ctx, M2M_ERR_CUDA, "setup: %s", cudaGetErrorString(e));
+    }
     if (s != M2M_OK) {
         g_create_error = ctx->err;
         m2m_destroy(ctx);
@@ -1664,41 +1670,43 @@ extern "C" m2m_status m2m_load_state(m2m_ctx *ctx, const char *path)
     ctx->n = hd.n;
     m.fx_w = hd.fx_w; m.fx_v2 = hd.fx_v2; m.fx_gh = hd.fx_gh; m.v2max = hd.v2max;
     if ((s = set_scales(ctx)) != M2M_OK) return s;
+    // everything on the fit's stream: it need not be ordered after the default stream, and k_head and
+    // the conversions read what the copies write
     const char *p = buf.data();
     for (int k = 0; k < narr; ++k) {
-        if (n) CU(cudaMemcpy(ctx->st[k], p, es * n, cudaMemcpyHostToDevice));
+        if (n) CU(cudaMemcpyAsync(ctx->st[k], p, es * n, cudaMemcpyHostToDevice, ctx->stream));
         p += es * n;
     }
-    if (n) CU(cudaMemcpy(ctx->cell, p, 2 * n, cudaMemcpyHostToDevice));
+    if (n) CU(cudaMemcpyAsync(ctx->cell, p, 2 * n, cudaMemcpyHostToDevice, ctx->stream));
     p += 2 * n;
-    if (n && apb) CU(cudaMemcpy(ctx->ap, p, apb, cudaMemcpyHostToDevice));
+    if (n && apb) CU(cudaMemcpyAsync(ctx->ap, p, apb, cudaMemcpyHostToDevice, ctx->stream));
     p += apb;
-    if (n && gxb) CU(cudaMemcpy(ctx->gx, p, gxb, cudaMemcpyHostToDevice));
+    if (n && gxb) CU(cudaMemcpyAsync(ctx->gx, p, gxb, cudaMemcpyHostToDevice, ctx->stream));
     p += gxb;
     double *dv[4] = {ctx->d_c, ctx->d_ytil, ctx->d_yraw, ctx->d_delta};
     for (auto d : dv) {
-        CU(cudaMemcpy(d, p, sizeof(double) * m.J, cudaMemcpyHostToDevice));
+        CU(cudaMemcpyAsync(d, p, sizeof(double) * m.J, cudaMemcpyHostToDevice, ctx->stream));
         p += sizeof(double) * m.J;
     }
-    CU(cudaMemcpy(ctx->d_rec, p, sizeof(double) * m.n_ap_total * m.rec_len, cudaMemcpyHostToDevice));
+    CU(cudaMemcpyAsync(ctx->d_rec, p, sizeof(double) * m.n_ap_total * m.rec_len, cudaMemcpyHostToDevice, ctx->stream));
     if (ctx->d_recf)
         k_convert_in<float><<<ctx->nsm, 256, 0, ctx->stream>>>(ctx->d_rec, ctx->d_recf, m.n_ap_total * m.rec_len);
     p += sizeof(double) * m.n_ap_total * m.rec_len;
     if (m.ncell) {
-        CU(cudaMemcpy(ctx->d_prior, p, sizeof(double) * m.ncell, cudaMemcpyHostToDevice));
+        CU(cudaMemcpyAsync(ctx->d_prior, p, sizeof(double) * m.ncell, cudaMemcpyHostToDevice, ctx->stream));
         p += sizeof(double) * m.ncell;
-        CU(cudaMemcpy(ctx->d_iprior, p, sizeof(double) * m.ncell, cudaMemcpyHostToDevice));
+        CU(cudaMemcpyAsync(ctx->d_iprior, p, sizeof(double) * m.ncell, cudaMemcpyHostToDevice, ctx->stream));
         if (ctx->d_ipriorf) k_convert_in<float><<<ctx->nsm, 256, 0, ctx->stream>>>(ctx->d_iprior, ctx->d_ipriorf, m.ncell);
         p += sizeof(double) * m.ncell;
-        CU(cudaMemcpy(ctx->d_lprior, p, sizeof(double) * m.ncell, cudaMemcpyHostToDevice));
+        CU(cudaMemcpyAsync(ctx->d_lprior, p, sizeof(double) * m.ncell, cudaMemcpyHostToDevice, ctx->stream));
         p += sizeof(double) * m.ncell;
-        CU(cudaMemcpy(ctx->d_prior_count, p, 8 * m.ncell, cudaMemcpyHostToDevice));
+        CU(cudaMemcpyAsync(ctx->d_prior_count, p, 8 * m.ncell, cudaMemcpyHostToDevice, ctx->stream));
         p += 8 * m.ncell;
-        if (m.smooth) CU(cudaMemcpy(ctx->d_prior_raw, p, sizeof(double) * m.ncell, cudaMemcpyHostToDevice));
+        if (m.smooth) CU(cudaMemcpyAsync(ctx->d_prior_raw, p, sizeof(double) * m.ncell, cudaMemcpyHostToDevice, ctx->stream));
         if (m.smooth) p += sizeof(double) * m.ncell;
     }
-    CU(cudaMemcpy(ctx->d_sc, p, sizeof(Scalars), cudaMemcpyHostToDevice));
-    CU(cudaMemset(ctx->d_hist, 0, sizeof(long long) * m.hist_words));
+    CU(cudaMemcpyAsync(ctx->d_sc, p, sizeof(Scalars), cudaMemcpyHostToDevice, ctx->stream));
+    CU(cudaMemsetAsync(ctx->d_hist, 0, sizeof(long long) * m.hist_words, ctx->stream));
     if ((s = persist_reset(ctx)) != M2M_OK) return s;
     k_head<<<1, 32, 0, ctx->stream>>>(m, ctx->d_sc, ctx->d_head);
     CU(cudaGetLastError());

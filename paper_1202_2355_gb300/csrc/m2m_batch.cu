@@ -236,6 +236,8 @@ static m2m_status batch_prepare(m2m_ctx *ctx)
     for (int i = 0; i < M; ++i) scs[i] = ctx->sub[i]->d_sc;
     if ((s = upload(ctx, B.d_scs, scs.data(), sizeof(Scalars *) * M)) != M2M_OK) return s;
     CU(cudaMalloc(&B.d_chi2, sizeof(double) * 2 * M));
+    // the copies are on the default stream, which the batch's own is not ordered after
+    CU(cudaStreamSynchronize(cudaStreamLegacy));
     B.nseg_total = (long long)seg.size();
     B.gens = gens;
     B.ready = true;

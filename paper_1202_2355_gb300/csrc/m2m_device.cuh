@@ -1972,7 +1972,8 @@ static inline cudaError_t upload_constants()
 {
     double t[32];
     exp2_table(t);
-    return cudaMemcpyToSymbol(kExp2j, t, sizeof t);
+    const cudaError_t e = cudaMemcpyToSymbol(kExp2j, t, sizeof t);
+    return e == cudaSuccess ? cudaStreamSynchronize(cudaStreamLegacy) : e;  // for kernels on any stream
 }
 
 // ---------------------------------------------------------------- finalize (last block)
