@@ -507,7 +507,7 @@ static m2m_status configure_kernels(m2m_ctx *ctx)
         // blocks that registers and threads allow on an SM (or blocks_per_sm) leave room for
         int rb = 0;
         const size_t base = std::max(smem_bytes<T>(m, 0, 0), red);
-        CU(cudaFuncSetAttribute(step_kernel<T>(ctx), cudaFuncAttributeMaxDynamicSharedMemorySize, int(base)));
+        CU(allow_smem(ctx->kstep, base));
         CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&rb, step_kernel<T>(ctx), ctx->block, base));
         if (rb < 1) return fail(ctx, M2M_ERR_ARG, "step kernel cannot be resident with block %d", ctx->block);
         if (ctx->bps > 0 && ctx->bps < rb) rb = ctx->bps;
@@ -529,8 +529,8 @@ static m2m_status configure_kernels(m2m_ctx *ctx)
     if (ctx->smem_step > size_t(maxsm))
         return fail(ctx, M2M_ERR_ARG, "observable tables and prior grid need %zu B of shared memory (limit %d)",
                     ctx->smem_step, maxsm);
-    CU(cudaFuncSetAttribute(step_kernel<T>(ctx), cudaFuncAttributeMaxDynamicSharedMemorySize, int(ctx->smem_step)));
-    CU(cudaFuncSetAttribute(k_materialize<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(ctx->smem_mat)));
+    CU(allow_smem(ctx->kstep, ctx->smem_step));
+    CU(allow_smem(reinterpret_cast<const void *>(k_materialize<T>), ctx->smem_mat));
     int occ = 0;
     CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, step_kernel<T>(ctx), ctx->block, ctx->smem_step));
     if (occ < 1) return fail(ctx, M2M_ERR_ARG, "step kernel cannot be resident with block %d", ctx->block);
@@ -2279,7 +2279,7 @@ extern "C" m2m_status m2m_observe_static(const m2m_observables *obs, int64_t n, 
     m.fx_v2 = pow2_floor(two62 / (Wb * (m.v2max > 1.0 ? m.v2max : 1.0)));
     m.fx_gh = pow2_floor(two62 / (Wb * 1.5));
     const size_t smem = sizeof(unsigned) * 3 * size_t(J);
-    CS(cudaFuncSetAttribute(k_static_observe, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+    CS(allow_smem(reinterpret_cast<const void *>(k_static_observe), smem));
     int occ = 0;
     CS(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_static_observe, 256, smem));
     long long grid = std::min<long long>((n + 255) / 256, (long long)nsm * std::max(occ, 1));

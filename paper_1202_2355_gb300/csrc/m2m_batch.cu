@@ -390,7 +390,7 @@ static m2m_status batch_configure(m2m_ctx *ctx, const m2m_options *opt)
         return fail(ctx, M2M_ERR_ARG, "the largest fit needs %zu B of shared memory (limit %d)", smem, B.maxsm);
     B.smem = smem;
     using Fn = BatchFn<T>;
-    CU(cudaFuncSetAttribute(reinterpret_cast<Fn>(B.kernel), cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+    CU(allow_smem(B.kernel, smem));
     B.block = opt->block > 0 ? opt->block : 256;
     if (B.block % 32 != 0 || B.block > 256) return fail(ctx, M2M_ERR_ARG, "block must be a multiple of 32, <= 256");
     int occ = 0;

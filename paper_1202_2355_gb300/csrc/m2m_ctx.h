@@ -194,6 +194,22 @@ inline void place_tables(m2m::Model &m, size_t limit)
     m.tab_smem = step_smem<T>(m) <= limit ? 1 : 0;
 }
 
+// Lets a kernel take `need` bytes of dynamic shared memory at a launch. The limit is the kernel's, not
+// a fit's: it is always raised to the most the device has, so that no fit, and no thread between
+// another's limit and its launch, lowers it for the others.
+inline cudaError_t allow_smem(const void *fn, size_t need)
+{
+    int dev = 0, most = 0;
+    cudaFuncAttributes a;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, fn);
+    if (e != cudaSuccess) return e;
+    most -= int(a.sharedSizeBytes);
+    if (need > size_t(most)) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 // Resident blocks per SM the step kernels are compiled for (register budget). The
 // batched mixed-precision kernel runs best at 4 blocks of 256 (64 registers; 1.147 ms
 // against 1.176 ms at 5 blocks on the 96-fit workload), the single-fit one at 5.

@@ -350,7 +350,7 @@ m2m_status bin_launch(m2m_ctx *ctx, K shared, K global, size_t bytes, long long 
     const bool sh = bytes <= size_t(maxsm);
     K fn = sh ? shared : global;
     if (!sh) bytes = 0;
-    CU(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes)));
+    CU(allow_smem(reinterpret_cast<const void *>(fn), bytes));
     int occ = 0;
     CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kDiagThreads, bytes));
     const long long want = (n + kDiagThreads - 1) / kDiagThreads, cap = (long long)ctx->nsm * (occ > 0 ? occ : 1);

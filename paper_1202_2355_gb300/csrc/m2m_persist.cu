@@ -195,7 +195,7 @@ m2m_status setup(m2m_ctx *ctx)
     CU(cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
     if (smem > size_t(maxsm)) return M2M_OK;
     StepsFn<T> fn = pick_steps<T, WPS>(m);
-    CU(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+    CU(allow_smem(reinterpret_cast<const void *>(fn), smem));
     int occ = 0;
     CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, ctx->block, smem));
     if (occ < 1) return M2M_OK;
