@@ -1129,6 +1129,7 @@ static const int kGraphSteps = 16;
 static m2m_status build_graph(m2m_ctx *ctx)
 {
     cudaGraph_t g = nullptr;
+    const RelaxedCapture relaxed;
     CU(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
     for (int k = 0; k < kGraphSteps; ++k) launch_one(ctx, 1, 0);
     cudaError_t e = cudaStreamEndCapture(ctx->stream, &g);
@@ -1168,12 +1169,15 @@ extern "C" m2m_status m2m_step(m2m_ctx *ctx, int64_t nsteps)
     // two steps or more of a fit that can: one launch for many (a single step finalizes in its
     // last block, without a meeting)
     // (plain launches on a stream under capture, as ever)
+    int64_t left = nsteps;
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     if (nsteps > 1 && persist_fits(ctx)) {
         CU(cudaStreamIsCapturing(ctx->stream, &capture));
-        if (capture == cudaStreamCaptureStatusNone) return persist_steps(ctx, nsteps);
+        if (capture == cudaStreamCaptureStatusNone) {
+            const m2m_status s = persist_steps(ctx, left);
+            if (s != M2M_OK) return s;
+        }
     }
-    int64_t left = nsteps;
     if (left >= kGraphSteps && !ctx->graph) {
         m2m_status s = build_graph(ctx);
         if (s != M2M_OK) return s;

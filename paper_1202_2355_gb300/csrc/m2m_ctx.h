@@ -141,7 +141,7 @@ void smooth_launch(m2m_ctx *ctx);
 m2m_status persist_setup(m2m_ctx *ctx);
 bool persist_fits(m2m_ctx *ctx);
 m2m_status persist_reset(m2m_ctx *ctx);
-m2m_status persist_steps(m2m_ctx *ctx, int64_t nsteps);
+m2m_status persist_steps(m2m_ctx *ctx, int64_t &left);
 void persist_free(m2m_ctx *ctx);
 int grid_for(m2m_ctx *ctx, int bps);  // blocks of a step kernel at most bps of which share an SM
 
@@ -193,6 +193,14 @@ inline void place_tables(m2m::Model &m, size_t limit)
     m.tab_smem = 1;
     m.tab_smem = step_smem<T>(m) <= limit ? 1 : 0;
 }
+
+// While it lives, calls of this thread are allowed though some thread captures a stream in the
+// global mode (event queries and the instantiation of a graph are not otherwise, and would end that capture).
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
 
 // Lets a kernel take `need` bytes of dynamic shared memory at a launch. The limit is the kernel's, not
 // a fit's: it is always raised to the most the device has, so that no fit, and no thread between
