@@ -145,10 +145,12 @@ __host__ __device__ __forceinline__ double big_double(const Big &a)
 // The leading 24 bits of a significand as a float in [1, 2).
 __host__ __device__ __forceinline__ float big_lead(u64 m) { return of_bits32(0x3f800000u | (unsigned(m >> 40) & 0x7fffffu)); }
 
-// The seed in [1/2, 1) as its 24 bits (a seed of 1 becomes 1 - 2^-24).
+// The seed as its 24 bits, in [1/2, 1): the hardware approximations may give 1, or a value below
+// 1/2 for an argument next to 2, whose significand would be read as nearly 1.
 __host__ __device__ __forceinline__ u64 seed_bits(float y)
 {
-    return (bits_of32(y < 0.99999994f ? y : 0.99999994f) & 0x7fffffu) | 0x800000u;
+    y = y < 0.99999994f ? y : 0.99999994f;
+    return (bits_of32(y > 0.5f ? y : 0.5f) & 0x7fffffu) | 0x800000u;
 }
 
 // A root in [1/2, 1] at scale 2^64 that its rounding may have carried a few units over either
