@@ -306,12 +306,13 @@ __host__ __device__ __forceinline__ double exp_int(double x, const u64 *t)
     return big_double(exp_big(x, t));
 }
 
-// exp(-t/2) for t >= 0 (the halving is one step of the exponent).
+// exp(-t/2) for t >= 0 (the halving is one step of the exponent); NaN of either sign stays NaN.
 __host__ __device__ __forceinline__ double exp_mhalf(double t, const u64 *tab)
 {
     const i64 b = bits_of(t);
     const double x = b > (64ll << 52) ? of_bits((b - (1ll << 52)) | i64(1ull << 63)) : 0.0;  // t < 2^-959 gives 1
-    return exp_int(b >= (2047ll << 52) ? of_bits(b | i64(1ull << 63)) : x, tab);  // inf and NaN: negated
+    const bool far = (b & 0x7fffffffffffffffll) >= (2047ll << 52);
+    return exp_int(far ? of_bits(b | i64(1ull << 63)) : x, tab);  // inf and NaN: negated
 }
 
 // ---------------------------------------------------------------- force factors

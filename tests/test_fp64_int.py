@@ -168,3 +168,7 @@ def test_special_values(lib, device):
     assert np.all(y[:5] == 0.0) and np.all(np.isposinf(y[5:8])) and np.isnan(y[8])
     y, _ = _run(lib, "exp_mhalf", device, [inf, 1414.0, 1e300, 0.0, -0.0, sub], errors=False)
     assert np.all(y[:3] == 0.0) and np.all(y[3:] == 1.0)
+    # NaN of either sign (an invalid operation gives the negative one on the device) stays NaN
+    y, _ = _run(lib, "exp_mhalf", device, np.array([0x7ff8 << 48, 0xfff8 << 48, (0xfff << 52) | 1], np.uint64).view(np.float64),
+                errors=False)
+    assert np.all(np.isnan(y)), y
