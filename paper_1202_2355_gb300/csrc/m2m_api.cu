@@ -570,8 +570,8 @@ static std::vector<unsigned char> host_tables(const m2m_ctx *ctx, const TabLayou
     return h;
 }
 
-// The rows of the finalize, chunk by chunk (see m2m::FinPlan); the fixed-point scales are
-// those of the loaded particles (1 before the first load).
+// The rows of the finalize, chunk by chunk (see m2m::FinPlan), with fixed-point scales of 1 until
+// the first load (set_scales).
 static std::vector<ObsRow> plan_rows(const m2m_ctx *ctx)
 {
     const Model &m = ctx->m;
@@ -584,7 +584,6 @@ static std::vector<ObsRow> plan_rows(const m2m_ctx *ctx)
                     ObsRow r{0.0, 0.0, 0.0, 0.0, 1.0, 1.0, -1, 0};
                     if (p0 + q < G.n_ap) {
                         r.j = G.obs_off + k * G.n_ap + p0 + q;
-                        r.iscale = ctx->obs_iscale.empty() ? 1.0 : ctx->obs_iscale[r.j];
                         r.post = ctx->obs_post[r.j];
                         r.cw = r.post / ctx->sig[r.j];
                         r.Y = ctx->Y[r.j];
@@ -686,19 +685,25 @@ static m2m_status upload_plan(m2m_ctx *ctx)
     return M2M_OK;
 }
 
-// The fixed-point scales of the loaded particles into obs_iscale and the rows of the finalize.
+// 1/scale of the sums of each kind of observable into the rows of the finalize.
+static __global__ void k_row_scales(ObsRow *rows, int n, const int *kind, double iw, double iv, double ig)
+{
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
+        const int j = rows[q].j;
+        if (j < 0) continue;
+        const int k = kind[j];
+        rows[q].iscale = k == kKindMass ? iw : (k == kKindV2 || k == kKindV1 ? iv : ig);
+    }
+}
+
+// The fixed-point scales of the loaded particles, queued on the fit's stream.
 static m2m_status set_scales(m2m_ctx *ctx)
 {
     const Model &m = ctx->m;
-    ctx->obs_iscale.resize(m.J);
-    for (int j = 0; j < m.J; ++j) {
-        const int k = ctx->obs_kind[j];
-        ctx->obs_iscale[j] = 1.0 / (k == kKindMass ? m.fx_w : ((k == kKindV2 || k == kKindV1) ? m.fx_v2 : m.fx_gh));
-    }
-    const std::vector<ObsRow> rows = plan_rows(ctx);
-    CU(cudaMemcpyAsync(ctx->d_plan, rows.data(), sizeof(ObsRow) * rows.size(), cudaMemcpyHostToDevice,
-                       ctx->stream));
-    CU(cudaStreamSynchronize(ctx->stream));
+    const int n = 32 * ctx->plan.n_chunks;
+    k_row_scales<<<(n + 255) / 256, 256, 0, ctx->stream>>>(reinterpret_cast<ObsRow *>(ctx->d_plan), n, ctx->d_kind,
+                                                           1.0 / m.fx_w, 1.0 / m.fx_v2, 1.0 / m.fx_gh);
+    CU(cudaGetLastError());
     return M2M_OK;
 }
 
@@ -855,7 +860,14 @@ extern "C" m2m_status m2m_create(const m2m_potential *pot, const m2m_observables
                                  const m2m_prior_grid *prior, double eps, double mu, double alpha,
                                  const m2m_options *opt, m2m_ctx **out)
 {
-    return create_impl(pot, obs, prior, eps, mu, alpha, opt, 0, out);
+    const m2m_status s = create_impl(pot, obs, prior, eps, mu, alpha, opt, 0, out);
+    if (s != M2M_OK) return s;
+    const m2m_status a = persist_alloc(*out);  // a batch's fits only once one of them steps alone
+    if (a == M2M_OK) return a;
+    g_create_error = (*out)->err;
+    destroy_impl(*out);
+    *out = nullptr;
+    return a;
 }
 
 // ------------------------------------------------------------------ launches

@@ -25,7 +25,7 @@ struct m2m_ctx {
     size_t smem_step = 0, smem_mat = 0;
 
     // host copies of the descriptors
-    std::vector<double> edges, Vp, isp, Y, sig, obs_post, obs_iscale, area_of_obs, lcE, scf_r;
+    std::vector<double> edges, Vp, isp, Y, sig, obs_post, area_of_obs, lcE, scf_r;
     std::vector<int> obs_kind;
     std::vector<unsigned short> lut;
     uint64_t config_hash = 0;
@@ -69,8 +69,7 @@ struct m2m_ctx {
     void *ksteps = nullptr;
     size_t smem_steps = 0;
     int steps_own = 0, steps_bps = 0;
-    long long *d_hist2 = nullptr;
-    void *d_meet = nullptr;
+    long long *d_hist2 = nullptr;  // two more sets of sums, and behind them the scratch of the meetings
 
     cudaGraphExec_t graph = nullptr;
     int graph_steps = 0;
@@ -139,6 +138,7 @@ void smooth_launch(m2m_ctx *ctx);
 
 // several steps per launch (m2m_persist.cu)
 m2m_status persist_setup(m2m_ctx *ctx);
+m2m_status persist_alloc(m2m_ctx *ctx);
 bool persist_fits(m2m_ctx *ctx);
 m2m_status persist_reset(m2m_ctx *ctx);
 m2m_status persist_steps(m2m_ctx *ctx, int64_t &left);

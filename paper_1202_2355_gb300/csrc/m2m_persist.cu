@@ -185,6 +185,9 @@ StepsFn<T> pick_steps(const Model &m)
     }
 }
 
+// Two sets of sums and the scratch of the meetings (8-byte words both).
+size_t scratch_bytes(const m2m_ctx *ctx) { return sizeof(long long) * 2 * size_t(ctx->m.hist_words) + sizeof(Meet); }
+
 template <class T, int WPS>
 m2m_status setup(m2m_ctx *ctx)
 {
@@ -200,10 +203,6 @@ m2m_status setup(m2m_ctx *ctx)
     CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, ctx->block, smem));
     if (occ < 1) return M2M_OK;
     ctx->steps_bps = std::min(occ, ctx->bps);
-    CU(cudaMalloc(&ctx->d_hist2, sizeof(long long) * 2 * m.hist_words));
-    CU(cudaMemset(ctx->d_hist2, 0, sizeof(long long) * 2 * m.hist_words));
-    CU(cudaMalloc(&ctx->d_meet, sizeof(Meet)));
-    CU(cudaMemset(ctx->d_meet, 0, sizeof(Meet)));
     ctx->ksteps = reinterpret_cast<void *>(fn);
     ctx->smem_steps = smem;
     ctx->steps_own = int(own);
@@ -259,7 +258,7 @@ m2m_status run(m2m_ctx *ctx, int nsteps, bool &done)
     State<T> P = state<T>(ctx);
     Buffers b = buffers(ctx);
     long long *h2 = ctx->d_hist2;
-    Meet *g = static_cast<Meet *>(ctx->d_meet);
+    Meet *g = reinterpret_cast<Meet *>(h2 + 2 * ctx->m.hist_words);
     const int grid = grid_for(ctx, ctx->steps_bps);
     int spread = (grid + ctx->nsm - 1) / ctx->nsm * b.plan.n_chunks > kOwnChunks;
     void *args[] = {&m, &k, &P, &b, &h2, &g, &nsteps, &ctx->steps_own, &spread};
@@ -302,15 +301,21 @@ bool persist_fits(m2m_ctx *ctx)
 void persist_free(m2m_ctx *ctx)
 {
     free_dev(ctx->d_hist2);
-    cudaFree(ctx->d_meet);
-    ctx->d_meet = nullptr;
+}
+
+// The scratch of these launches, zeroed, unless the fit has it.
+m2m_status persist_alloc(m2m_ctx *ctx)
+{
+    if (!ctx->ksteps || ctx->d_hist2) return M2M_OK;
+    const RelaxedCapture relaxed;
+    CU(cudaMalloc(&ctx->d_hist2, scratch_bytes(ctx)));
+    return persist_reset(ctx);
 }
 
 m2m_status persist_reset(m2m_ctx *ctx)
 {
-    if (!ctx->ksteps) return M2M_OK;
-    CU(cudaMemsetAsync(ctx->d_hist2, 0, sizeof(long long) * 2 * ctx->m.hist_words, ctx->stream));
-    CU(cudaMemsetAsync(ctx->d_meet, 0, sizeof(Meet), ctx->stream));
+    if (!ctx->d_hist2) return M2M_OK;
+    CU(cudaMemsetAsync(ctx->d_hist2, 0, scratch_bytes(ctx), ctx->stream));
     return M2M_OK;
 }
 
@@ -318,6 +323,8 @@ m2m_status persist_reset(m2m_ctx *ctx)
 // its turn) while it is the fit's turn; left: the steps that remain for the caller.
 m2m_status persist_steps(m2m_ctx *ctx, int64_t &left)
 {
+    const m2m_status a = persist_alloc(ctx);
+    if (a != M2M_OK) return a;
     while (left > 0) {
         const int now = int(std::min<int64_t>(left, kPersistSteps));
         bool done = false;
