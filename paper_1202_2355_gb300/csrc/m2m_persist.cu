@@ -19,6 +19,7 @@
 // again. Waits are bounded: a block that gives up sets kErrTimeout and returns, and so do all
 // others in turn.
 #include "m2m_ctx.h"
+#include "m2m_meet.cuh"
 
 #include <algorithm>
 #include <mutex>
@@ -31,38 +32,6 @@ constexpr int kPersistSteps = 64;
 // Most chunk-blocks an SM (chunks of observables times blocks an SM) with which every block
 // finalizes for itself (see `spread`): at most so many chunk sums are then in a block's memory.
 constexpr int kOwnChunks = 8;
-constexpr unsigned kPollLimit = 1u << 24;  // about ten seconds of polling
-
-// Scratch of the meetings; all zero between launches.
-struct Meet {
-    unsigned arrived, done, failed, pad;
-    double wcheck[3];
-};
-
-// Every block arrives and waits for `target` arrivals. Returns false after the poll limit or
-// once another block has given up.
-__device__ bool meet(Meet *g, unsigned target, bool *ok)
-{
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(&g->arrived, 1u);
-        unsigned polls = 0, v;
-        bool good = true;
-        do {
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&g->arrived) : "memory");
-            if (v < target && (++polls & 1023u) == 0) {
-                unsigned f;
-                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(f) : "l"(&g->failed) : "memory");
-                if (f || polls >= kPollLimit) good = false;
-            }
-        } while (v < target && good);
-        if (!good) atomicExch(&g->failed, 1u);
-        *ok = good;
-    }
-    __syncthreads();
-    return *ok;
-}
 
 template <class T, int WPS, int MINB, unsigned M0, unsigned M1, unsigned M2, unsigned M3>
 __global__ void __launch_bounds__(256, MINB) k_steps(const Model m, const Cst<T> k, const State<T> P, const Buffers b,
