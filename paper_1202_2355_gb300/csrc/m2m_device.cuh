@@ -2451,7 +2451,15 @@ __device__ __forceinline__ void block_zero(const Model &m, const Smem<T> &S)
 // The per-particle part of one step for particles i0, i0 + stride, ... below i1:
 // the pending force of change, the push, the deposit, the prior binning, and the
 // write-back of the state.
-template <class T, bool GA, unsigned M0, unsigned M1, unsigned M2, unsigned M3>
+//
+// LATE: the next particle's loads are issued after the force of change instead of before it. Their
+// ten values are then not alive across the force of change, where the mixed batched kernel and that of
+// the global deposits (64 registers) otherwise spill two or three into local memory and miss the
+// L1 with them (long-scoreboard stalls 0.5 -> 2.5 per instruction). us per step, before and after: 96
+// Hernquist + NFW fits of 52M particles 934 -> 816, Hernquist 873 -> 794, log halo 873 -> 793; maps
+// of 8M 5 % in all. The other kernels lose by it and load early: FP64 1M 119.2 -> 121.5, the mixed
+// one of five blocks an SM 45.9 -> 46.4 at 2M, many mixed steps per launch up to 2 %.
+template <class T, bool GA, bool LATE, unsigned M0, unsigned M1, unsigned M2, unsigned M3>
 __device__ __forceinline__ void step_particles(const Model &m, const Model &mh, const Cst<T> &k, const State<T> &P,
                                                const Buffers &b,
                                                const Smem<T> &S, const StepFlags<T> &f, int push, long long i0,
@@ -2501,7 +2509,7 @@ __device__ __forceinline__ void step_particles(const Model &m, const Model &mh, 
         const T gin = ngx;
         const T fa_in = nfa;
         const T *gp = gxc ? &gin : static_cast<const T *>(nullptr);
-        if (i + stride < i1) fetch(i + stride);
+        if (!LATE && i + stride < i1) fetch(i + stride);
         T w, u;
         if constexpr (kLogWeights<T>) {
             u = wst + f.lwscale;
@@ -2518,6 +2526,7 @@ __device__ __forceinline__ void step_particles(const Model &m, const Model &mh, 
             }
             u = w;
         }
+        if (LATE && i + stride < i1) fetch(i + stride);
         if (keeps_accel<T>(mh)) {
             T fa;
             if (push) {
@@ -2712,7 +2721,7 @@ __global__ void __launch_bounds__(kStepMaxThreads<T, GA>, (GA && sizeof(T) == 4)
     unsigned err = 0;
     Total<T> wtot;
     T wdep = T(0);  // floating-point twin of wtot, for the fixed-point range check
-    step_particles<T, GA, M0, M1, M2, M3>(m, m, k, P, b, S, f, push, lo + threadIdx.x, hi, blockDim.x, err, wtot, wdep);
+    step_particles<T, GA, GA && sizeof(T) == 4, M0, M1, M2, M3>(m, m, k, P, b, S, f, push, lo + threadIdx.x, hi, blockDim.x, err, wtot, wdep);
     block_flush<T, WPS, GA>(m, k, b.sc, b.hist, &b.sc->Wcheck, S, f.prior_step, err, wtot, wdep, f.scf_step);
     if (GA || m.fin_wide || m.shard) return;  // k_finalize follows (a shard's after the exchange of its sums)
     // last block to finish runs the finalize
@@ -2872,10 +2881,10 @@ __global__ void __launch_bounds__(256, MINB) k_step_batch(const BatchArgs<T> a, 
         Total<T> wtot;
         T wdep = T(0);
         if constexpr (BANK)
-            step_particles<T, false, M0, M1, M2, M3>(m, bank.shape, bank.cst[sg.model], P, b, S, f, 1,
+            step_particles<T, false, sizeof(T) == 4, M0, M1, M2, M3>(m, bank.shape, bank.cst[sg.model], P, b, S, f, 1,
                                                      sg.begin + threadIdx.x, sg.end, blockDim.x, err, wtot, wdep);
         else
-            step_particles<T, false, M0, M1, M2, M3>(m, m, k, P, b, S, f, 1, sg.begin + threadIdx.x, sg.end,
+            step_particles<T, false, sizeof(T) == 4, M0, M1, M2, M3>(m, m, k, P, b, S, f, 1, sg.begin + threadIdx.x, sg.end,
                                                      blockDim.x, err, wtot, wdep);
         block_flush<T, WPS, false>(m, k, b.sc, b.hist, &b.sc->Wcheck, S, f.prior_step, err, wtot, wdep, f.scf_step);
         if (block_is_last(&b.sc->blocks_done, a.nseg[cur], &am_last)) {

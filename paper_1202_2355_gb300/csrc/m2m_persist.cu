@@ -72,8 +72,8 @@ __global__ void __launch_bounds__(256, MINB) k_steps(const Model m, const Cst<T>
         unsigned err = 0;
         Total<T> wtot;
         T wdep = T(0);
-        step_particles<T, false, M0, M1, M2, M3>(m, m, k, P, b, S, f, 1, lo + threadIdx.x, hi, blockDim.x, err, wtot,
-                                                 wdep);
+        step_particles<T, false, false, M0, M1, M2, M3>(m, m, k, P, b, S, f, 1, lo + threadIdx.x, hi, blockDim.x, err,
+                                                        wtot, wdep);
         block_flush<T, WPS, false>(m, k, b.sc, hist, &g->wcheck[set], S, f.prior_step, err, wtot, wdep, 0);
         good = meet(g, (meetings += gridDim.x), &ok);
         if (!good) break;
