@@ -1765,11 +1765,17 @@ struct Total<float> {
     __device__ long long word(int, float) const { return s; }
 };
 
+// hi + lo 2^-32 in FP64, with the whole part of the fraction word carried first: how a sum is split
+// over its two words depends on the blocks that added it, and beyond 2^53 the rounding of hi would too.
+__device__ __forceinline__ double fx_join(long long hi, long long lo)
+{
+    return double(hi + (lo >> 32)) + double(lo & 0xffffffffll) * (1.0 / 4294967296.0);
+}
 template <int WPS>
 __device__ __forceinline__ double fx_read(const long long *h, int slot)
 {
     if (WPS == 1) return double(__ldcg(h + slot));
-    return double(__ldcg(h + 2 * slot)) + double(__ldcg(h + 2 * slot + 1)) * (1.0 / 4294967296.0);
+    return fx_join(__ldcg(h + 2 * slot), __ldcg(h + 2 * slot + 1));
 }
 
 // ---------------------------------------------------------------- force of change
@@ -2130,8 +2136,7 @@ __device__ void window_priors(const Model &m, const Buffers &b, long long *hist,
             box[q] = __ldcg(col + size_t(hi) * nx) - (lo >= 0 ? __ldcg(col + size_t(lo) * nx) : 0ull);
         }
         const long long cnt = (long long)box[0];
-        double sum = double((long long)box[1]);
-        if (WPS == 2) sum += double((long long)box[2]) * (1.0 / 4294967296.0);
+        double sum = WPS == 2 ? fx_join((long long)box[1], (long long)box[WPS]) : double((long long)box[1]);
         sum = sum / m.fx_w * s_ren;
         const double pr = cnt > 0 ? sum / double(cnt) : 0.0;
         write_prior(b, c, pr);
