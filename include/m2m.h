@@ -237,7 +237,8 @@ m2m_status m2m_load_particles(m2m_ctx *ctx, int64_t n, const double *pos, const 
 m2m_status m2m_load_particles_device(m2m_ctx *ctx, int64_t n, const double *pos_dev,
                                      const double *vel_dev, const double *w_dev);
 
-/* Advance nsteps >= 0 M2M steps, asynchronously on the context stream. */
+/* Advance nsteps >= 0 M2M steps, asynchronously on the context stream. Fits on
+ * streams of their own do not wait for one another. */
 m2m_status m2m_step(m2m_ctx *ctx, int64_t nsteps);
 
 /* Wait for the context stream; report any latched device error. */

@@ -466,7 +466,7 @@ template <class T, int WPS>
 static m2m_status configure_kernels(m2m_ctx *ctx)
 {
     Model &m = ctx->m;
-    // the finalize reuses the start of the dynamic shared memory for a block reduction
+    // (the finalize in the last block takes the start of the dynamic shared memory: step_smem)
     int maxsm = 0, smsm = 0;
     CU(cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
     place_tables<T>(m, size_t(maxsm));

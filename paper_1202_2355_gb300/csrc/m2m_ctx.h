@@ -219,8 +219,8 @@ inline cudaError_t allow_smem(const void *fn, size_t need)
 }
 
 // Resident blocks per SM the step kernels are compiled for (register budget). The
-// batched mixed-precision kernel runs best at 4 blocks of 256 (64 registers; 1.147 ms
-// against 1.176 ms at 5 blocks on the 96-fit workload), the single-fit one at 5.
+// batched mixed-precision kernel runs best at 4 blocks of 256 (64 registers; 2.5 % faster than
+// 5 blocks on the 96-fit workload), the single-fit one at 5.
 template <class T>
 constexpr int kMinBlocks = sizeof(T) == 8 ? 2 : 5;
 template <class T>

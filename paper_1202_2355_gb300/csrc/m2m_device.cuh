@@ -642,9 +642,6 @@ __device__ __forceinline__ T scf_circ(const Model &m, const Cst<T> &k, T R, T &v
     return phi + T(0.5) * vc2;
 }
 
-// SCF: whether the code of the self-consistent potential is compiled in (only the generic
-// step kernel and the helpers around it need it; the kernels specialised to an observable
-// shape run the other potentials without its registers).
 // -phi of the spherical potentials at r (ir = 1/r), G M/(r + a) + G M_s ln(1 + r/r_s)/r, and, if
 // vc2 is not null, v_c^2 = G M r/(r + a)^2 + G M_s mu/r.
 __host__ __device__ __forceinline__ Big well_big(const Model &m, const Cst<double> &k, const Big &r, const Big &ir,
@@ -671,6 +668,9 @@ struct FnTables {
     const u64 *et, *ln;
 };
 
+// The potential. SCF: whether the code of the self-consistent one is compiled in (only the generic
+// step kernel and the helpers around it need it; the kernels specialised to an observable
+// shape run the other potentials without its registers).
 template <class T, bool SCF = true>
 __host__ __device__ __forceinline__ T potential(const Model &m, const Cst<T> &k, T x, T y, T z,
                                                 FnTables fn = FnTables{nullptr, nullptr})
@@ -1401,9 +1401,6 @@ __host__ __device__ __forceinline__ T circ_energy(const Model &m, const Cst<T> &
     return phi + T(0.5) * vc2;
 }
 
-// Lc(E): closed form for the Hernquist potential (E_c = -(u+1)/(2u^2) GM/a with
-// u = R/a + 1), otherwise the host table of E_c(ln R) bracketed by binary search,
-// interpolated, and refined by secant steps on E_c(R) = E.
 // Square root, quotient (b > 0), exponential and logarithm of the prior binning: FP64 on the
 // integer pipe where fn has the tables.
 __device__ __forceinline__ float p_sqrt(float x, FnTables) { return d_sqrt(x); }
@@ -1426,6 +1423,9 @@ __device__ __forceinline__ const double *lc_table<double>(const Buffers &b) { re
 template <>
 __device__ __forceinline__ const float *lc_table<float>(const Buffers &b) { return b.lcEf; }
 
+// Lc(E): closed form for the Hernquist potential (E_c = -(u+1)/(2u^2) GM/a with
+// u = R/a + 1), otherwise the host table of E_c(ln R) bracketed by binary search,
+// interpolated, and refined by secant steps on E_c(R) = E.
 template <class T, bool SCF = true>
 __device__ T circular_L(const Model &m, const Cst<T> &k, const LcTable<T> *lcE, T E, FnTables fn)
 {
@@ -1840,7 +1840,7 @@ __device__ __forceinline__ T foc_update_log(const Model &m, const Cst<T> &k, con
         }
         un = u + log1p(h);
     }
-    // exp_tab overflows above 709 (NaN of either sign is flagged too)
+    // exp_int overflows above 709 (NaN of either sign is flagged too)
     const long long ub = bits_of(un);
     if ((ub & 0x7fffffffffffffffll) > 0x7ff0000000000000ll || ub > 0x4086280000000000ll) err |= kErrNonFinite;
     return un;
@@ -1982,11 +1982,13 @@ static inline cudaError_t upload_constants()
     return e == cudaSuccess ? cudaStreamSynchronize(cudaStreamLegacy) : e;  // for kernels on any stream
 }
 
-// ---------------------------------------------------------------- finalize (last block)
+// ---------------------------------------------------------------- finalize
 //
-// Run by the last block of the step kernel once every block has added its sums:
-// converts the fixed-point sums, renormalises, smooths (eq. myts), forms Delta_j,
-// chi^2 (eqs. delta, chi) and the force-of-change coefficients, the prior means on
+// Run once every block has added its sums, by the last block of the step kernel, by k_finalize or
+// between the steps of k_steps: converts the fixed-point sums, renormalises, smooths (eq. myts), forms
+// Delta_j, chi^2 (eqs. delta, chi) and the force-of-change coefficients, the prior means on
+// update steps, and clears the sums for the next step.
+
 // The sum of v over the block, for any block size (a multiple of 32), to every thread: warp
 // shuffles, then the warps' sums from shared memory in warp order (the same order in every
 // kernel that ends with the finalize). red: 32 doubles.
@@ -2003,7 +2005,7 @@ __device__ __forceinline__ double fold_block(double v, double *red)
 // The self-consistent potential at an update (Sec. 6), in the finalize: the mass-to-light
 // ratio follows the chi^2 gradient, d ln Upsilon/dt = -eps_ups sum_j Delta_j/sigma_j D_j over
 // the update_every steps to the next update (not at the load); then the interval tables
-// TA, TB of scf_field from the new coefficients a_lm,k and Upsilon. red: blockDim doubles.
+// TA, TB of scf_field from the new coefficients a_lm,k and Upsilon. red: 32 doubles.
 template <int WPS>
 __device__ void scf_finalize(const Model &m, const Buffers &b, double s_ren, int init, double *red)
 {
@@ -2076,7 +2078,6 @@ __device__ void scf_finalize(const Model &m, const Buffers &b, double s_ren, int
     __syncthreads();
 }
 
-// update steps, and clears the sums for the next step. red: blockDim doubles.
 // Priors of the grid-less variant (Sec. 7): the mean weight of the particles in the window of
 // cells |k' - k| <= pwin_E, |l' - l| <= pwin_x around each cell (k, l), cut at the grid's
 // edges. The window sums come from cumulative sums of the cells' integer words, first along
@@ -2458,12 +2459,13 @@ __device__ __forceinline__ void block_zero(const Model &m, const Smem<T> &S)
 // write-back of the state.
 //
 // LATE: the next particle's loads are issued after the force of change instead of before it. Their
-// ten values are then not alive across the force of change, where the mixed batched kernel and that of
-// the global deposits (64 registers) otherwise spill two or three into local memory and miss the
-// L1 with them (long-scoreboard stalls 0.5 -> 2.5 per instruction). us per step, before and after: 96
-// Hernquist + NFW fits of 52M particles 934 -> 816, Hernquist 873 -> 794, log halo 873 -> 793; maps
-// of 8M 5 % in all. The other kernels lose by it and load early: FP64 1M 119.2 -> 121.5, the mixed
-// one of five blocks an SM 45.9 -> 46.4 at 2M, many mixed steps per launch up to 2 %.
+// ten values are then not alive across the force of change, where the mixed batched kernel (64
+// registers) otherwise spills two or three into local memory and misses the L1 with them (long-scoreboard
+// stalls 0.5 -> 2.5 per instruction), and the loads of the mixed global-deposit kernel do not queue before
+// its records (3.1 -> 2.1). us per step, before and after: 96 Hernquist + NFW fits of 52M particles
+// 934 -> 816, Hernquist 873 -> 794, log halo 873 -> 793; maps of 4M 84 -> 78. The other kernels lose by it
+// and load early: FP64 1M 119.2 -> 121.5, the mixed one of five blocks an SM 45.9 -> 46.4 at 2M, many
+// mixed steps per launch up to 2 %.
 template <class T, bool GA, bool LATE, unsigned M0, unsigned M1, unsigned M2, unsigned M3>
 __device__ __forceinline__ void step_particles(const Model &m, const Model &mh, const Cst<T> &k, const State<T> &P,
                                                const Buffers &b,

@@ -11,7 +11,7 @@
 // (the line lies at eight chunk-blocks an SM). Steps that update the priors meet a second time in either
 // case. The arithmetic and its order are those of k_step, bit for bit.
 //
-// Measured against one launch per step: 20,000 FP64 particles 20.5 -> 13.7 us per step (the sizes at
+// Measured against one launch per step: 20,000 FP64 particles 18.9 -> 13.5 us per step (the sizes at
 // persist_fits).
 //
 // Three sets of sums take turns: set s % 3 collects step s, is read after that step's meeting,
@@ -259,8 +259,9 @@ m2m_status persist_setup(m2m_ctx *ctx)
 // Whether the fit takes several steps per launch: all blocks resident at once, and in mixed
 // precision at most 8,192 particles an SM. The mixed kernel for one step keeps five blocks on an SM,
 // this one four (its step loop takes registers); us per step of this one and that one, Hernquist,
-// 150 observables: 1,000 particles 8.7 and 15.1, 100,000 17.6 and 19.9, 1M 34.4 and 35.7,
-// 2M 51.2 and 47.3. FP64 (two blocks in both): 1,000 13.0 and 19.5, 1M 155 and 158.
+// 150 observables: 1,000 particles 8.6 and 13.7, 100,000 16.5 and 18.7, 1M 32.7 and 32.7,
+// 2M 49.7 and 45.5. FP64 (two blocks in both): 1,000 12.8 and 17.9, 20,000 13.5 and 18.9, 1M 118.0
+// and 117.4.
 bool persist_fits(m2m_ctx *ctx)
 {
     if (ctx->precision == M2M_PREC_MIXED && ctx->n > 8192ll * ctx->nsm) return false;
